@@ -204,7 +204,7 @@ static void free_scene(rt_scene *s) {
     cudaFree(s->d_esc); cudaFree(s->io_rx); cudaFree(s->io_e); cudaFree(s->io_fl); cudaFree(s->d_img); cudaFree(s->d_txb);
     cudaFree(s->d_txw); cudaFree(s->d_bvh); cudaFree(s->d_bvh_tri); cudaFree(s->d_cand); cudaFree(s->d_cimg);
     cudaFree(s->d_face_mat); cudaFree(s->d_face_box);
-    cudaFree(s->dcb.dir); cudaFree(s->dcb.fn); cudaFree(s->dcb.keys); cudaFree(s->dcb.cand); cudaFree(s->dcb.cimg);
+    cudaFree(s->dcb.dir); cudaFree(s->dcb.fn); cudaFree(s->dcb.keys); cudaFree(s->dcb.table); cudaFree(s->dcb.cand); cudaFree(s->dcb.cimg);
     cudaFree(s->dcb.n_cand); cudaFree(s->d_lbvh); cudaFree(s->d_lbvh_tri); cudaFree(s->d_pc0);
 }
 
@@ -698,8 +698,9 @@ int rt_candidates_device(rt_scene *s, int n_rays, int max_order, void *stream) {
         CK(cudaMalloc(&s->dcb.keys, sizeof(unsigned long long) * RT_DEV_CAND_SLOTS));
         CK(cudaMalloc(&s->dcb.cand, sizeof(int4) * RT_DEV_CAND_SLOTS));
         CK(cudaMalloc(&s->dcb.cimg, sizeof(float4) * 6 * (size_t)RT_DEV_CAND_SLOTS));
-        CK(cudaMalloc(&s->dcb.n_cand, sizeof(int) * 2));
-        CK(cudaMemset(s->dcb.n_cand, 0, sizeof(int) * 2));
+        CK(cudaMalloc(&s->dcb.table, sizeof(unsigned long long) * RT_DEV_CAND_TABLE));
+        CK(cudaMalloc(&s->dcb.n_cand, sizeof(int) * 3));
+        CK(cudaMemset(s->dcb.n_cand, 0, sizeof(int) * 3));
         if (!s->d_bvh) {
             CK(cudaMalloc(&s->d_lbvh, sizeof(float4) * s->h_bvh.size()));
             CK(cudaMalloc(&s->d_lbvh_tri, sizeof(int) * s->h_bvh_tri.size()));

@@ -146,15 +146,17 @@ void ray_directions(int n_rays, std::vector<double> &dir);
 constexpr int BVH_MIN_TRI = 64;        // scenes with more triangles traverse the BVH on the device
 
 // Device ray launch (candidates.cu): at most RT_DEV_CAND_SLOTS ray prefixes
-// (n_rays x max_order); the finished list is sorted and made unique in one
-// block's shared memory.
+// (n_rays x max_order), made unique in a hash set of twice as many slots (a
+// power of two); the finished list is sorted in one block's shared memory.
+constexpr int RT_DEV_CAND_TABLE = 2 * RT_DEV_CAND_SLOTS;
 struct DevCandBufs {
     double *dir;               // [n_rays][3]
     double *fn;                // [n_face][3]
-    unsigned long long *keys;  // [RT_DEV_CAND_SLOTS]
+    unsigned long long *keys;  // [RT_DEV_CAND_SLOTS] the distinct prefixes found
+    unsigned long long *table; // [RT_DEV_CAND_TABLE] the hash set of them
     int4 *cand;                // [RT_DEV_CAND_SLOTS]
     float4 *cimg;              // [RT_DEV_CAND_SLOTS][3][2]
-    int *n_cand;               // [1]
+    int *n_cand;               // [3]: the list's length, stack overflow, distinct prefixes
 };
 int launch_ray_candidates(const float4 *tri, const float4 *bvh, const int *bvh_tri, const dq4 *face64,
                           const double tx[3], int n_rays, int max_order, const DevCandBufs &B, cudaStream_t st);
