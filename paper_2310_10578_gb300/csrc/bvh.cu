@@ -3,9 +3,8 @@
 // of a ray launch from the transmitter (orders 1-3), which the planar class
 // kernel then validates per receiver by the image method.
 //
-// BVH: binary, median split of the triangle centroids along the longest
-// axis of their bounds, leaves of at most BVH_LEAF triangles (depth <=
-// ceil(log2(n / BVH_LEAF)) + 1 <= 32 for any n < 2^31), nodes numbered
+// BVH: binary, surface-area splits (see Builder), leaves of at most BVH_LEAF
+// triangles, at most 31 levels below the root, nodes numbered
 // breadth first (the top levels first).  Node i is two float4: (box min,
 // first) and (box max, count); count > 0: a leaf over bvh_tri[first ..
 // first + count); count == 0: an inner node with children first and
@@ -53,54 +52,124 @@ inline int float_bits(float f) {
     return i;
 }
 
+// The split of a node: the plane of least surface-area cost among SAH_BINS
+// bins of the centroids on each axis.  A room's shell and walls are hundreds of
+// times larger than its furniture; a median split keeps them among small
+// triangles down to the leaves, so that boxes of every level overlap along a
+// segment (random segments of up to 20 m among 193 572 office triangles met 124
+// boxes and 24 triangles to their first hit or end; with this split 68 and 11).
+// The median split stays for nodes that no plane divides, and where a node's
+// depth and the levels that median splits still need below it reach MAX_DEPTH:
+// the device walks' stacks count on that.
+constexpr int SAH_BINS = 16;
+constexpr int MAX_DEPTH = 32;
+
 struct Builder {
-    const float *tri;
-    std::vector<int> idx;
-    std::vector<float> cen;     // [n][3]
+    struct Item {
+        float b[6], c[3];       // the triangle's box and centroid
+        int t;
+    };
+    std::vector<Item> it;       // in leaf order as the build goes on (moved, not indexed: its passes stream)
     std::vector<float4> nodes;
 
-    void bounds(int lo, int hi, float bmin[3], float bmax[3]) const {
-        for (int k = 0; k < 3; ++k) { bmin[k] = INFINITY; bmax[k] = -INFINITY; }
-        for (int i = lo; i < hi; ++i) {
-            const float *v = tri + 9 * (size_t)idx[i];
-            for (int c = 0; c < 3; ++c)
-                for (int k = 0; k < 3; ++k) {
-                    bmin[k] = fminf(bmin[k], v[3 * c + k]);
-                    bmax[k] = fmaxf(bmax[k], v[3 * c + k]);
-                }
+    void set(int node, const float b[6], int first, int count) {
+        nodes[2 * node] = make_float4(pad_lo(b[0]), pad_lo(b[1]), pad_lo(b[2]), int_bits(first));
+        nodes[2 * node + 1] = make_float4(pad_hi(b[3]), pad_hi(b[4]), pad_hi(b[5]), int_bits(count));
+    }
+    static void empty(float b[6]) {
+        for (int k = 0; k < 3; ++k) { b[k] = INFINITY; b[3 + k] = -INFINITY; }
+    }
+    static void grow(float b[6], const float *o) {
+        for (int k = 0; k < 3; ++k) {
+            b[k] = std::min(b[k], o[k]);
+            b[3 + k] = std::max(b[3 + k], o[3 + k]);
         }
     }
-    void set(int node, int lo, int hi, int first, int count) {
-        float bmin[3], bmax[3];
-        bounds(lo, hi, bmin, bmax);
-        nodes[2 * node] = make_float4(pad_lo(bmin[0]), pad_lo(bmin[1]), pad_lo(bmin[2]), int_bits(first));
-        nodes[2 * node + 1] = make_float4(pad_hi(bmax[0]), pad_hi(bmax[1]), pad_hi(bmax[2]), int_bits(count));
+    static float area(const float b[6]) {
+        const float x = b[3] - b[0], y = b[4] - b[1], z = b[5] - b[2];
+        return x * y + y * z + z * x;
     }
-    // node covers idx[lo, hi)
-    void build(int node, int lo, int hi) {
-        if (hi - lo <= BVH_LEAF) {
-            set(node, lo, hi, lo, hi - lo);
-            return;
+    // it[lo, hi) partitioned at the returned position by the best bin plane,
+    // or lo when there is none
+    int sah(int lo, int hi, const float cmin[3], const float cmax[3]) {
+        struct Bin { float b[6]; int n; } bin[3][SAH_BINS];
+        float sc[3];
+        const int nb = hi - lo <= 2 * SAH_BINS ? SAH_BINS / 2 : SAH_BINS;       // (most nodes are small)
+        for (int k = 0; k < 3; ++k) {
+            sc[k] = cmax[k] > cmin[k] ? nb / (cmax[k] - cmin[k]) : 0.0f;
+            for (int s = 0; s < nb; ++s) { empty(bin[k][s].b); bin[k][s].n = 0; }
         }
-        float cmin[3] = {INFINITY, INFINITY, INFINITY}, cmax[3] = {-INFINITY, -INFINITY, -INFINITY};
+        auto slot = [&](const Item &q, int k) {
+            const int s = (int)((q.c[k] - cmin[k]) * sc[k]);
+            return s < nb - 1 ? s : nb - 1;
+        };
         for (int i = lo; i < hi; ++i)
             for (int k = 0; k < 3; ++k) {
-                cmin[k] = fminf(cmin[k], cen[3 * (size_t)idx[i] + k]);
-                cmax[k] = fmaxf(cmax[k], cen[3 * (size_t)idx[i] + k]);
+                Bin &q = bin[k][slot(it[i], k)];
+                grow(q.b, it[i].b);
+                ++q.n;
             }
-        int ax = 0;
-        for (int k = 1; k < 3; ++k)
-            if (cmax[k] - cmin[k] > cmax[ax] - cmin[ax]) ax = k;
-        const int mid = lo + (hi - lo) / 2;
-        std::nth_element(idx.begin() + lo, idx.begin() + mid, idx.begin() + hi, [&](int a, int b) {
-            const float ca = cen[3 * (size_t)a + ax], cb = cen[3 * (size_t)b + ax];
-            return ca < cb || (ca == cb && a < b);
-        });
+        float best = INFINITY;
+        int ax = -1, at = 0;
+        for (int k = 0; k < 3; ++k) {
+            if (sc[k] == 0.0f) continue;
+            float right[SAH_BINS], b[6];
+            int n = 0;
+            empty(b);
+            for (int s = nb - 1; s > 0; --s) {
+                grow(b, bin[k][s].b);
+                n += bin[k][s].n;
+                right[s] = n ? area(b) * n : INFINITY;
+            }
+            empty(b);
+            n = 0;
+            for (int s = 0; s + 1 < nb; ++s) {
+                grow(b, bin[k][s].b);
+                n += bin[k][s].n;
+                const float cost = n ? area(b) * n + right[s + 1] : INFINITY;
+                if (cost < best) { best = cost; ax = k; at = s; }
+            }
+        }
+        if (ax < 0) return lo;
+        return (int)(std::partition(it.begin() + lo, it.begin() + hi, [&](const Item &q) { return slot(q, ax) <= at; }) -
+                     it.begin());
+    }
+    // levels below a node of n triangles under median splits
+    static int levels(int n) {
+        int l = 0;
+        for (; n > BVH_LEAF; n = (n + 1) / 2) ++l;
+        return l;
+    }
+    // node covers it[lo, hi)
+    void build(int node, int lo, int hi, int depth) {
+        float b[6], cmin[3] = {INFINITY, INFINITY, INFINITY}, cmax[3] = {-INFINITY, -INFINITY, -INFINITY};
+        empty(b);
+        for (int i = lo; i < hi; ++i) {
+            grow(b, it[i].b);
+            for (int k = 0; k < 3; ++k) {
+                cmin[k] = std::min(cmin[k], it[i].c[k]);
+                cmax[k] = std::max(cmax[k], it[i].c[k]);
+            }
+        }
+        if (hi - lo <= BVH_LEAF) {
+            set(node, b, lo, hi - lo);
+            return;
+        }
+        int mid = depth + 1 + levels(hi - lo) < MAX_DEPTH ? sah(lo, hi, cmin, cmax) : lo;
+        if (mid == lo || mid == hi) {
+            int ax = 0;
+            for (int k = 1; k < 3; ++k)
+                if (cmax[k] - cmin[k] > cmax[ax] - cmin[ax]) ax = k;
+            mid = lo + (hi - lo) / 2;
+            std::nth_element(it.begin() + lo, it.begin() + mid, it.begin() + hi, [&](const Item &p, const Item &q) {
+                return p.c[ax] < q.c[ax] || (p.c[ax] == q.c[ax] && p.t < q.t);
+            });
+        }
         const int left = (int)nodes.size() / 2;
         nodes.resize(nodes.size() + 4);
-        set(node, lo, hi, left, 0);
-        build(left, lo, mid);
-        build(left + 1, mid, hi);
+        set(node, b, left, 0);
+        build(left, lo, mid, depth + 1);
+        build(left + 1, mid, hi, depth + 1);
     }
 };
 
@@ -146,16 +215,20 @@ void bvh_build(const float *tri, int n_tri, std::vector<float4> &nodes, std::vec
     order.clear();
     if (n_tri <= 0) return;
     Builder B;
-    B.tri = tri;
-    B.idx.resize(n_tri);
-    B.cen.resize(3 * (size_t)n_tri);
+    B.it.resize(n_tri);
     for (int t = 0; t < n_tri; ++t) {
-        B.idx[t] = t;
+        Builder::Item &q = B.it[t];
+        Builder::empty(q.b);
         const float *v = tri + 9 * (size_t)t;
-        for (int k = 0; k < 3; ++k) B.cen[3 * (size_t)t + k] = (v[k] + v[3 + k] + v[6 + k]) * (1.0f / 3.0f);
+        for (int c = 0; c < 3; ++c) {
+            const float p[6] = {v[3 * c], v[3 * c + 1], v[3 * c + 2], v[3 * c], v[3 * c + 1], v[3 * c + 2]};
+            Builder::grow(q.b, p);
+        }
+        for (int k = 0; k < 3; ++k) q.c[k] = (v[k] + v[3 + k] + v[6 + k]) * (1.0f / 3.0f);
+        q.t = t;
     }
     B.nodes.resize(2);
-    B.build(0, 0, n_tri);
+    B.build(0, 0, n_tri, 0);
     // renumber the nodes breadth first (children pairs stay adjacent), so
     // that the top levels are the array's first nodes: the class kernels
     // stage that prefix (the top treelet) in shared memory
@@ -182,7 +255,8 @@ void bvh_build(const float *tri, int n_tri, std::vector<float4> &nodes, std::vec
         nodes[2 * k] = lo;
         nodes[2 * k + 1] = hi;
     }
-    order.swap(B.idx);
+    order.resize(n_tri);
+    for (int i = 0; i < n_tri; ++i) order[i] = B.it[i].t;
 }
 
 void ray_face_normals(const float *tri, const int *tri_face, int n_tri, int n_face, std::vector<double> &fn) {
