@@ -134,6 +134,8 @@ struct rt_scene {
     float4 *d_txw = nullptr;            // the same for each face's source image, see DevScene::txw
     float4 *d_face_mat = nullptr;       // face materials, see DevScene::face_mat
     float4 *d_face_box = nullptr;       // per face its culling box, see DevScene::face_box
+    float4 *d_face_occ = nullptr;       // per face its polygon, see DevScene::face_occ
+    uint32_t *d_hid = nullptr;          // [RT_MAX_BODIES / 32], see FrameDev::hid
     bool any_dielectric = false;
     // large-scene mode: the triangle BVH (host copy for the ray launch; on the
     // device above BVH_MIN_TRI triangles) and the candidate face sequences
@@ -203,9 +205,62 @@ static void free_scene(rt_scene *s) {
     cudaFree(s->d_face64); cudaFree(s->d_face_rng); cudaFree(s->d_face_tris); cudaFree(s->d_freq); cudaFree(s->d_fqc);
     cudaFree(s->d_esc); cudaFree(s->io_rx); cudaFree(s->io_e); cudaFree(s->io_fl); cudaFree(s->d_img); cudaFree(s->d_txb);
     cudaFree(s->d_txw); cudaFree(s->d_bvh); cudaFree(s->d_bvh_tri); cudaFree(s->d_cand); cudaFree(s->d_cimg);
-    cudaFree(s->d_face_mat); cudaFree(s->d_face_box);
+    cudaFree(s->d_face_mat); cudaFree(s->d_face_box); cudaFree(s->d_face_occ); cudaFree(s->d_hid);
     cudaFree(s->dcb.dir); cudaFree(s->dcb.fn); cudaFree(s->dcb.keys); cudaFree(s->dcb.table); cudaFree(s->dcb.cand); cudaFree(s->dcb.cimg);
     cudaFree(s->dcb.n_cand); cudaFree(s->d_lbvh); cudaFree(s->d_lbvh_tri); cudaFree(s->d_pc0);
+}
+
+// The face of triangles t[0 .. n) as one convex polygon: a single triangle, or
+// two that share an edge and form a strictly convex, planar quadrilateral.
+// occ[4]: the vertices, their number in occ[0].w (int bits; 0: neither).
+static void face_polygon(const float *tri, const int *t, int n, float4 occ[4]) {
+    for (int k = 0; k < 4; ++k) occ[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto put = [&](int k, const float *v) { occ[k].x = v[0]; occ[k].y = v[1]; occ[k].z = v[2]; };
+    auto count = [&](int nv) { memcpy(&occ[0].w, &nv, sizeof(float)); };
+    const float *A = tri + 9 * (size_t)t[0];
+    if (n == 1) {
+        for (int k = 0; k < 3; ++k) put(k, A + 3 * k);
+        count(3);
+        return;
+    }
+    if (n != 2) return;
+    const float *B = tri + 9 * (size_t)t[1];
+    auto same = [](const float *a, const float *b) { return a[0] == b[0] && a[1] == b[1] && a[2] == b[2]; };
+    int lone = -1, far = -1, shared = 0;
+    for (int k = 0; k < 3; ++k) {
+        bool in = false;
+        for (int j = 0; j < 3; ++j) in = in || same(A + 3 * k, B + 3 * j);
+        if (in) ++shared; else lone = k;
+        in = false;
+        for (int j = 0; j < 3; ++j) in = in || same(B + 3 * k, A + 3 * j);
+        if (!in) far = k;
+    }
+    if (shared != 2 || lone < 0 || far < 0) return;
+    const float *q[4] = {A + 3 * lone, A + 3 * ((lone + 1) % 3), B + 3 * far, A + 3 * ((lone + 2) % 3)};
+    double N[3] = {0, 0, 0}, turn[4][3];
+    for (int k = 0; k < 4; ++k) {
+        const float *a = q[k], *b = q[(k + 1) & 3], *c = q[(k + 2) & 3];
+        double u[3], w[3];
+        for (int j = 0; j < 3; ++j) { u[j] = (double)b[j] - a[j]; w[j] = (double)c[j] - b[j]; }
+        const double lu = sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]), lw = sqrt(w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
+        for (int j = 0; j < 3; ++j) {
+            const int x = (j + 1) % 3, y = (j + 2) % 3;
+            turn[k][j] = (u[x] * w[y] - u[y] * w[x]) / (lu * lw);
+            N[j] += turn[k][j];
+        }
+    }
+    const double nn = sqrt(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
+    if (!(nn > 0.0)) return;
+    double off = 0.0;
+    for (int k = 0; k < 4; ++k) {
+        if (!(turn[k][0] * N[0] + turn[k][1] * N[1] + turn[k][2] * N[2] > 1e-3 * nn)) return;
+        double d = 0.0;
+        for (int j = 0; j < 3; ++j) d += N[j] / nn * ((double)q[k][j] - q[0][j]);
+        off = fmax(off, fabs(d));
+    }
+    if (off > 1e-5) return;                     // (far within the occlusion test's margin)
+    for (int k = 0; k < 4; ++k) put(k, q[k]);
+    count(4);
 }
 
 // distance from point p to the solid of body b (0 if inside)
@@ -493,6 +548,13 @@ int rt_scene_create(const float *tri_xyz, const int *tri_face, int n_tri, const 
         CKS(cudaMalloc(&s->d_bvh_tri, sizeof(int) * s->h_bvh_tri.size()));
         CKS(cudaMemcpy(s->d_bvh, s->h_bvh.data(), sizeof(float4) * s->h_bvh.size(), cudaMemcpyHostToDevice));
         CKS(cudaMemcpy(s->d_bvh_tri, s->h_bvh_tri.data(), sizeof(int) * s->h_bvh_tri.size(), cudaMemcpyHostToDevice));
+        std::vector<float4> occ(4 * (size_t)nf);
+        for (int f = 0; f < nf; ++f)
+            face_polygon(s->tri.data(), face_tris.data() + s->faces[f].first, s->faces[f].count, &occ[4 * (size_t)f]);
+        CKS(cudaMalloc(&s->d_face_occ, sizeof(float4) * occ.size()));
+        CKS(cudaMemcpy(s->d_face_occ, occ.data(), sizeof(float4) * occ.size(), cudaMemcpyHostToDevice));
+        CKS(cudaMalloc(&s->d_hid, sizeof(uint32_t) * (RT_MAX_BODIES / 32)));
+        CKS(cudaMemset(s->d_hid, 0, sizeof(uint32_t) * (RT_MAX_BODIES / 32)));
     }
     if (n_tri > 0) {
         CKS(cudaMemcpy(s->d_tri, htri.data(), sizeof(float4) * 3 * n_tri, cudaMemcpyHostToDevice));
@@ -872,6 +934,8 @@ static int make_dev(rt_scene *s, const rt_options *opt, DevScene &D, int *prec, 
     }
     D.face_mat = s->any_dielectric ? s->d_face_mat : nullptr;
     D.face_box = s->d_face_box;
+    D.face_occ = s->d_face_occ;
+    D.hid = s->d_hid;
     memcpy(D.tx, s->tx, sizeof(D.tx));
     memcpy(D.pol, s->pol, sizeof(D.pol));
     D.band_len = s->band_len;
@@ -1034,6 +1098,7 @@ struct rt_batch {
     float4 *d_body = nullptr, *d_txb = nullptr;   // [n_frames][max_body][2]
     FreqC *d_fqc = nullptr;                       // [n_frames][nch]
     FrameDev *d_frames = nullptr;                 // [n_frames]
+    uint32_t *d_hid = nullptr;                    // [n_frames][RT_MAX_BODIES / 32] (scenes with a BVH)
     unsigned long long *d_ctr = nullptr;          // [CTR_N]
     // spatial ordering of the receivers: cell counts [n_frames][RX_CELLS],
     // ranks, the sorted receivers and the permutation [total receivers]
@@ -1055,7 +1120,7 @@ static void free_batch(rt_batch *b) {
     if (b->gexec) cudaGraphExecDestroy(b->gexec);
     if (b->graph) cudaGraphDestroy(b->graph);
     cudaFree(b->d_body); cudaFree(b->d_txb); cudaFree(b->d_fqc); cudaFree(b->d_frames); cudaFree(b->d_ctr);
-    cudaFree(b->d_cnt); cudaFree(b->d_rank); cudaFree(b->d_rxs); cudaFree(b->d_perm);
+    cudaFree(b->d_hid); cudaFree(b->d_cnt); cudaFree(b->d_rank); cudaFree(b->d_rxs); cudaFree(b->d_perm);
 }
 
 // queue one evaluation of the batch on st (no synchronisation)
@@ -1151,8 +1216,14 @@ int rt_batch_create(rt_scene *s, int n_frames, const int32_t *n_rx, int n_f, int
         CKB(cudaMalloc(&b->d_rxs, sizeof(float) * 3 * nr));
         CKB(cudaMalloc(&b->d_perm, sizeof(int32_t) * nr));
     }
+    if (s->d_bvh) {
+        const size_t nh = (size_t)n_frames * (RT_MAX_BODIES / 32);
+        CKB(cudaMalloc(&b->d_hid, sizeof(uint32_t) * nh));
+        CKB(cudaMemset(b->d_hid, 0, sizeof(uint32_t) * nh));
+    }
     for (int f = 0; f < n_frames; ++f) {
         FrameDev &F = b->fr[f];
+        F.hid = b->d_hid ? b->d_hid + (size_t)f * (RT_MAX_BODIES / 32) : nullptr;
         F.body = b->d_body + (size_t)f * 2 * (max_body > 0 ? max_body : 1);
         F.txb = b->d_txb + (size_t)f * 2 * (max_body > 0 ? max_body : 1);
         F.fqc = b->d_fqc + (size_t)f * b->nch;

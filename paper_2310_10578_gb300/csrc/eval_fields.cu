@@ -71,7 +71,12 @@ struct Ctx {
     const int2 *face_rng;
     const int *face_tris;
     const float4 *face_box;      // see DevScene
+    const float4 *face_occ;      // see DevScene (with bvh)
     int n_tri, n_face, n_body;
+    // the bodies that get candidates: all n_body of them, or (scenes with a
+    // BVH, body classes) the n_cand_body of blist that the source may see
+    const uint16_t *blist;
+    int n_cand_body;
     float band;
     v3t<float> S, pol;
     const float4 *fock;          // [FOCK_N][2], then the P segment [FOCK_NP][2] (see DevScene)
@@ -307,6 +312,175 @@ __device__ __forceinline__ int tris_bvh(const Ctx &c, v3t<T> A, v3t<T> B, int sf
     return hit ? D_YES : (uns ? D_UNSURE : D_NO);
 }
 
+// ---- occlusion of whole regions (scenes with a BVH).  Every segment between
+// two boxes X and Y is blocked if one convex polygon of the scene (a face, or a
+// triangle) separates them: X and Y strictly on opposite sides of its plane,
+// and X, for every corner y of Y and every edge e of the polygon, on the inner
+// side of the plane through y and e.  (For a fixed y the set of points that y
+// sees through the polygon is convex, and the segment from a point x to it
+// crosses the plane inside the polygon; for a fixed x the same set of points y
+// is convex too, so the corners of Y decide for all of it.)  Distances of more
+// than a margin (1 mm + 8 bands) and a bound of the rounding of the products
+// are required, so that the decision of each such segment -- "blocked" in FP64,
+// away from every tie -- is the one the segment's own test takes.  Leaving the
+// candidates of such a region out changes no decision; their re-decisions in
+// FP64 fall away with them.
+struct Box {
+    v3t<float> lo, hi;           // corners (as given: no rounding)
+    v3t<float> c, h;             // centre, half extents (to within the margin)
+};
+__device__ __forceinline__ Box box_of(const float lo[3], const float hi[3]) {
+    Box b;
+    b.lo = mk3(lo[0], lo[1], lo[2]);
+    b.hi = mk3(hi[0], hi[1], hi[2]);
+    b.c = (b.lo + b.hi) * 0.5f;
+    b.h = (b.hi - b.lo) * 0.5f;
+    return b;
+}
+__device__ __forceinline__ float hull_margin(const Ctx &c) { return 1e-3f + 8.0f * c.band; }
+__device__ __forceinline__ Box body_box(const Ctx &c, int b) {
+    const float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
+    const bool sph = q1.y == 0.0f;
+    const float m = hull_margin(c);
+    const float lo[3] = {q0.x - q0.w - m, q0.y - q0.w - m, (sph ? q0.z - q0.w : q0.z) - m};
+    const float hi[3] = {q0.x + q0.w + m, q0.y + q0.w + m, (sph ? q0.z + q0.w : q0.z + q1.x) + m};
+    return box_of(lo, hi);
+}
+// triangle t (its face's polygon where the face is one) blocks X -> Y
+__device__ __noinline__ bool occludes(const Ctx &c, int t, const Box &X, const Box &Y) {
+    const float m = hull_margin(c);
+    const float4 nq = c.tri_aux[3 * t];
+    const float sx = nq.x * X.c.x + nq.y * X.c.y + nq.z * X.c.z - nq.w, sy = nq.x * Y.c.x + nq.y * Y.c.y + nq.z * Y.c.z - nq.w;
+    const float ex = fabsf(nq.x) * X.h.x + fabsf(nq.y) * X.h.y + fabsf(nq.z) * X.h.z + m;
+    const float ey = fabsf(nq.x) * Y.h.x + fabsf(nq.y) * Y.h.y + fabsf(nq.z) * Y.h.z + m;
+    if (!((sx > ex && sy < -ey) || (sx < -ex && sy > ey))) return false;
+    const float4 *v = c.face_occ + 4 * (size_t)__float_as_int(c.tri[3 * t].w);
+    int nv = __float_as_int(v[0].w);
+    if (nv == 0) { v = c.tri + 3 * (size_t)t; nv = 3; }
+    float sg = 0.0f;
+    for (int k = 0; k < 8; ++k) {
+        if (((k & 1) && Y.hi.x == Y.lo.x) || ((k & 2) && Y.hi.y == Y.lo.y) || ((k & 4) && Y.hi.z == Y.lo.z)) continue;
+        const v3t<float> y = mk3((k & 1) ? Y.hi.x : Y.lo.x, (k & 2) ? Y.hi.y : Y.lo.y, (k & 4) ? Y.hi.z : Y.lo.z);
+        const v3t<float> w = X.c - y;
+        const float lw = fabsf(w.x) + fabsf(w.y) + fabsf(w.z);
+        v3t<float> a = ld3<float>(v[nv - 1]) - y;
+        if (sg == 0.0f)      // the polygon's orientation as seen from y (the same for all of Y)
+            sg = dot3(cross3(a, ld3<float>(v[0]) - y), ld3<float>(v[1]) - y) > 0.0f ? 1.0f : -1.0f;
+        for (int i = 0; i < nv; ++i) {
+            const v3t<float> b = ld3<float>(v[i]) - y;
+            const v3t<float> n = cross3(a, b);
+            // (each component of n within 3e-7 |a|_1 |b|_1, the sum within 4 more roundings)
+            const float err = 4e-6f * (fabsf(a.x) + fabsf(a.y) + fabsf(a.z)) * (fabsf(b.x) + fabsf(b.y) + fabsf(b.z)) * lw;
+            const float ext = fabsf(n.x) * X.h.x + fabsf(n.y) * X.h.y + fabsf(n.z) * X.h.z;
+            if (!(sg * dot3(n, w) > ext + m * norm3(n) + err)) return false;
+            a = b;
+        }
+    }
+    return true;
+}
+// Which bodies of each frame are hidden from the transmitter altogether
+// (FrameDev::hid, bit b % 32 of word b / 32): no reflection, no creeping ray.
+// One warp per body; as the ray launch's, its walk takes up to 32 nodes at a
+// time from a stack in shared memory, since one walk after another by a lane
+// alone is some 100 us of dependent loads, ahead of everything else.  0.07 ms
+// for 110 bodies among 193 572 triangles; with most of those bodies out, the
+// body kernels of 1 M receivers went from 31 and 32 ms to 2.2 and 1.7 ms.
+constexpr int HID_WARPS = 4;
+constexpr int HID_STACK = 1088;
+__global__ void __launch_bounds__(32 * HID_WARPS) k_src_hidden(DevScene S, FrameDev F1, const FrameDev *frames) {
+    __shared__ int s_stack[HID_WARPS][HID_STACK];
+    __shared__ Ctx s_c[HID_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = blockIdx.x * HID_WARPS + warp;
+    const FrameDev *F = frames ? frames + blockIdx.y : &F1;
+    if (b >= F->n_body) return;
+    Ctx &c = s_c[warp];
+    if (lane == 0) {
+        c.tri = S.tri; c.tri_aux = S.tri_alt; c.face_occ = S.face_occ; c.bvh = S.bvh; c.bvh_tri = S.bvh_tri;
+        c.body = F->body;
+        c.band = frames ? F->band : S.band_len;
+    }
+    __syncwarp();
+    const Box X = body_box(c, b);
+    const Box Y = box_of(S.tx, S.tx);
+    const v3t<float> inv = mk3(seg_inv(Y.c.x - X.c.x), seg_inv(Y.c.y - X.c.y), seg_inv(Y.c.z - X.c.z));
+    int *stack = s_stack[warp];
+    int sp = 1;
+    bool hidden = false;
+    if (lane == 0) stack[0] = 0;
+    __syncwarp();
+    while (sp > 0 && !hidden) {
+        // (near the stack's end one node at a time: depth first, at most the tree's depth more)
+        const int np = min(min(32, sp), max(1, HID_STACK - 40 - sp));
+        int first = 0, count = 0, push = 0;
+        sp -= np;
+        if (lane < np) {
+            const int nd = stack[sp + lane];
+            first = __float_as_int(S.bvh[2 * nd].w);
+            count = __float_as_int(S.bvh[2 * nd + 1].w);
+            if (count == 0) {
+                push = (seg_box(X.c, inv, S.bvh[2 * first], S.bvh[2 * first + 1], 0.0f) ? 1 : 0) |
+                       (seg_box(X.c, inv, S.bvh[2 * first + 2], S.bvh[2 * first + 3], 0.0f) ? 2 : 0);
+            }
+        }
+        __syncwarp();
+        const unsigned m0 = __ballot_sync(0xffffffffu, push & 1), m1 = __ballot_sync(0xffffffffu, push & 2);
+        const unsigned lt = (1u << lane) - 1u;
+        if (sp + __popc(m0) + __popc(m1) > HID_STACK) break;       // (a tree deeper than the build makes: not hidden)
+        if (push & 1) stack[sp + __popc(m0 & lt)] = first;
+        if (push & 2) stack[sp + __popc(m0) + __popc(m1 & lt)] = first + 1;
+        sp += __popc(m0) + __popc(m1);
+        __syncwarp();
+        bool hit = false;
+        for (int j = 0; j < count && !hit; ++j) hit = occludes(c, S.bvh_tri[first + j], X, Y);
+        hidden = __any_sync(0xffffffffu, hit);
+    }
+    if (lane == 0) {
+        if (hidden) atomicOr(F->hid + (b >> 5), 1u << (b & 31));
+        else atomicAnd(F->hid + (b >> 5), ~(1u << (b & 31)));
+    }
+}
+
+// every body (but sb) against a segment (FP32); uns: uncertain ones before
+__device__ __forceinline__ int bodies_all(const Ctx &c, v3t<float> A, v3t<float> B, int sb, float band, int uns) {
+    // bodies: a squared-distance test against the segment's closest point
+    // to the centre (cylinders: to the axis, in projection) rejects the
+    // bodies that are clearly apart -- distance above a + band, so the
+    // margin of the full test would be below -band.  Four bodies at a
+    // time without branches (sphere and cylinder differ by a select), so
+    // their dependent chains overlap; the full test only for the rest.
+    const v3t<float> D = B - A;
+    const float qa = D.x * D.x + D.y * D.y;
+    const float iqa = (qa > 0.0f) ? 1.0f / qa : 0.0f;
+    const float idd = 1.0f / (qa + D.z * D.z);
+    const float tlo = (float)EPS_TRIM, thi = 1.0f - (float)EPS_TRIM;
+    const int nb = c.n_body;
+    for (int b0 = 0; b0 < nb; b0 += 4) {
+        unsigned near = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int b = min(b0 + k, nb - 1);
+            const float4 q0 = c.body[2 * b];
+            const bool sph = c.body[2 * b + 1].y == 0.0f;
+            const float wx = q0.x - A.x, wy = q0.y - A.y, wz = sph ? q0.z - A.z : 0.0f;
+            const float dz = sph ? D.z : 0.0f;
+            const float t = fminf(fmaxf((wx * D.x + wy * D.y + wz * dz) * (sph ? idd : iqa), tlo), thi);
+            const float hx = D.x * t - wx, hy = D.y * t - wy, hz = dz * t - wz;
+            const float ab = q0.w + band;
+            const bool n = (b0 + k < nb) && (b0 + k != sb) && (hx * hx + hy * hy + hz * hz <= ab * ab);
+            near |= n ? (1u << k) : 0u;
+        }
+        while (near) {
+            const int b = b0 + __ffs(near) - 1;
+            near &= near - 1;
+            int r = seg_body(c, b, A, B, band);
+            if (r == D_YES) return D_YES;
+            uns |= (r == D_UNSURE);
+        }
+    }
+    return uns ? D_UNSURE : D_NO;
+}
+
 // 0 visible, 1 blocked, 2 unsure.  Faces sf1/sf2 and body sb are skipped.
 template <typename T>
 __device__ __forceinline__ int blocked_impl(const Ctx &c, v3t<T> A, v3t<T> B, int sf1, int sf2, int sb, T band) {
@@ -369,37 +543,38 @@ __device__ __forceinline__ int blocked_impl(const Ctx &c, v3t<T> A, v3t<T> B, in
         }
         return D_NO;
     }
-    if constexpr (sizeof(T) == 4) {
-        // bodies: a squared-distance test against the segment's closest point
-        // to the centre (cylinders: to the axis, in projection) rejects the
-        // bodies that are clearly apart -- distance above a + band, so the
-        // margin of the full test would be below -band.  Four bodies at a
-        // time without branches (sphere and cylinder differ by a select), so
-        // their dependent chains overlap; the full test only for the rest.
-        const v3t<float> D = B - A;
-        const float qa = D.x * D.x + D.y * D.y;
-        const float iqa = (qa > 0.0f) ? 1.0f / qa : 0.0f;
-        const float idd = 1.0f / (qa + D.z * D.z);
-        const float tlo = (float)EPS_TRIM, thi = 1.0f - (float)EPS_TRIM;
-        const int nb = c.n_body;
-        for (int b0 = 0; b0 < nb; b0 += 4) {
-            unsigned near = 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int b = min(b0 + k, nb - 1);
-                const float4 q0 = c.body[2 * b];
-                const bool sph = c.body[2 * b + 1].y == 0.0f;
-                const float wx = q0.x - A.x, wy = q0.y - A.y, wz = sph ? q0.z - A.z : 0.0f;
-                const float dz = sph ? D.z : 0.0f;
-                const float t = fminf(fmaxf((wx * D.x + wy * D.y + wz * dz) * (sph ? idd : iqa), tlo), thi);
-                const float hx = D.x * t - wx, hy = D.y * t - wy, hz = dz * t - wz;
-                const float ab = q0.w + band;
-                const bool n = (b0 + k < nb) && (b0 + k != sb) && (hx * hx + hy * hy + hz * hz <= ab * ab);
-                near |= n ? (1u << k) : 0u;
-            }
-            while (near) {
-                const int b = b0 + __ffs(near) - 1;
-                near &= near - 1;
+    if constexpr (sizeof(T) == 4) return bodies_all(c, A, B, sb, band, uns);
+    return uns ? D_UNSURE : D_NO;
+}
+// One out-of-line copy per precision: the visibility loop is called from ten
+// places per receiver; inlining it everywhere overflows the instruction cache.
+__device__ __noinline__ int blocked(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb, float band) {
+    return blocked_impl(c, A, B, sf1, sf2, sb, band);
+}
+// The bodies (but sb) of the mask occ, nw words, against a segment (FP32): uns
+// tells of uncertain ones among the triangles before
+__device__ __forceinline__ int bodies_masked(const Ctx &c, v3t<float> A, v3t<float> B, int sb, float band,
+                                             const uint32_t *occ, int nw, int uns) {
+    const v3t<float> D = B - A;
+    const float qa = D.x * D.x + D.y * D.y;
+    const float iqa = (qa > 0.0f) ? 1.0f / qa : 0.0f;
+    const float idd = 1.0f / (qa + D.z * D.z);
+    const float tlo = (float)EPS_TRIM, thi = 1.0f - (float)EPS_TRIM;
+#pragma unroll 1
+    for (int w = 0; w < nw; ++w) {
+        unsigned cand = occ[w];
+        if (sb >= 0 && sb >> 5 == w) cand &= ~(1u << (sb & 31));
+        while (cand) {
+            const int b = 32 * w + __ffs(cand) - 1;
+            cand &= cand - 1;
+            const float4 q0 = c.body[2 * b];
+            const bool sph = c.body[2 * b + 1].y == 0.0f;
+            const float wx = q0.x - A.x, wy = q0.y - A.y, wz = sph ? q0.z - A.z : 0.0f;
+            const float dz = sph ? D.z : 0.0f;
+            const float t = fminf(fmaxf((wx * D.x + wy * D.y + wz * dz) * (sph ? idd : iqa), tlo), thi);
+            const float hx = D.x * t - wx, hy = D.y * t - wy, hz = dz * t - wz;
+            const float ab = q0.w + band;
+            if (hx * hx + hy * hy + hz * hz <= ab * ab) {
                 int r = seg_body(c, b, A, B, band);
                 if (r == D_YES) return D_YES;
                 uns |= (r == D_UNSURE);
@@ -408,11 +583,106 @@ __device__ __forceinline__ int blocked_impl(const Ctx &c, v3t<T> A, v3t<T> B, in
     }
     return uns ? D_UNSURE : D_NO;
 }
-// One out-of-line copy per precision: the visibility loop is called from ten
-// places per receiver; inlining it everywhere overflows the instruction cache.
-__device__ __noinline__ int blocked(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb, float band) {
-    return blocked_impl(c, A, B, sf1, sf2, sb, band);
+// ---- a leg's triangles for a whole warp (scenes with a BVH, FP32): the lanes
+// `lanes` (all of which call this; `alive`: this lane has a segment) test the
+// same leg of the same candidate for neighbouring receivers.
+//   A triangle that blocks one lane's segment mostly blocks its neighbours' too,
+// so the warp walks the BVH for one lane at a time, all lanes on that one
+// segment, up to 32 nodes a step from a stack in shared memory, and every lane
+// then tries the triangle found.  A segment that nothing blocks ends that: the
+// lanes still left walk for themselves (in the light each would need its own
+// walk anyway, and 32 of them side by side cost less than 32 of the warp's).
+//   By itself a lane's walk is a chain of some 70 dependent loads, and a warp's
+// takes as long as its longest; this one takes six to ten steps.  The candidate
+// class of the office went from 38.6 to 33.9 ms with it (and with the legs'
+// occluder masks).  Taking the last eight lit lanes in turn too was slower, 45.1
+// against 40.6 ms for the whole evaluation.
+constexpr int COOP_STACK = 416;
+constexpr int COOP_ROUNDS = 6;
+// a triangle that certainly blocks a -> b, or -1; *uns: one that may
+__device__ __forceinline__ int coop_walk(const Ctx &c, unsigned lanes, v3t<float> a, v3t<float> b, int sf1, int sf2,
+                                         float band, int *stk, bool *uns) {
+    const int lane = threadIdx.x & 31, rank = __popc(lanes & ((1u << lane) - 1u)), nact = __popc(lanes);
+    const unsigned lt = (1u << lane) - 1u;
+    const v3t<float> inv = mk3(seg_inv(b.x - a.x), seg_inv(b.y - a.y), seg_inv(b.z - a.z));
+    int sp = 1, found = -1;
+    bool u = false;
+    __syncwarp(lanes);
+    if (rank == 0) stk[0] = 0;
+    __syncwarp(lanes);
+    while (sp > 0) {
+        // (near the stack's end one node at a time: depth first, at most the tree's depth more)
+        const int np = min(min(nact, sp), max(1, COOP_STACK - 40 - sp));
+        int first = 0, count = 0, push = 0;
+        sp -= np;
+        if (rank < np) {
+            const int nd = stk[sp + rank];
+            const float4 *nb = (nd < c.bvh_top_n) ? c.bvh_top : c.bvh;
+            first = __float_as_int(nb[2 * nd].w);
+            count = __float_as_int(nb[2 * nd + 1].w);
+            if (count == 0) {
+                const float4 *cb = (first + 1 < c.bvh_top_n) ? c.bvh_top : c.bvh;
+                push = (seg_box(a, inv, cb[2 * first], cb[2 * first + 1], band) ? 1 : 0) |
+                       (seg_box(a, inv, cb[2 * first + 2], cb[2 * first + 3], band) ? 2 : 0);
+            }
+        }
+        __syncwarp(lanes);
+        const unsigned m0 = __ballot_sync(lanes, push & 1), m1 = __ballot_sync(lanes, push & 2);
+        if (sp + __popc(m0) + __popc(m1) > COOP_STACK) {      // (a tree deeper than the build makes)
+            u = true;
+            break;
+        }
+        if (push & 1) stk[sp + __popc(m0 & lt)] = first;
+        if (push & 2) stk[sp + __popc(m0) + __popc(m1 & lt)] = first + 1;
+        sp += __popc(m0) + __popc(m1);
+        int hit = -1;
+        for (int j = 0; j < count && hit < 0; ++j) {
+            const int t = c.bvh_tri[first + j];
+            const int f = __float_as_int(c.tri[3 * t].w);
+            if (f == sf1 || f == sf2) continue;
+            const int r = seg_tri(c, t, a, b, c.band);
+            if (r == D_YES) hit = t;
+            u = u || r == D_UNSURE;
+        }
+        const unsigned hb = __ballot_sync(lanes, hit >= 0);
+        if (hb) {
+            found = __shfl_sync(lanes, hit, __ffs(hb) - 1);
+            break;
+        }
+        __syncwarp(lanes);
+    }
+    *uns = __any_sync(lanes, u);
+    return found;
 }
+__device__ __noinline__ int tris_coop(const Ctx &c, unsigned lanes, bool alive, v3t<float> A, v3t<float> B, int sf1,
+                                      int sf2, float band, int *stk) {
+    const int lane = threadIdx.x & 31;
+    int res = D_NO;
+    unsigned todo = __ballot_sync(lanes, alive);
+    for (int k = 0; k < COOP_ROUNDS && todo; ++k) {
+        const int ld = __ffs(todo) - 1;
+        const v3t<float> a = mk3(__shfl_sync(lanes, A.x, ld), __shfl_sync(lanes, A.y, ld), __shfl_sync(lanes, A.z, ld));
+        const v3t<float> b = mk3(__shfl_sync(lanes, B.x, ld), __shfl_sync(lanes, B.y, ld), __shfl_sync(lanes, B.z, ld));
+        bool u;
+        const int t = coop_walk(c, lanes, a, b, sf1, sf2, band, stk, &u);
+        if (t < 0) {
+            if (lane == ld) {
+                res = u ? D_UNSURE : D_NO;
+                alive = false;
+            }
+            break;
+        }
+        if (alive && (lane == ld || seg_tri(c, t, A, B, band) == D_YES)) {
+            res = D_YES;
+            alive = false;
+        }
+        todo = __ballot_sync(lanes, alive);
+    }
+    if (alive) res = tris_bvh<float>(c, A, B, sf1, sf2, band);
+    __syncwarp(lanes);
+    return res;
+}
+
 // A leg with an occluder mask (FP32): the faces (but sf1, sf2) as in blocked;
 // the bodies (but sb) are those of the mask occ, nw words (a superset of the
 // bodies that can pass the distance test), or all of them without a mask.
@@ -446,33 +716,7 @@ __device__ __noinline__ int blocked_mask(const Ctx &c, v3t<float> A, v3t<float> 
             }
         }
     }
-    const v3t<float> D = B - A;
-    const float qa = D.x * D.x + D.y * D.y;
-    const float iqa = (qa > 0.0f) ? 1.0f / qa : 0.0f;
-    const float idd = 1.0f / (qa + D.z * D.z);
-    const float tlo = (float)EPS_TRIM, thi = 1.0f - (float)EPS_TRIM;
-#pragma unroll 1
-    for (int w = 0; w < nw; ++w) {
-        unsigned cand = occ[w];
-        if (sb >= 0 && sb >> 5 == w) cand &= ~(1u << (sb & 31));
-        while (cand) {
-            const int b = 32 * w + __ffs(cand) - 1;
-            cand &= cand - 1;
-            const float4 q0 = c.body[2 * b];
-            const bool sph = c.body[2 * b + 1].y == 0.0f;
-            const float wx = q0.x - A.x, wy = q0.y - A.y, wz = sph ? q0.z - A.z : 0.0f;
-            const float dz = sph ? D.z : 0.0f;
-            const float t = fminf(fmaxf((wx * D.x + wy * D.y + wz * dz) * (sph ? idd : iqa), tlo), thi);
-            const float hx = D.x * t - wx, hy = D.y * t - wy, hz = dz * t - wz;
-            const float ab = q0.w + band;
-            if (hx * hx + hy * hy + hz * hz <= ab * ab) {
-                int r = seg_body(c, b, A, B, band);
-                if (r == D_YES) return D_YES;
-                uns |= (r == D_UNSURE);
-            }
-        }
-    }
-    return uns ? D_UNSURE : D_NO;
+    return bodies_masked(c, A, B, sb, band, occ, nw, uns);
 }
 __device__ __noinline__ int blocked(const Ctx &c, v3t<dx> A, v3t<dx> B, int sf1, int sf2, int sb, dx band) {
     return blocked_impl(c, A, B, sf1, sf2, sb, band);
@@ -777,6 +1021,31 @@ __device__ int cand_seq(const Ctx &c, int q, int4 sq, v3t<T> S, v3t<T> P, T band
     const v3t<T> E = (k == 1) ? Q[0] : ((k == 2) ? Q[1] : Q[2]);
     if (!conj(acc, vis_to_dec(blocked(c, E, P, fs[k - 1], -1, -1, band)))) return D_NO;
     return acc;
+}
+
+// the legs of a sequence for the warp's lanes `lanes` (which all take the same
+// one; d: this lane's decision so far): triangles by tris_coop, bodies by the
+// legs' occluder masks wm (nw words each; nw = 0: every body)
+__device__ __forceinline__ int seq_vis_coop(const Ctx &c, unsigned lanes, int4 sq, v3t<float> S, v3t<float> P, float band,
+                                            const v3t<float> Q[3], int d, const uint32_t *wm, int nw, int *stk) {
+    const int k = sq.w;
+    v3t<float> A = S;
+    int fa = -1;
+#pragma unroll 1
+    for (int m = 0; m <= k; ++m) {
+        if (!__any_sync(lanes, d != D_NO)) break;
+        const int fb = m == k ? -1 : (m == 0 ? sq.x : (m == 1 ? sq.y : sq.z));
+        const v3t<float> B = m == k ? P : (m == 0 ? Q[0] : (m == 1 ? Q[1] : Q[2]));
+        const int r = tris_coop(c, lanes, d != D_NO, A, B, fa, fb, band, stk);
+        if (d != D_NO && conj(d, vis_to_dec(r))) {
+            if (nw) conj(d, vis_to_dec(bodies_masked(c, A, B, -1, band, wm + m * nw, nw, 0)));
+            else conj(d, vis_to_dec(bodies_all(c, A, B, -1, band, 0)));
+        }
+        __syncwarp(lanes);
+        A = B;
+        fa = fb;
+    }
+    return d;
 }
 
 // frame of the (S, c, P) problem: u towards S, v towards P (sphere: 3-D; cylinder: horizontal)
@@ -2296,16 +2565,16 @@ __device__ __forceinline__ void apply_records(const Ctx &c, AccS<float> &acc, co
 // tile by the per-receiver test too (FP32 with its band, or FP64), so
 // leaving them out changes no decision and no field.
 constexpr int SEQ_MASK_WORDS = 512;      // culling up to 16384 candidates (a larger list is not culled)
-__device__ __forceinline__ bool seq_may_hit(const Ctx &c, int q, int4 sq, const float lo[3], const float hi[3]) {
-    const int k = sq.w;
-    const int f = (k == 1) ? sq.x : ((k == 2) ? sq.y : sq.z);
-    const float4 I = c.cimg[6 * q + 2 * (k - 1)];
+// the points where the segments from the image I (after reflection m of
+// sequence sq, face f) to the box [lo, hi] cross f's plane, within f's box:
+// false if none can lie on f; [lo, hi] becomes the box of those that may
+__device__ __forceinline__ bool cross_box(const Ctx &c, float4 I, int f, float lo[3], float hi[3]) {
     const float4 pl = c.face32[f];
+    const float4 b0 = c.face_box[2 * f], b1 = c.face_box[2 * f + 1];
     const float di = pl.x * I.x + pl.y * I.y + pl.z * I.z - pl.w;
     const float m = 2.0f * c.band;
-    if (!(fabsf(di) > m)) return true;
     const float sg = di > 0.0f ? 1.0f : -1.0f;
-    bool same = true, opp = true;
+    bool same = fabsf(di) > m, opp = same;
     float qlo[3] = {INFINITY, INFINITY, INFINITY}, qhi[3] = {-INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
@@ -2320,19 +2589,37 @@ __device__ __forceinline__ bool seq_may_hit(const Ctx &c, int q, int4 sq, const 
         qlo[2] = fminf(qlo[2], z); qhi[2] = fmaxf(qhi[2], z);
     }
     if (same) return false;
-    if (!opp) return true;
-    const float4 b0 = c.face_box[2 * f], b1 = c.face_box[2 * f + 1];
-    return qlo[0] <= b1.x && qhi[0] >= b0.x && qlo[1] <= b1.y && qhi[1] >= b0.y && qlo[2] <= b1.z && qhi[2] >= b0.z;
+    const float bl[3] = {b0.x, b0.y, b0.z}, bh[3] = {b1.x, b1.y, b1.z};
+    const float g = hull_margin(c);             // (the crossing points' own rounding)
+    bool any = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        // the box straddles the plane: nothing but the face's box is known
+        if (opp) any = any && qlo[k] <= bh[k] && qhi[k] >= bl[k];
+        lo[k] = opp ? fmaxf(qlo[k] - g, bl[k]) : bl[k];
+        hi[k] = opp ? fminf(qhi[k] + g, bh[k]) : bh[k];
+    }
+    return any;
 }
-// All 32 lanes of a warp: the box of the tile's receivers (lanes with ok),
-// then bit lane of word w set iff candidate 32 w + lane is in share part of
-// nparts, within max_order, and not culled.  Returns false (no mask) when
-// the list is too long to be culled.
-__device__ __noinline__ bool seq_tile_mask(const Ctx &c, const float *rx, int n_rx, int r, bool ok, int part,
-                                           int nparts, int max_order, uint32_t *mask) {
-    if (c.n_cand > 32 * SEQ_MASK_WORDS) return false;
-    const int lane = threadIdx.x & 31;
-    float lo[3], hi[3];
+__device__ __forceinline__ bool seq_may_hit(const Ctx &c, int q, int4 sq, const float lo[3], const float hi[3]) {
+    const int k = sq.w;
+    const int f = (k == 1) ? sq.x : ((k == 2) ? sq.y : sq.z);
+    float l[3] = {lo[0], lo[1], lo[2]}, h[3] = {hi[0], hi[1], hi[2]};
+    return cross_box(c, c.cimg[6 * q + 2 * (k - 1)], f, l, h);
+}
+// The whole sequence for the box of a tile's receivers: the region of each
+// earlier reflection point is that of the segments from its image to the next
+// one's region; no path of the tile takes a sequence with an empty region.
+__device__ __noinline__ bool seq_culled(const Ctx &c, int q, const float tlo[3], const float thi[3]) {
+    const int4 sq = c.cand[q];
+    float lo[3] = {tlo[0], tlo[1], tlo[2]}, hi[3] = {thi[0], thi[1], thi[2]};
+    for (int m = sq.w - 1; m >= 0; --m)
+        if (!cross_box(c, c.cimg[6 * q + 2 * m], m == 0 ? sq.x : (m == 1 ? sq.y : sq.z), lo, hi)) return true;
+    return false;
+}
+// All 32 lanes of a warp: the box of the receivers of the lanes with ok;
+// false when there is none
+__device__ __forceinline__ bool tile_box(const float *rx, int n_rx, int r, bool ok, float lo[3], float hi[3]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const float v = ok ? rx[k * n_rx + r] : 0.0f;
@@ -2344,21 +2631,63 @@ __device__ __noinline__ bool seq_tile_mask(const Ctx &c, const float *rx, int n_
             hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
         }
     }
-    const int nw = (c.n_cand + 31) >> 5;
-    for (int w = 0; w < nw; ++w) {
-        const int q = 32 * w + lane;
-        bool keep = false;
-        if (q < c.n_cand && (1 + q) % nparts == part && lo[0] <= hi[0]) {
-            const int4 sq = c.cand[q];
-            if (sq.w <= max_order) keep = seq_may_hit(c, q, sq, lo, hi);
+    return lo[0] <= hi[0];
+}
+// The candidates of share part of nparts: those q with (1 + q) mod nparts =
+// part; the k-th of them, and how many of n there are.
+__device__ __forceinline__ int seq_of(int k, int part, int nparts) { return (part + nparts - 1) % nparts + nparts * k; }
+__device__ __forceinline__ int seq_share(int n, int part, int nparts) {
+    const int q0 = (part + nparts - 1) % nparts;
+    return n > q0 ? (n - q0 + nparts - 1) / nparts : 0;
+}
+// All 32 lanes of a warp: bit lane of word w set iff candidate 32 w + lane of
+// share part of nparts is within max_order and not culled for the tile.
+// First the last reflection, a candidate per lane; then, 32 of what is left at
+// a time (list: 64 slots of the warp), the whole sequence.  Returns false (no
+// mask) when the list is too long to be culled.
+//   A candidate that stays costs a BVH walk per receiver at least.  Of 2549
+// candidates of an office of 193 572 triangles, 360 pass the last reflection's
+// test per tile on average and 62 the whole sequence's (242 of 532 on one floor
+// section).  A walk for the whole tile instead -- is there one polygon that
+// hides the tile from the next region? -- was slower than the receivers' own
+// walks, 232 against 43 ms: those run side by side and end at the first of the
+// many small pieces of furniture, which hides no region by itself.
+__device__ __noinline__ bool seq_tile_mask(const Ctx &c, const float *rx, int n_rx, int r, bool ok, int part,
+                                           int nparts, int max_order, uint32_t *mask, int *list) {
+    if (c.n_cand > 32 * SEQ_MASK_WORDS) return false;
+    const int lane = threadIdx.x & 31;
+    float lo[3], hi[3];
+    const bool some = tile_box(rx, n_rx, r, ok, lo, hi);
+    const int nq = seq_share(c.n_cand, part, nparts), nw = (nq + 31) >> 5;
+    int have = 0;
+    if (nw == 0 && lane == 0) mask[0] = 0u;
+    for (int w = 0; w <= nw; ++w) {
+        if (w < nw) {
+            const int k = 32 * w + lane, q = seq_of(k, part, nparts);
+            bool keep = false;
+            if (k < nq && some) {
+                const int4 sq = c.cand[q];
+                if (sq.w <= max_order) keep = seq_may_hit(c, q, sq, lo, hi);
+            }
+            const unsigned word = __ballot_sync(0xffffffffu, keep);
+            if (lane == 0) mask[w] = word;
+            if (keep) list[have + __popc(word & ((1u << lane) - 1u))] = k;
+            have += __popc(word);
+            __syncwarp();
+            if (have < 32) continue;
         }
-        const unsigned word = __ballot_sync(0xffffffffu, keep);
-        if (lane == 0) mask[w] = word;
+        // (at the end the last few)
+        const int n = min(have, 32);
+        const int k = lane < n ? list[lane] : -1;
+        const int rest = lane + 32 < have ? list[lane + 32] : -1;
+        if (k >= 0 && seq_culled(c, seq_of(k, part, nparts), lo, hi)) atomicAnd(&mask[k >> 5], ~(1u << (k & 31)));
+        __syncwarp();
+        if (rest >= 0) list[lane] = rest;
+        have -= n;
+        __syncwarp();
     }
-    __syncwarp();
     return true;
 }
-
 // fields with the path list: the warps sharing a receiver take slots by
 // atomics (the list is in no particular order); returns the overflow flag
 __device__ __noinline__ uint32_t list_path(uint64_t *codes, int32_t *counts, int cap, int r, uint64_t code) {
@@ -2379,7 +2708,7 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                                               const uint32_t *occ_rx, int part, int nparts,
                                               AccS<T> acc, float *rec, uint32_t &fl, unsigned &nesc, int &npath,
                                               int &nrec_out, const uint32_t *qmask = nullptr, unsigned lanes = 0u,
-                                              uint32_t *pwm = nullptr) {
+                                              uint32_t *pwm = nullptr, int *cstk = nullptr) {
     constexpr bool BODIES = (CLS & CLS_BODIES) != 0;
     const bool fp32 = sizeof(T) == 4;
     const T band = fp32 ? T(c.band) : T(0);
@@ -2436,17 +2765,15 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
     // planar occluder masks (FP32 fields, enumeration): the lanes `lanes`
     // (every lane of the warp that evaluates a receiver) share them; pnw mask
     // words per leg, 0 without masks
-    constexpr bool PM = sizeof(T) == 4 && !PATHS && CLS == CLS_PLANAR;
+    constexpr bool PM = sizeof(T) == 4 && ((!PATHS && CLS == CLS_PLANAR) || CLS == CLS_SEQ);
     unsigned pl = 0u;
     int pnw = 0;
     float tcx = 0.0f, tcy = 0.0f, tcr = 0.0f;
     if constexpr (PM) {
-        if (pwm && lanes && c.n_body > 0 && c.n_body <= OCC_MAX_BODIES) {
-            pl = __ballot_sync(lanes, !inside);
-            if (pl) {
-                pnw = (c.n_body + 31) >> 5;
-                if (!inside) lanes_box(pl, true, Pf.x, Pf.y, tcx, tcy, tcr);
-            }
+        if (lanes) pl = __ballot_sync(lanes, !inside);
+        if (pwm && pl && c.n_body > 0 && c.n_body <= OCC_MAX_BODIES) {
+            pnw = (c.n_body + 31) >> 5;
+            if (!inside) lanes_box(pl, true, Pf.x, Pf.y, tcx, tcy, tcr);
         }
     }
     if (inside) {
@@ -2455,7 +2782,21 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
         if constexpr ((CLS & (CLS_PLANAR | CLS_SEQ)) != 0) {
             // ---- direct ray (candidate 0)
             if ((enable & RT_EN_LOS) && part == 0) {
-                int d = cand_los<T>(c, Sx, P, band);
+                int d;
+                if constexpr (CLS == CLS_SEQ && sizeof(T) == 4) {
+                    if (pl && c.bvh) {
+                        if (pnw) {
+                            const float cx[2] = {c.S.x, tcx}, cy[2] = {c.S.y, tcy}, cr[2] = {0.0f, tcr};
+                            leg_masks<1>(c, pl, cx, cy, cr, pwm, pnw);
+                        }
+                        const v3t<float> no[3] = {};
+                        d = seq_vis_coop(c, pl, make_int4(-1, -1, -1, 0), Sx, P, band, no, D_YES, pwm, pnw, cstk);
+                    } else {
+                        d = cand_los<T>(c, Sx, P, band);
+                    }
+                } else {
+                    d = cand_los<T>(c, Sx, P, band);
+                }
                 if (d == D_UNSURE) { escalated(); d = esc_los(c, Pf); }
                 if (d == D_YES) {
                     emit(PT_LOS, 0, 0);
@@ -2471,24 +2812,47 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
               if ((enable & RT_EN_PLANAR) && max_order >= 1) {
                 // the tile's mask (seq_tile_mask) lists this share's candidates
                 // that survive culling; without one, every candidate of the share
-                int w = 0, q = -1;
+                int w = qmask ? 0 : -1, q;
                 uint32_t word = qmask ? qmask[0] : 0u;
-                const int nw = (c.n_cand + 31) >> 5;
+                const int nq = seq_share(c.n_cand, part, nparts), nw = (nq + 31) >> 5;
 #pragma unroll 1
                 for (;;) {
                     if (qmask) {
                         while (word == 0u && ++w < nw) word = qmask[w];
                         if (word == 0u) break;
-                        q = 32 * w + __ffs(word) - 1;
+                        q = seq_of(32 * w + __ffs(word) - 1, part, nparts);
                         word &= word - 1u;
                     } else {
-                        if (++q >= c.n_cand) break;
-                        if ((1 + q) % nparts != part) continue;
+                        if (++w >= nq) break;
+                        q = seq_of(w, part, nparts);
                     }
                     const int4 sq = c.cand[q];
                     if (sq.w > max_order) continue;
                     v3t<T> Q[3];
-                    int d = cand_seq<T>(c, q, sq, Sx, P, band, Q);
+                    int d;
+                    if constexpr (sizeof(T) == 4) {
+                        if (pl && c.bvh) {
+                            d = cand_seq_geom<T>(c, q, sq, P, band, Q);
+                            const bool v = d != D_NO;
+                            if (!__any_sync(pl, v)) continue;        // (the whole warp)
+                            if (pnw) {
+                                float cx[5], cy[5], cr[5];
+                                cx[0] = c.S.x; cy[0] = c.S.y; cr[0] = 0.0f;
+#pragma unroll
+                                for (int m = 0; m < 3; ++m) {
+                                    if (m < sq.w) lanes_box(pl, v, Q[m].x, Q[m].y, cx[m + 1], cy[m + 1], cr[m + 1]);
+                                    else { cx[m + 1] = tcx; cy[m + 1] = tcy; cr[m + 1] = tcr; }
+                                }
+                                cx[4] = tcx; cy[4] = tcy; cr[4] = tcr;
+                                leg_masks<4>(c, pl, cx, cy, cr, pwm, pnw);
+                            }
+                            d = seq_vis_coop(c, pl, sq, Sx, P, band, Q, d, pwm, pnw, cstk);
+                        } else {
+                            d = cand_seq<T>(c, q, sq, Sx, P, band, Q);
+                        }
+                    } else {
+                        d = cand_seq<T>(c, q, sq, Sx, P, band, Q);
+                    }
                     if constexpr (sizeof(T) == 4) {
                         if (d == D_UNSURE) { escalated(); d = esc_seq(c, q, sq, Pf, Q); }
                     }
@@ -2620,7 +2984,9 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
             constexpr int PER = recs_per_unit(CLS);
             int nrec = 0;
 #pragma unroll 1
-            for (int b = b_begin + part; b < b_end; b += nparts) {
+            for (int bi = b_begin + part; bi < b_end; bi += nparts) {
+                // (scenes with a BVH: bi counts the bodies the source may see)
+                const int b = (CLS != CLS_WCREEP && c.blist) ? c.blist[bi] : bi;
                 if constexpr (RECS) {
                     // one frequency chunk: records that could overflow are turned
                     // into fields here (with several chunks the caller sizes the
@@ -2800,7 +3166,8 @@ __device__ __noinline__ void occ_masks(const Ctx &c, float t0x, float t0y, float
     const int lane = threadIdx.x & 31, nb = c.n_body;
     const float margin = 1e-3f + 8.0f * c.band;
 #pragma unroll 1
-    for (int b = wi; b < nb; b += nwarps) {
+    for (int bi = wi; bi < c.n_cand_body; bi += nwarps) {
+        const int b = c.blist ? c.blist[bi] : bi;
         const float4 qb = c.body[2 * b];
         const float rad = fmaxf(rr, qb.w) + c.band + margin;
 #pragma unroll 1
@@ -2840,6 +3207,24 @@ __device__ __forceinline__ void tile_masks(const Ctx &c, const float *rx, int n_
         occ_masks(c, along_x ? x0 : xm, along_x ? ym : y0, along_x ? x1 : xm, along_x ? ym : y1, rr, out, wi,
                   nwarps);
     }
+}
+
+// the whole block: the bodies without their bit in hid, in order; ends with a
+// barrier.  (An office's walls hide most of its bodies from a transmitter: the
+// warps of a tile share the rest evenly, where a skipped body in its owner's
+// loop left the others waiting.)
+__device__ __noinline__ void body_list(Ctx &c, const uint32_t *hid, uint16_t *list) {
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int n = 0;
+        for (int b0 = 0; b0 < c.n_body; b0 += 32) {
+            const unsigned word = ~hid[b0 >> 5] & (b0 + 32 <= c.n_body ? 0xffffffffu : (1u << (c.n_body - b0)) - 1u);
+            if (word >> lane & 1u) list[n + __popc(word & ((1u << lane) - 1u))] = (uint16_t)(b0 + lane);
+            n += __popc(word);
+        }
+        if (lane == 0) c.n_cand_body = n;
+    }
+    __syncthreads();
 }
 
 // copy n bytes (a multiple of 4) from global to shared memory, all threads
@@ -2905,6 +3290,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         c.face_rng = S.face_rng;
         c.face_tris = S.face_tris;
         c.face_box = S.face_box;
+        c.face_occ = S.face_occ;
         c.body = body_sm ? s_body : F1.body;
         c.n_tri = S.n_tri; c.n_face = S.n_face; c.n_body = frames ? 0 : F1.n_body;
         c.band = S.band_len;
@@ -2934,6 +3320,15 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
     const Ctx &c = s_ctx;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int NW = blk_of(CLS, sizeof(T) == 4) / 32;
+    // scenes with a BVH: the bodies not hidden from the source (body_list)
+    constexpr bool BLIST = BODIES && CLS != CLS_WCREEP;
+    __shared__ uint16_t s_blist[BLIST ? RT_MAX_BODIES : 1];
+    if (threadIdx.x == 0) {
+        s_ctx.blist = BLIST && S.bvh ? s_blist : nullptr;
+        s_ctx.n_cand_body = s_ctx.n_body;
+    }
+    __syncthreads();
+    if (BLIST && S.bvh && !frames) body_list(s_ctx, F1.hid, s_blist);
     if constexpr (PATHS) {
         // (one frame only)
         const float *rx = rx_base;
@@ -2960,6 +3355,10 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         // the launch's queue and lists every candidate itself (codes in the
         // canonical order)
         __shared__ uint32_t s_qmask_p[CLS == CLS_SEQ ? NW : 1][CLS == CLS_SEQ ? SEQ_MASK_WORDS : 1];
+        __shared__ int s_qlist_p[CLS == CLS_SEQ ? NW : 1][64];
+        constexpr bool COOP_P = CLS == CLS_SEQ && sizeof(T) == 4;
+        __shared__ uint32_t s_pwm_p[COOP_P ? NW : 1][COOP_P ? 4 * (OCC_MAX_BODIES / 32) : 1];
+        __shared__ int s_cstk_p[COOP_P ? NW : 1][COOP_P ? COOP_STACK : 1];
         for (;;) {
             unsigned long long t = 0;
             if (lane == 0) t = atomicAdd(queue, 1ull);
@@ -2973,8 +3372,9 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
             bool qm_on = false;
             if constexpr (CLS == CLS_SEQ) {
                 qm_on = seq_tile_mask(c, rx, n_rx, r < n_rx ? r : n_rx - 1, r < n_rx, 0, 1, S.max_order,
-                                      &s_qmask_p[warp][0]);
+                                      &s_qmask_p[warp][0], &s_qlist_p[warp][0]);
             }
+            const unsigned lanes_p = __ballot_sync(0xffffffffu, r < n_rx);
             if (r < n_rx) {
                 AccS<T> acc{nullptr};                // no fields in this mode
                 uint32_t fl;
@@ -2983,9 +3383,11 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                 int nrec;
                 eval_receiver<T, PATHS, CLS, LIST>(c, s_fqs, 1, S.enable, S.max_order, rx, n_rx, r, codes, counts, cap,
                                                    F1.hl,
-                                             0, CLS == CLS_WCREEP ? c.n_face * c.n_body : c.n_body, true, false, 0,
+                                             0, CLS == CLS_WCREEP ? c.n_face * c.n_body : c.n_cand_body, true, false, 0,
                                              occ_on ? s_occ_mine : nullptr, 0, 1, acc,
-                                             nullptr, fl, nesc, npath, nrec, qm_on ? &s_qmask_p[warp][0] : nullptr);
+                                             nullptr, fl, nesc, npath, nrec, qm_on ? &s_qmask_p[warp][0] : nullptr,
+                                             COOP_P ? lanes_p : 0u, &s_pwm_p[COOP_P ? warp : 0][0],
+                                             &s_cstk_p[COOP_P ? warp : 0][0]);
                 counts[r] = npath;
                 if (fl_base) fl_base[r] = accumulate ? (fl_base[r] | fl) : fl;
                 if (nesc) atomicAdd(esc_counter, (unsigned long long)nesc);
@@ -3024,7 +3426,11 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         T *s_part = WIDE ? reinterpret_cast<T *>(s_rec) : &s_part_st[0][0][0];
         __shared__ uint32_t s_fl[NW][32];
         __shared__ uint32_t s_qmask[CLS == CLS_SEQ ? NW : 1][CLS == CLS_SEQ ? SEQ_MASK_WORDS : 1];
-        __shared__ uint32_t s_pwm[CLS == CLS_PLANAR ? NW : 1][CLS == CLS_PLANAR ? 3 * (OCC_MAX_BODIES / 32) : 1];
+        __shared__ int s_qlist[CLS == CLS_SEQ ? NW : 1][64];
+        constexpr bool COOP = CLS == CLS_SEQ && sizeof(T) == 4;
+        constexpr bool LEGM = COOP || CLS == CLS_PLANAR;
+        __shared__ uint32_t s_pwm[LEGM ? NW : 1][LEGM ? 4 * (OCC_MAX_BODIES / 32) : 1];
+        __shared__ int s_cstk[COOP ? NW : 1][COOP ? COOP_STACK : 1];
         __shared__ unsigned long long s_unit;
         __shared__ int s_fi, s_new;
         __shared__ FrameDev s_fr;
@@ -3072,8 +3478,10 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                     s_ctx.txb = body_sm ? s_txb : s_fr.txb;
                     s_ctx.n_body = s_fr.n_body;
                     s_ctx.band = s_fr.band;
+                    s_ctx.n_cand_body = s_fr.n_body;
                 }
                 __syncthreads();
+                if (BLIST && S.bvh) body_list(s_ctx, s_fr.hid, s_blist);
                 if (occ_on) {
                     occ_masks(c, c.S.x, c.S.y, c.S.x, c.S.y, 0.0f, s_occ_src, warp, NW);
                     __syncthreads();
@@ -3084,7 +3492,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
             const float *rx = rx_base + 3 * Fr.rx_off;
             float *e_out = e_base + Fr.e_off;
             uint32_t *flags_out = fl_base ? fl_base + Fr.rx_off : nullptr;
-            const int n_b = BODIES ? (CLS == CLS_WCREEP ? c.n_face * c.n_body : c.n_body) : 0;
+            const int n_b = BODIES ? (CLS == CLS_WCREEP ? c.n_face * c.n_body : c.n_cand_body) : 0;
             // bodies per geometry pass: all of them with one frequency chunk (full
             // record buffers are flushed on the way), else as many as the buffer holds
             const int bc = (RECS && nch > 1) ? NWT * (rcap / PER) : (n_b > 0 ? n_b : 1);
@@ -3102,7 +3510,8 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
             bool qm_on = false;
             if constexpr (CLS == CLS_SEQ) {
                 if (n_rx > 0)
-                    qm_on = seq_tile_mask(c, rx, n_rx, rok ? r : n_rx - 1, rok, part, NWT, S.max_order, &s_qmask[warp][0]);
+                    qm_on = seq_tile_mask(c, rx, n_rx, rok ? r : n_rx - 1, rok, part, NWT, S.max_order, &s_qmask[warp][0],
+                                          &s_qlist[warp][0]);
             }
             AccS<T> acc{s_part + warp * prow * 32 + lane};     // the warp's partial sums, summed in place
             float *rec = s_rec + warp * (rcap * REC_N * 32) + lane;
@@ -3118,7 +3527,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                                                  Fr.hl, b0, min(b0 + bc, n_b), b0 == 0, nch == 1, rcap,
                                                  occ_on ? s_occ_rx + grp * S.n_body * occ_w : nullptr, part,
                                                  NWT, acc, rec, fl, nesc, npath, nrec,
-                                                 qm_on ? &s_qmask[warp][0] : nullptr, lanes, &s_pwm[warp][0]);
+                                                 qm_on ? &s_qmask[warp][0] : nullptr, lanes, &s_pwm[LEGM ? warp : 0][0], &s_cstk[COOP ? warp : 0][0]);
                 s_fl[warp][lane] = fl;
                 if (nesc && ch0 == 0) atomicAdd(esc_counter, (unsigned long long)nesc);
 #pragma unroll 1
@@ -3327,6 +3736,16 @@ static int run(const DevScene &S, const Work &W, int precision, bool paths, bool
     LaunchCtx L{ctr, 0, stream};
     const int nchunks = paths ? 1 : (S.n_f + NFC - 1) / NFC;
     cudaError_t e;
+    // scenes with a BVH: the bodies hidden from the transmitter first
+    const int hid = S.bvh && S.n_body > 0 && (S.enable & (RT_EN_BODYREFL | RT_EN_CREEP_SOFT | RT_EN_CREEP_HARD)) ? 1 : 0;
+    if (hid) {
+        k_src_hidden<<<dim3((S.n_body + HID_WARPS - 1) / HID_WARPS, W.frames ? W.n_frames : 1), 32 * HID_WARPS, 0,
+                       stream>>>(S, W.F1, W.frames);
+        if ((e = cudaGetLastError()) != cudaSuccess) {
+            set_error(std::string("k_src_hidden launch: ") + cudaGetErrorString(e));
+            return RT_ERR_CUDA;
+        }
+    }
     if (precision == RT_PREC_FP64) {
         e = paths ? launch_all<dx, true>(S, W, nchunks, L) : launch_all<dx, false>(S, W, nchunks, L);
         if (list && e == cudaSuccess) e = launch_all<dx, true>(S, W, 1, L);
@@ -3335,7 +3754,7 @@ static int run(const DevScene &S, const Work &W, int precision, bool paths, bool
     } else {
         e = list ? launch_all<float, false, true>(S, W, nchunks, L) : launch_all<float, false>(S, W, nchunks, L);
     }
-    *n_launches = L.n;
+    *n_launches = L.n + hid;          // (with k_src_hidden)
     if (e != cudaSuccess) {
         set_error(std::string("k_eval launch: ") + cudaGetErrorString(e));
         return RT_ERR_CUDA;
@@ -3354,6 +3773,7 @@ int launch_eval(const DevScene &S, const float *rx_soa, int n_rx, float *e_out, 
     W.F1.body = S.body;
     W.F1.txb = S.txb;
     W.F1.fqc = S.fqc;
+    W.F1.hid = S.hid;
     W.F1.n_rx = n_rx;
     W.F1.n_body = S.n_body;
     W.F1.band = S.band_len;
@@ -3964,7 +4384,7 @@ __global__ void __launch_bounds__(128) k_adjoint(DevScene S, const float *__rest
     typedef decltype(DT().v) SC;
     Ctx c;
     c.tri = S.tri; c.tri_aux = S.tri_alt; c.face32 = S.face32; c.face64 = S.face64;
-    c.face_rng = S.face_rng; c.face_tris = S.face_tris; c.face_box = S.face_box; c.body = S.body;
+    c.face_rng = S.face_rng; c.face_tris = S.face_tris; c.face_box = S.face_box; c.face_occ = nullptr; c.blist = nullptr; c.n_cand_body = S.n_body; c.body = S.body;
     c.n_tri = S.n_tri; c.n_face = S.n_face; c.n_body = S.n_body;
     c.band = 0.0f;
     c.S = mk3(S.tx[0], S.tx[1], S.tx[2]);

@@ -75,6 +75,9 @@ struct DevScene {
     const int2 *face_rng;      // [n_face]: first, count in face_tris
     const float4 *face_box;    // [n_face][2]: box of the face's triangles (min, max), grown by the margin
                                // beyond which the FP32 face-membership test is a certain no
+    const float4 *face_occ;    // [n_face][4] the face as one convex polygon (scenes with a BVH): its vertices, their
+                               // number in the first's w (int bits); 0: its triangles are taken one by one
+    uint32_t *hid;             // see FrameDev::hid (a plain evaluation's)
     const int *face_tris;      // [n_tri]
     const float4 *body;        // [n_body][2]: (cx, cy, cz, a), (h, type, 0, 0)
     const float4 *fock32;      // [FOCK_N][2]: (G.re, G.im, h G'.re, h G'.im) soft, hard; then
@@ -122,6 +125,8 @@ struct FrameDev {
     const float4 *body;        // [n_body][2], as DevScene::body
     const float4 *txb;         // [n_body][2], as DevScene::txb
     const FreqC *fqc;          // [ceil(n_f / NFC)] frequency constants
+    uint32_t *hid;             // [RT_MAX_BODIES / 32] bodies hidden from the transmitter (scenes with a BVH; written by
+                               // each evaluation's first kernel), or nullptr
     long long rx_off;          // first receiver: SoA block at rx + 3 rx_off, flags at flags + rx_off
     long long e_off;           // first output float
     unsigned long long tile0;  // first tile of the batch's tile range
