@@ -3822,77 +3822,547 @@ int launch_eval_batch(const DevScene &S, const FrameDev *frames_dev, const Frame
 // field derivative with respect to its body's centre and radius, the
 // transmitter position and the frequency.  Visibility is held fixed: the
 // paths are those of the forward path list (rt_paths), and each one's
-// geometry and field are recomputed here in dual numbers (dual.cuh), by the
-// same construction as the forward path: image points for planar
-// reflections (Eq. 3), the specular point on the body (its derivative from
-// one Newton step in dual arithmetic at the root, which is the
-// implicit-function derivative), the tangent points and geodesic of the
-// creeping ray (Eq. 4, Fig. 1), the Fock--Pekeris functions (table
-// derivative from the cubic Hermite interpolant, residue series term by
-// term), the transition function through w'(z) = -2 z w(z) + 2j/sqrt(pi).
+// geometry is recomputed here in dual numbers (dual.cuh), by the same
+// construction as the forward path: image points for planar reflections
+// (Eq. 3), the specular point on the body (its derivative from one Newton step
+// in dual arithmetic at the root, which is the implicit-function derivative),
+// the tangent points and geodesic of the creeping ray (Eq. 4, Fig. 1).  The
+// field is a function of a dozen scalars of that geometry and the frequency:
+// it is differentiated backwards from dLoss/dE (adj_apply, adj_ray), with the
+// slopes of the Fock--Pekeris functions (table derivative from the cubic
+// Hermite interpolant, residue series term by term) and of the transition
+// function through w'(z) = -2 z w(z) + 2j/sqrt(pi).
 //
-// F8 (FP32 duals, the default): the forward FP32 construction -- FP32
-// geometry, table and Faddeeva coefficients -- with each path's length for
-// the phase as double-float from the same exact pieces the forward FP32
-// kernel uses (the source's FP64 images, the tangent lengths from exact
-// squares), so its phase keeps the forward's accuracy.  Direct, planar and
-// creeping paths take F8; reflections off a body take D8 in both modes.
-// D8 (FP64 duals, RT_PREC_FP64): the forward FP64 construction.
+// FP32 duals (the default): the forward FP32 construction -- FP32 geometry,
+// table and Faddeeva coefficients -- with each path's length for the phase as
+// double-float from the same exact pieces the forward FP32 kernel uses (the
+// source's FP64 images, the tangent lengths from exact squares), so its phase
+// keeps the forward's accuracy.  Direct, planar and creeping paths take them;
+// reflections off a body take FP64 duals in both modes.
+// FP64 duals (RT_PREC_FP64): the forward FP64 construction.
 
-template <> __device__ __forceinline__ void face_plane<D8>(const Ctx &c, int f, v3t<D8> *n, D8 *d) {
-    dq4 q = c.face64[f]; *n = mk3<D8>(q.x, q.y, q.z); *d = D8(q.w);
+template <> __device__ __forceinline__ void face_plane<D3>(const Ctx &c, int f, v3t<D3> *n, D3 *d) {
+    dq4 q = c.face64[f]; *n = mk3<D3>(q.x, q.y, q.z); *d = D3(q.w);
 }
+template <> __device__ __forceinline__ void face_plane<D7>(const Ctx &c, int f, v3t<D7> *n, D7 *d) {
+    dq4 q = c.face64[f]; *n = mk3<D7>(q.x, q.y, q.z); *d = D7(q.w);
+}
+
+// ---- FP64: Fock--Pekeris functions of a dual xi: value and slope in scalars (the
+// residue series term by term above XI_HI, else the table's cubic Hermite
+// interpolant and its slope), then the chain rule once.  A term of the series
+// is left out once it is below 2^-60 of the first.
+__device__ __forceinline__ double adj_res(const Ctx &c, int n, int k, double *x, double *y) {
+    const dq4 q = c.res64[2 * n + k];
+    *x = q.x; *y = q.y;
+    return q.z;
+}
+__device__ __forceinline__ void adj_node(const Ctx &c, int j, int k, cpx<double> *g, cpx<double> *hd) {
+    const double2 a = c.fock64[(j * 2 + k) * 2], q = c.fock64[(j * 2 + k) * 2 + 1];
+    *g = mkc(a.x, a.y);
+    *hd = mkc(q.x * XI_STEP, q.y * XI_STEP);
+}
+template <int N>
+__device__ __forceinline__ cpx<DualT<double, N>> cchain(cpx<double> y, cpx<double> dy, const DualT<double, N> &x) {
+    return mkc<DualT<double, N>>(dchain<double, N>(y.re, dy.re, x), dchain<double, N>(y.im, dy.im, x));
+}
+template <int N>
+__device__ void pekeris(const Ctx &c, const DualT<double, N> &xid, cpx<DualT<double, N>> &ps, cpx<DualT<double, N>> &ph, bool regular) {
+    const double xi = xid.v;
+    const double ci = 0.19947114020071633897 / xi, dci = -ci / xi;   // c/xi = (ci, -ci)
+    cpx<double> v[2], d[2];
+    bool reg;
+    if (xi > double(XI_HI)) {
+        const double cut = 42.0;
+        const cpx<double> pre = mkc<double>(-0.27248264483602590, 0.07301150463530957);    // -e^{-j pi/12} / (2 sqrt(pi))
+#pragma unroll 1
+        for (int k = 0; k < 2; ++k) {
+            cpx<double> s = mkc<double>(0.0, 0.0), ds = s;
+            double x0, y0;
+            adj_res(c, 0, k, &x0, &y0);
+#pragma unroll 1
+            for (int n = 0; n < FOCK_NRES; ++n) {
+                double x, y;
+                const double z = adj_res(c, n, k, &x, &y);
+                if (xi * (x - x0) > cut) break;
+                double sn, cs;
+                dsincos(xi * y, &sn, &cs);
+                const double e = Exp(-(xi * x)) * z;
+                const cpx<double> t = mkc<double>(e * cs, -(e * sn));
+                s = s + t;
+                ds = ds - mkc<double>(x, y) * t;
+            }
+            v[k] = pre * s;
+            d[k] = pre * ds;
+        }
+        reg = false;                               // P
+    } else {
+        const double u = (xi - double(XI_LO)) * double(1.0 / XI_STEP);
+        const int j = min(max((int)u, 0), FOCK_N - 2);
+        const double t = u - double(j), t2 = t * t, omt = 1.0 - t;
+        const double h00 = (1.0 + 2.0 * t) * omt * omt, h10 = t * omt * omt, h01 = t2 * (3.0 - 2.0 * t),
+                h11 = t2 * (t - 1.0);
+        const double ih = double(1.0 / XI_STEP);             // d/dxi = (d/dt) / XI_STEP
+        const double d00 = (6.0 * t2 - 6.0 * t) * ih, d10 = (1.0 - 4.0 * t + 3.0 * t2) * ih, d01 = -d00,
+                d11 = (3.0 * t2 - 2.0 * t) * ih;
+        const cpx<double> rot = cexpi(xi * xi * xi * double(1.0 / 12.0));
+        const double w = 0.25 * xi * xi;             // e^{j xi^3/12}' = j w e^{..}
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            cpx<double> g0, q0, g1, q1;
+            adj_node(c, j, k, &g0, &q0);
+            adj_node(c, j + 1, k, &g1, &q1);
+            const cpx<double> G = g0 * h00 + q0 * h10 + g1 * h01 + q1 * h11, D = g0 * d00 + q0 * d10 + g1 * d01 + q1 * d11;
+            v[k] = G * rot;
+            d[k] = (D + mkc<double>(-w * G.im, w * G.re)) * rot;
+        }
+        reg = true;                                // P + c/xi
+    }
+    if (reg != regular) {
+        const double sg = regular ? 1.0 : -1.0;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            v[k] = v[k] + mkc<double>(sg * ci, -(sg * ci));
+            d[k] = d[k] + mkc<double>(sg * dci, -(sg * dci));
+        }
+    }
+    ps = cchain<N>(v[0], d[0], xid);
+    ph = cchain<N>(v[1], d[1], xid);
+}
+
+// w(z) of a dual z, with w'(z) = -2 z w(z) + 2j / sqrt(pi)
+template <typename S, int N>
+__device__ __forceinline__ cpx<DualT<S, N>> faddeeva_dual(const cpx<DualT<S, N>> &zd, cpx<S> w) {
+    const cpx<S> z = mkc(zd.re.v, zd.im.v);
+    const cpx<S> wp = z * w * S(-2) + mkc(S(0), S(1.1283791670955126));
+    cpx<DualT<S, N>> r;
+    r.re.v = w.re; r.im.v = w.im;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        r.re.d[k] = wp.re * zd.re.d[k] - wp.im * zd.im.d[k];
+        r.im.d[k] = wp.re * zd.im.d[k] + wp.im * zd.re.d[k];
+    }
+    return r;
+}
+template <int N>
+__device__ __forceinline__ cpx<DualT<double, N>> faddeeva_t(const Ctx &c, const cpx<DualT<double, N>> &zd) {
+    const cpx<dx> w = faddeeva_dx(c, mkc<dx>(zd.re.v, zd.im.v));
+    return faddeeva_dual<double, N>(zd, mkc(w.re.v, w.im.v));
+}
+
+// the path phasor e^{-j k L}
+__device__ __forceinline__ cpx<double> adj_phase(const FreqC &fq, int f, double L) {
+    double cyc = L * fq.fc[f], s, co;
+    cyc -= floor(cyc);                              // the integer cycles (no derivative)
+    sincospi(2.0 * cyc, &s, &co);
+    return mkc(co, -s);
+}
+// Re(a) Re(b) + Im(a) Im(b): the loss's change for a field's change b, a = dLoss/dE
+__device__ __forceinline__ double cdot(cpx<double> a, cpx<double> b) { return a.re * b.re + a.im * b.im; }
+
+// the gradients of one path: body (4) and transmitter (3) slots, and the
+// frequencies of the chunk; dLoss/dE of its receiver
+struct AccAdj {
+    const float *gE;        // [n_f][3][n_rx][2]
+    int n_rx, r, f0;
+    double g[7];
+    double gf[NFC];
+};
+__device__ __forceinline__ void adj_ge(const AccAdj &a, int f, cpx<double> g[3]) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const float *v = a.gE + 2 * (((size_t)(a.f0 + f) * 3 + q) * a.n_rx + a.r);   // (any float alignment)
+        g[q] = mkc<double>(double(v[0]), double(v[1]));
+    }
+}
+
+// The frequency-independent factors of a body path's field, in duals:
+//   E = (e1 Cs Es + e2 Ch Eh) A c0 e^{-j k L} j^jpow,
+// for a creeping ray (RB false) C = the Fock bracket at xi = m x, c0 = -m
+// sqrt(2 / k); for a reflection C = its uniform coefficient at xi = -2 m x, c0
+// = 1; m = (k / 2)^{1/3} rcb, K = sqrt(k L' / (2 m^2)).
+struct AdjRec {
+    D7 Es, Eh, A, Lp, rcb, x, L;
+    v3t<D7> e1, e2;
+};
+struct AdjBrk {
+    cpx<double> s, h, s_x, h_x, s_k;              // the bracket, its slopes in xi, and in K (the same for both)
+};
+__device__ __noinline__ AdjBrk adj_bracket(const Ctx &c, double xi, double K) {
+    typedef DualT<double, 2> D2;
+    cpx<D2> Bs, Bh;
+    fock_bracket_impl<D2>(c, dvar_t<double, 2>(xi, 0), dvar_t<double, 2>(K, 1), Bs, Bh);
+    AdjBrk b;
+    b.s = mkc(Bs.re.v, Bs.im.v);
+    b.h = mkc(Bh.re.v, Bh.im.v);
+    b.s_x = mkc(Bs.re.d[0], Bs.im.d[0]);
+    b.h_x = mkc(Bh.re.d[0], Bh.im.d[0]);
+    b.s_k = mkc(Bs.re.d[1], Bs.im.d[1]);
+    return b;
+}
+// The path's field contracted with dLoss/dE backwards: per frequency the loss's
+// slope in each of the record's scalars, from one evaluation of the bracket
+// with its two slopes; their sum over the frequencies then meets the scalars'
+// tangents once.  (Forward duals through the field carried all eight tangents
+// through every Fock function, phasor and product.)
+template <bool RB>
+__device__ __noinline__ void adj_apply(const Ctx &c, const FreqC &fq, const AdjRec &R, int jpow, AccAdj &acc) {
+    const double Es = R.Es.v, Eh = R.Eh.v, A = R.A.v, Lp = R.Lp.v, rcb = R.rcb.v, x = R.x.v, L = R.L.v;
+    const double e1[3] = {R.e1.x.v, R.e1.y.v, R.e1.z.v}, e2[3] = {R.e2.x.v, R.e2.y.v, R.e2.z.v};
+    double gEs = 0, gEh = 0, gA = 0, gLp = 0, grcb = 0, gx = 0, gL = 0, ge1[3] = {0, 0, 0}, ge2[3] = {0, 0, 0};
+#pragma unroll 1
+    for (int f = 0; f < fq.nf; ++f) {
+        const double k = fq.kd[f], m = cbrt(fq.kd[f] * 0.5) * rcb;
+        const double xi = RB ? -2.0 * m * x : m * x;
+        const bool fock = !RB || xi >= double(XI_LO);
+        double K = 0.0;
+        AdjBrk b;
+        if (fock) {
+            K = Sqrt(k * Lp / (2.0 * m * m));
+            b = adj_bracket(c, xi, K);
+            if (RB) {
+                // R = p B, p = -sqrt(-4 / xi) e^{-j xi^3 / 12}, p' / p = -1 / (2 xi) - j xi^2 / 4
+                double sn, cs;
+                dsincos(-(xi * xi * xi) * double(1.0 / 12.0), &sn, &cs);
+                const cpx<double> p = mkc<double>(cs, sn) * (-Sqrt(-4.0 / xi)), q = mkc<double>(-0.5 / xi, -0.25 * xi * xi);
+                b.s_x = p * (q * b.s + b.s_x);
+                b.h_x = p * (q * b.h + b.h_x);
+                b.s_k = p * b.s_k;
+                b.s = p * b.s;
+                b.h = p * b.h;
+            }
+        } else {
+            b.s = mkc<double>(-1.0, 0.0);
+            b.h = mkc<double>(1.0, 0.0);
+        }
+        cpx<double> u = adj_phase(fq, f, R.L.v);
+        if (jpow & 1) u = mkc<double>(-u.im, u.re);
+        if (jpow & 2) u = mkc<double>(-u.re, -u.im);
+        if (!RB) u = u * (-(m * Sqrt(2.0 / k)));
+        cpx<double> g[3];
+        adj_ge(acc, f, g);
+        const cpx<double> G1 = g[0] * e1[0] + g[1] * e1[1] + g[2] * e1[2], G2 = g[0] * e2[0] + g[1] * e2[1] + g[2] * e2[2];
+        const cpx<double> us = b.s * u, uh = b.h * u;
+        const double ls = cdot(G1, us), lh = cdot(G2, uh), l0 = Es * ls + Eh * lh;
+        gEs += A * ls;
+        gEh += A * lh;
+        gA += l0;
+        const cpx<double> as = us * (A * Es), ah = uh * (A * Eh);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            ge1[q] += cdot(g[q], as);
+            ge2[q] += cdot(g[q], ah);
+        }
+        // d(field)/dL = -j k field
+        const double t = (G1.re * as.im - G1.im * as.re) + (G2.re * ah.im - G2.im * ah.re);
+        gL += k * t;
+        double dk = L * t;
+        if (!RB) {                                 // c0 ~ rcb k^{-1/6}
+            grcb += A * l0 / rcb;
+            dk -= A * l0 / (6.0 * k);
+        }
+        if (fock) {                                // xi ~ rcb x k^{1/3}, K ~ L'^{1/2} rcb^{-1} k^{1/6}
+            const double lx = A * (Es * cdot(G1, b.s_x * u) + Eh * cdot(G2, b.h_x * u));
+            const double lk = A * (Es * cdot(G1, b.s_k * u) + Eh * cdot(G2, b.s_k * u));
+            grcb += (lx * xi - lk * K) / rcb;
+            gx += lx * (RB ? -2.0 * m : m);
+            if (Lp > 0.0) gLp += lk * K / (2.0 * Lp);
+            dk += (lx * xi * double(1.0 / 3.0) + lk * K * double(1.0 / 6.0)) / k;
+        }
+        acc.gf[f] += (double)dk * (2.0 * M_PI / 299792458.0);
+    }
+#pragma unroll
+    for (int k = 0; k < 7; ++k)
+        acc.g[k] += (double)(gEs * R.Es.d[k] + gEh * R.Eh.d[k] + gA * R.A.d[k] + gLp * R.Lp.d[k] + grcb * R.rcb.d[k] +
+                             gx * R.x.d[k] + ge1[0] * R.e1.x.d[k] + ge1[1] * R.e1.y.d[k] + ge1[2] * R.e1.z.d[k] +
+                             ge2[0] * R.e2.x.d[k] + ge2[1] * R.e2.y.d[k] + ge2[2] * R.e2.z.d[k] + gL * R.L.d[k]);
+}
+// the same for a planar path: E = e e^{-j k L} / L, its polarisation e complex
+// (CX) where a face is dielectric; only the transmitter moves it
+template <bool CX>
+__device__ __noinline__ void adj_ray(const FreqC &fq, const cpx<D3> e[3], const D3 &Ld,
+                                     AccAdj &acc) {
+    const double A = 1.0 / Ld.v, L = Ld.v;
+    double gA = 0, gL = 0, gr[3] = {0, 0, 0}, gi[3] = {0, 0, 0};
+#pragma unroll 1
+    for (int f = 0; f < fq.nf; ++f) {
+        const double k = fq.kd[f];
+        const cpx<double> u = adj_phase(fq, f, Ld.v);
+        cpx<double> g[3];
+        adj_ge(acc, f, g);
+        double l0 = 0, t0 = 0;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const double s = cdot(g[q], u), t = g[q].re * u.im - g[q].im * u.re;      // <g, u>, <g, -j u>
+            gr[q] += A * s;
+            l0 += e[q].re.v * s;
+            t0 += e[q].re.v * t;
+            if (CX) {
+                gi[q] -= A * t;
+                l0 -= e[q].im.v * t;
+                t0 += e[q].im.v * s;
+            }
+        }
+        gA += l0;
+        gL += k * A * t0;
+        acc.gf[f] += (double)(A * t0 * L) * (2.0 * M_PI / 299792458.0);
+    }
+    gL -= gA * A * A;                              // (the amplitude 1 / L)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        double v = gr[0] * e[0].re.d[k] + gr[1] * e[1].re.d[k] + gr[2] * e[2].re.d[k] + gL * Ld.d[k];
+        if (CX) v += gi[0] * e[0].im.d[k] + gi[1] * e[1].im.d[k] + gi[2] * e[2].im.d[k];
+        acc.g[DS_SX + k] += (double)v;
+    }
+}
+
+// body b's centre and radius as parameters (slots 0-3)
+__device__ __forceinline__ void adj_body(const Ctx &c, int b, v3t<D7> &cc, D7 &a, bool &sphere) {
+    float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
+    cc = mk3<D7>(dvar_t<double, 7>(q0.x, DS_CX), dvar_t<double, 7>(q0.y, DS_CY), dvar_t<double, 7>(q0.z, DS_CZ));
+    a = dvar_t<double, 7>(q0.w, DS_A);
+    sphere = q1.y == 0.0f;
+}
+
+// the reflection point's angle as a dual: the FP64 root (refined to the
+// bisection root), then one Newton step on dL/dpsi = 0 in dual arithmetic
+// (the implicit-function derivative)
+__device__ __noinline__ void adj_refl_root(const D7 &a, const D7 &ds, const D7 &pu, const D7 &pv, const D7 &gam, D7 *cs,
+                                           D7 *sn) {
+    dx c0, s0;
+    refl_root(dx(a.v), dx(ds.v), dx(pu.v), dx(pv.v), dx(gam.v), &c0, &s0);
+    const D7 psi(atan2(s0.v, c0.v));
+    D7 s, c;
+    SinCos(psi, &s, &c);
+    const D7 qx = a * c, qy = a * s;
+    const D7 lS = Sqrt((qx - ds) * (qx - ds) + qy * qy);
+    const D7 lP = Sqrt((qx - pu) * (qx - pu) + (qy - pv) * (qy - pv));
+    const D7 gS = a * ds * s / lS, gP = a * (pu * s - pv * c) / lP;
+    const D7 h = (ds * qx - gS * gS) / lS + (pu * qx + pv * qy - gP * gP) / lP;
+    SinCos(psi - (gS + gP) / h, sn, cs);
+}
+
+// reflection off body b (the forward construction, without decisions): FP64
+// duals in both precisions (the FP32 chain through the specular point left
+// errors of ~1e-3 of the gradient on the test scenes)
+__device__ __noinline__ void adj_rb(const Ctx &c, int b, const v3t<D7> &S, const v3t<D7> &P, AdjRec &R) {
+    v3t<D7> cc;
+    D7 a;
+    bool sphere;
+    adj_body(c, b, cc, a, sphere);
+    Frame<D7> F;
+    if (sphere) sphere_frame(S, P, cc, a, F, D7(0.0));
+    else cyl_frame(S, P, cc.x, cc.y, a, F, D7(0.0));
+    D7 cs, sn;
+    adj_refl_root(a, F.ds, F.pu, F.pv, F.gam, &cs, &sn);
+    const v3t<D7> n = F.u * cs + F.v * sn;
+    v3t<D7> Q;
+    if (sphere) {
+        Q = cc + n * a;
+    } else {
+        const D7 qx = a * cs, qy = a * sn;
+        const D7 l1 = Sqrt((qx - F.ds) * (qx - F.ds) + qy * qy);
+        const D7 l2 = Sqrt((qx - F.pu) * (qx - F.pu) + (qy - F.pv) * (qy - F.pv));
+        const D7 zq = S.z + (P.z - S.z) * l1 / (l1 + l2);
+        Q = mk3<D7>(cc.x + a * n.x, cc.y + a * n.y, zq);
+    }
+    const v3t<D7> di = Q - S;
+    const D7 si = norm3(di), sr = norm3(P - Q);
+    const v3t<D7> shi = di * (D7(1.0) / si);
+    const D7 ct = -dot3(shi, n);
+    D7 f1, f2(0.0), rho;                           // curvature terms and the surface's radius in the incidence plane
+    if (sphere) {
+        f1 = D7(2.0) / (a * ct);
+        f2 = D7(2.0) * ct / a;
+        rho = a;
+    } else {
+        f1 = D7(2.0) * (D7(1.0) - shi.z * shi.z) / (a * ct);
+        const D7 sphi = -(shi.x * n.y) + shi.y * n.x;
+        rho = (sphi == D7(0.0)) ? D7(INFINITY) : a * (D7(1.0) - ct * ct) / (sphi * sphi);
+    }
+    const D7 cth = Fmax(ct, D7(COS_MIN));          // (as in cand_rb)
+    const v3t<D7> shr = unit3(shi + n * (D7(2.0) * cth));
+    v3t<D7> ep = cross3(n, shi);
+    const D7 ne = norm3(ep);
+    if (ne == D7(0.0)) {
+        const v3t<D7> tmp = (Fabs(n.x) < D7(0.9)) ? mk3<D7>(1, 0, 0) : mk3<D7>(0, 1, 0);
+        ep = unit3(cross3(n, tmp));
+    } else {
+        ep = ep * (D7(1.0) / ne);
+    }
+    const v3t<D7> e0 = src_pol(c, shi);
+    R.Es = dot3(e0, ep);
+    R.Eh = dot3(e0, cross3(ep, shi));
+    R.e1 = ep;
+    R.e2 = cross3(ep, shr);
+    const D7 r1 = D7(1.0) / (D7(1.0) / si + f1), r2 = D7(1.0) / (D7(1.0) / si + f2);
+    R.A = Sqrt(r1 * r2 / ((r1 + sr) * (r2 + sr))) / si;
+    R.Lp = si * sr / (si + sr);
+    R.rcb = Cbrt(rho);
+    R.x = cth;
+    R.L = si + sr;
+}
+
+// creeping ray round body b, dir 0 short way, 1 long way, with enc extra
+// turns; wall >= 0: fed by the reflection at face wall (the creeping ray of
+// the source's image there).  jpow: powers of j of the ray's caustics; ei: the
+// imaginary part of the incident field's (Es, Eh) behind a dielectric wall.
+// Returns the parts of the field (2: with ei), 0: no finite field.
+__device__ __noinline__ int adj_creep(const Ctx &c, int b, int dir, int enc, const v3t<D7> &S0,
+                                      const v3t<D7> &P, unsigned enable, int wall, AdjRec &R, int *jpow,
+                                      D7 ei[2]) {
+    v3t<D7> cc;
+    D7 a;
+    bool sphere;
+    adj_body(c, b, cc, a, sphere);
+    v3t<D7> S = S0;
+    if (wall >= 0) {
+        v3t<D7> n;
+        D7 d;
+        face_plane<D7>(c, wall, &n, &d);
+        S = mirror_pt(S0, n, d);
+    }
+    Frame<D7> F;
+    if (sphere) sphere_frame(S, P, cc, a, F, D7(0.0));
+    else cyl_frame(S, P, cc.x, cc.y, a, F, D7(0.0));
+    const D7 TWO_PI(double(6.283185307179586476925286766559));
+    D7 dpsi = (dir == 0) ? (F.gam - F.bs - F.bp) : (TWO_PI - F.gam - F.bs - F.bp);
+    dpsi = dpsi + TWO_PI * D7(double(enc));
+    D7 psi1 = (dir == 0) ? F.bs : -F.bs;
+    D7 psi2 = (dir == 0) ? F.gam - F.bp : F.gam + F.bp;
+    D7 s1, c1, s2, c2;
+    SinCos(psi1, &s1, &c1);
+    SinCos(psi2, &s2, &c2);
+    const v3t<D7> n1 = F.u * c1 + F.v * s1, n2 = F.u * c2 + F.v * s2;
+    v3t<D7> Q1, Q2;
+    D7 sp, sq, t, rho;
+    *jpow = 0;
+    if (sphere) {
+        Q1 = cc + n1 * a;
+        Q2 = cc + n2 * a;
+        sp = F.sps;
+        sq = F.sqp;
+        t = a * dpsi;
+        rho = a;
+        *jpow = (dir == 1);
+        D7 sg, cg;
+        SinCos(F.gam, &sg, &cg);
+        const D7 dperp = F.dp * sg;
+        if (!(dperp > D7(0.0))) return 0;
+        D7 sb, cb;
+        SinCos(F.bs, &sb, &cb);
+        R.A = Sqrt(a * sb / dperp) / Sqrt(sq) / sp;
+        if (enc & 1) R.A = -R.A;                 // the (-1) of an odd number of extra turns
+    } else {
+        const D7 ds_ = F.sps, dp_ = F.sqp;
+        const D7 dz = P.z - S.z;
+        const D7 H = ds_ + a * dpsi + dp_;
+        const D7 ell = Sqrt(H * H + dz * dz);
+        const D7 sin0 = H / ell;
+        const D7 z1 = S.z + dz * ds_ / H, z2 = S.z + dz * (ds_ + a * dpsi) / H;
+        Q1 = mk3<D7>(cc.x + a * n1.x, cc.y + a * n1.y, z1);
+        Q2 = mk3<D7>(cc.x + a * n2.x, cc.y + a * n2.y, z2);
+        sp = ds_ / sin0;
+        t = a * dpsi / sin0;
+        sq = dp_ / sin0;
+        rho = a / (sin0 * sin0);
+        R.A = D7(1.0) / Sqrt(sp * sq * (sp + t + sq));
+    }
+    // the field's factors (as field_creep and field_wcreep)
+    const v3t<D7> t1 = unit3(Q1 - S), t2 = unit3(P - Q2);
+    const v3t<D7> b1 = cross3(t1, n1);
+    int parts = 1;
+    if (wall >= 0) {
+        D7 dQ;
+        const v3t<D7> Qw = wall_point(c, wall, S, Q1, &dQ);
+        const v3t<D7> si = unit3(Qw - S0), e0 = src_pol(c, si);
+        cpx<D7> E[3] = {mkc<D7>(e0.x, D7(0.0)), mkc<D7>(e0.y, D7(0.0)), mkc<D7>(e0.z, D7(0.0))};
+        reflect_face(c, wall, E, si, t1);
+        const cpx<D7> Es = c3dot(E, b1), Eh = c3dot(E, n1);
+        R.Es = Es.re;
+        R.Eh = Eh.re;
+        if (dielectric(c, wall)) {
+            ei[0] = Es.im;
+            ei[1] = Eh.im;
+            parts = 2;
+        }
+    } else {
+        const v3t<D7> e0 = src_pol(c, t1);
+        R.Es = dot3(e0, b1);
+        R.Eh = dot3(e0, n1);
+    }
+    if (!(enable & RT_EN_CREEP_SOFT)) { R.Es = D7(0.0); ei[0] = D7(0.0); }
+    if (!(enable & RT_EN_CREEP_HARD)) { R.Eh = D7(0.0); ei[1] = D7(0.0); }
+    R.e1 = cross3(t2, n2);
+    R.e2 = n2;
+    R.Lp = sp * sq / (sp + sq);
+    R.rcb = Cbrt(rho);
+    R.x = t / rho;
+    R.L = sp + t + sq;
+    return parts;
+}
+
+// planar paths of order 0 to 3 (faces fs):
+// the images by mirroring the dual-number source, the points backwards from P
+__device__ __noinline__ void adj_planar(const Ctx &c, int order, const int fs[3], const v3t<D3> &S,
+                                        const v3t<D3> &P, const FreqC &fq, AccAdj &acc) {
+    v3t<D3> X[3], Q[3];
+    D3 L;
+    bool cx = false;
+    v3t<D3> I = S;
+#pragma unroll 1
+    for (int m = 0; m < order; ++m) {
+        v3t<D3> n; D3 d;
+        face_plane<D3>(c, fs[m], &n, &d);
+        I = mirror_pt(I, n, d);
+        X[m] = I;
+        cx = cx || dielectric(c, fs[m]);
+    }
+    v3t<D3> Y = P;
+#pragma unroll 1
+    for (int m = order - 1; m >= 0; --m) {
+        v3t<D3> n; D3 d;
+        face_plane<D3>(c, fs[m], &n, &d);
+        const D3 di = dot3(n, X[m]) - d, dy = dot3(n, Y) - d;
+        Q[m] = X[m] + (Y - X[m]) * (di / (di - dy));
+        const D3 l = norm3(Y - Q[m]);
+        L = m == order - 1 ? l : L + l;
+        Y = Q[m];
+    }
+    const v3t<D3> d0 = Y - S;
+    const D3 l0 = norm3(d0);
+    L = order == 0 ? l0 : L + l0;
+    v3t<D3> s = d0 * (D3(1.0) / l0);
+    const v3t<D3> e0 = src_pol(c, s);
+    cpx<D3> E[3] = {mkc<D3>(e0.x, D3(0.0)), mkc<D3>(e0.y, D3(0.0)), mkc<D3>(e0.z, D3(0.0))};
+    if (cx) {
+#pragma unroll 1
+        for (int m = 0; m < order; ++m) {
+            const v3t<D3> so = unit3((m + 1 < order ? Q[m + 1] : P) - Q[m]);
+            reflect_face(c, fs[m], E, s, so);
+            s = so;
+        }
+        adj_ray<true>(fq, E, L, acc);
+    } else {
+        v3t<D3> e = e0;
+#pragma unroll 1
+        for (int m = 0; m < order; ++m) {
+            v3t<D3> n; D3 d;
+            face_plane<D3>(c, fs[m], &n, &d);
+            e = pec_mirror(e, n);
+        }
+        E[0].re = e.x; E[1].re = e.y; E[2].re = e.z;
+        adj_ray<false>(fq, E, L, acc);
+    }
+}
+
+// ---- FP32 duals, forward through the field (eight tangents): a gradient is
+// rounded in FP32 path by path, so its digits past the seventh are those of
+// this order of operations; FP32 lanes are not what bounds the kernel.
 template <> __device__ __forceinline__ void face_plane<F8>(const Ctx &c, int f, v3t<F8> *n, F8 *d) {
     float4 q = c.face32[f]; *n = mk3<F8>(q.x, q.y, q.z); *d = F8(q.w);
 }
 
-// Fock--Pekeris functions of a dual xi: the residue series term by term
-// above XI_HI, else the table's cubic Hermite interpolant and its slope
-__device__ void pekeris(const Ctx &c, const D8 &xi, cpx<D8> &ps, cpx<D8> &ph, bool regular) {
-    const double cc = (0.5 / sqrt(M_PI)) * cos(M_PI / 4.0);
-    const D8 ci = D8(cc) / xi;
-    if (xi.v > XI_HI) {
-        cpx<D8> ss = mkc<D8>(0.0, 0.0), sh = mkc<D8>(0.0, 0.0);
-        for (int n = 0; n < FOCK_NRES; ++n) {
-            dq4 rs = c.res64[2 * n], rh = c.res64[2 * n + 1];
-            D8 sn, cs;
-            SinCos(xi * D8(rs.y), &sn, &cs);
-            D8 e = Exp(-(xi * D8(rs.x))) * D8(rs.z);
-            ss = ss + mkc<D8>(e * cs, -(e * sn));
-            SinCos(xi * D8(rh.y), &sn, &cs);
-            e = Exp(-(xi * D8(rh.x))) * D8(rh.z);
-            sh = sh + mkc<D8>(e * cs, -(e * sn));
-        }
-        const cpx<D8> pre = mkc<D8>(-cos(M_PI / 12.0) * (0.5 / sqrt(M_PI)), sin(M_PI / 12.0) * (0.5 / sqrt(M_PI)));
-        ps = pre * ss;
-        ph = pre * sh;
-        if (regular) { ps = ps + mkc<D8>(ci, -ci); ph = ph + mkc<D8>(ci, -ci); }
-        return;
-    }
-    // cubic Hermite interpolant of G and its derivative in xi
-    const double u = (xi.v - XI_LO) / XI_STEP;
-    const int j = min(max((int)u, 0), FOCK_N - 2);
-    const double t = u - j, t2 = t * t, omt = 1.0 - t;
-    const double h00 = (1 + 2 * t) * omt * omt, h10 = t * omt * omt * XI_STEP, h01 = t2 * (3 - 2 * t),
-                 h11 = t2 * (t - 1) * XI_STEP;
-    // d/dxi = (d/dt) / XI_STEP
-    const double d00 = (6 * t2 - 6 * t) / XI_STEP, d10 = 1 - 4 * t + 3 * t2, d01 = (6 * t - 6 * t2) / XI_STEP,
-                 d11 = 3 * t2 - 2 * t;
-    cpx<D8> G[2];
-    for (int k = 0; k < 2; ++k) {
-        double2 g0 = c.fock64[(j * 2 + k) * 2], q0 = c.fock64[(j * 2 + k) * 2 + 1];
-        double2 g1 = c.fock64[((j + 1) * 2 + k) * 2], q1 = c.fock64[((j + 1) * 2 + k) * 2 + 1];
-        const double gr = h00 * g0.x + h10 * q0.x + h01 * g1.x + h11 * q1.x;
-        const double gi = h00 * g0.y + h10 * q0.y + h01 * g1.y + h11 * q1.y;
-        const double dr = d00 * g0.x + d10 * q0.x + d01 * g1.x + d11 * q1.x;
-        const double di = d00 * g0.y + d10 * q0.y + d01 * g1.y + d11 * q1.y;
-        G[k] = mkc<D8>(dchain<double>(gr, dr, xi), dchain<double>(gi, di, xi));
-    }
-    const cpx<D8> rot = cexpi(xi * xi * xi / D8(12.0));
-    ps = G[0] * rot;
-    ph = G[1] * rot;
-    if (!regular) { ps = ps - mkc<D8>(ci, -ci); ph = ph - mkc<D8>(ci, -ci); }
-}
 __device__ void pekeris(const Ctx &c, const F8 &xi, cpx<F8> &ps, cpx<F8> &ph, bool regular) {
     const F8 ci = F8(0.19947114f) / xi;               // c/xi = (ci, -ci)
     if (xi.v > (float)XI_HI) {
@@ -3938,59 +4408,17 @@ __device__ void pekeris(const Ctx &c, const F8 &xi, cpx<F8> &ps, cpx<F8> &ph, bo
     if (!regular) { ps = ps - mkc<F8>(ci, -ci); ph = ph - mkc<F8>(ci, -ci); }
 }
 
-// w(z) of a dual z, with w'(z) = -2 z w + 2j / sqrt(pi)
-template <typename S>
-__device__ __forceinline__ cpx<DualT<S>> faddeeva_dual(const cpx<DualT<S>> &zd, cpx<S> w) {
-    const cpx<S> z = mkc(zd.re.v, zd.im.v);
-    const cpx<S> wp = z * w * S(-2) + mkc(S(0), S(1.1283791670955126));
-    cpx<DualT<S>> r;
-    r.re.v = w.re; r.im.v = w.im;
-#pragma unroll
-    for (int k = 0; k < ND; ++k) {
-        r.re.d[k] = wp.re * zd.re.d[k] - wp.im * zd.im.d[k];
-        r.im.d[k] = wp.re * zd.im.d[k] + wp.im * zd.re.d[k];
-    }
-    return r;
-}
-__device__ cpx<D8> faddeeva_t(const Ctx &c, const cpx<D8> &zd) {
-    cpx<double> z = mkc(zd.re.v, zd.im.v);
-    const double L = c.weid_L;
-    cpx<double> lm = mkc(L + z.im, -z.re), lp = mkc(L - z.im, z.re);
-    cpx<double> Z = cdiv(lp, lm);
-    cpx<double> p = mkc(c.weid64[WEIDEMAN_N - 1], 0.0);
-    for (int n = WEIDEMAN_N - 2; n >= 0; --n) p = p * Z + mkc(c.weid64[n], 0.0);
-    cpx<double> w = cdiv(p * 2.0, lm * lm) + cdiv(mkc(0.56418958354775628, 0.0), lm);
-    return faddeeva_dual<double>(zd, w);
-}
 __device__ cpx<F8> faddeeva_t(const Ctx &c, const cpx<F8> &zd) {
-    return faddeeva_dual<float>(zd, faddeeva<float>(c, mkc(zd.re.v, zd.im.v)));
+    return faddeeva_dual<float, 8>(zd, faddeeva<float>(c, mkc(zd.re.v, zd.im.v)));
 }
-
 // wavenumber, (k/2)^{1/3} with the frequency as slot DS_F
-__device__ __forceinline__ D8 kof(const FreqC &fq, int f, const D8 &) {
-    D8 k(fq.kd[f]);
-    k.d[DS_F] = 2.0 * M_PI / 299792458.0;
-    return k;
-}
 __device__ __forceinline__ F8 kof(const FreqC &fq, int f, const F8 &) {
     F8 k(fq.k[f]);
     k.d[DS_F] = (float)(2.0 * M_PI / 299792458.0);
     return k;
 }
-__device__ __forceinline__ D8 khof(const FreqC &fq, int f, const D8 &x) { return Cbrt(kof(fq, f, x) * D8(0.5)); }
 __device__ __forceinline__ F8 khof(const FreqC &fq, int f, const F8 &x) { return Cbrt(kof(fq, f, x) * F8(0.5f)); }
 
-// the path phasor e^{-j k L}; FP64 duals: from the dual length itself
-__device__ __forceinline__ cpx<D8> phasor(const FreqC &fq, int f, const D8 &L) {
-    D8 fc(fq.fc[f]);
-    fc.d[DS_F] = 1.0 / 299792458.0;
-    D8 cyc = L * fc;
-    cyc.v -= floor(cyc.v);                      // the integer cycles (no derivative)
-    D8 s, co;
-    SinCosPi(cyc * D8(2.0), &s, &co);
-    return mkc<D8>(co, -s);
-}
-__device__ __forceinline__ D8 len_val(const D8 &L) { return L; }
 // FP32 duals: the length's tangents from the dual, its value as double-float
 // (the phase as the FP32 fraction of L / lambda, integer cycles dropped)
 struct LenF8 {
@@ -4006,7 +4434,7 @@ __device__ __forceinline__ cpx<F8> phasor(const FreqC &fq, int f, const LenF8 &L
     F8 c;
     c.v = fr;
 #pragma unroll
-    for (int k = 0; k < ND; ++k) c.d[k] = L.l.d[k] * ilf;
+    for (int k = 0; k < 8; ++k) c.d[k] = L.l.d[k] * ilf;
     c.d[DS_F] += (L.h.hi + L.h.lo) * (float)(1.0 / 299792458.0);    // d(L f / c)/df
     F8 s, co;
     SinCosPi(c * F8(2.0f), &s, &co);
@@ -4014,92 +4442,28 @@ __device__ __forceinline__ cpx<F8> phasor(const FreqC &fq, int f, const LenF8 &L
 }
 __device__ __forceinline__ F8 len_val(const LenF8 &L) { return L.l; }
 
-template <typename DT> struct AdjLen;
-template <> struct AdjLen<D8> { typedef D8 type; };
-template <> struct AdjLen<F8> { typedef LenF8 type; };
-__device__ __forceinline__ D8 mk_len(const D8 &l, dfl) { return l; }
-__device__ __forceinline__ LenF8 mk_len(const F8 &l, dfl h) { return LenF8{l, h}; }
 
 // contracts each path field's tangents with dLoss/dE of its receiver
-struct AccAdj {
-    const float *gE;        // [n_f][3][n_rx][2]
-    int n_rx, r, f0;
-    double g[ND - 1];       // body and transmitter slots
-    double gf[NFC];         // frequency slot, per frequency of the chunk
-};
-template <typename S>
-__device__ __forceinline__ void acc_put(AccAdj &a, int f, const cpx<DualT<S>> &x, const cpx<DualT<S>> &y,
-                                        const cpx<DualT<S>> &z) {
-    const cpx<DualT<S>> *e[3] = {&x, &y, &z};
+__device__ __forceinline__ void acc_put(AccAdj &a, int f, const cpx<F8> &x, const cpx<F8> &y,
+                                        const cpx<F8> &z) {
+    const cpx<F8> *e[3] = {&x, &y, &z};
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
         const size_t idx = ((size_t)(a.f0 + f) * 3 + q) * a.n_rx + a.r;
-        const S gr = a.gE[2 * idx], gi = a.gE[2 * idx + 1];
+        const float gr = a.gE[2 * idx], gi = a.gE[2 * idx + 1];
 #pragma unroll
-        for (int k = 0; k < ND - 1; ++k) a.g[k] += (double)(gr * e[q]->re.d[k] + gi * e[q]->im.d[k]);
+        for (int k = 0; k < 7; ++k) a.g[k] += (double)(gr * e[q]->re.d[k] + gi * e[q]->im.d[k]);
         a.gf[f] += (double)(gr * e[q]->re.d[DS_F] + gi * e[q]->im.d[DS_F]);
     }
 }
 
-// body b's centre and radius as parameters (slots 0-3)
-template <typename S>
-__device__ __forceinline__ void adj_body(const Ctx &c, int b, v3t<DualT<S>> &cc, DualT<S> &a, bool &sphere) {
+__device__ __forceinline__ void adj_body8(const Ctx &c, int b, v3t<F8> &cc, F8 &a, bool &sphere) {
     float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
-    cc = mk3<DualT<S>>(dvar_t<S>(q0.x, DS_CX), dvar_t<S>(q0.y, DS_CY), dvar_t<S>(q0.z, DS_CZ));
-    a = dvar_t<S>(q0.w, DS_A);
+    cc = mk3<F8>(dvar_t<float, 8>(q0.x, DS_CX), dvar_t<float, 8>(q0.y, DS_CY), dvar_t<float, 8>(q0.z, DS_CZ));
+    a = dvar_t<float, 8>(q0.w, DS_A);
     sphere = q1.y == 0.0f;
 }
-
-// the reflection point's angle as a dual: the root in the dual's precision
-// (FP64: refined to the bisection root; FP32: the forward FP32 root, refined
-// in double-float or FP64 near grazing), then one Newton step on dL/dpsi = 0
-// in dual arithmetic (the implicit-function derivative)
-__device__ __forceinline__ void refl_root_val(double a, double ds, double pu, double pv, double gam, double *c0,
-                                              double *s0) {
-    dx cc, ss;
-    refl_root(dx(a), dx(ds), dx(pu), dx(pv), dx(gam), &cc, &ss);
-    *c0 = cc.v; *s0 = ss.v;
-}
-__device__ __forceinline__ void refl_root_val(float a, float ds, float pu, float pv, float gam, float *c0, float *s0) {
-    float err = 0.0f, sn, cs;
-    refl_n32(a, ds, pu, pv, gam, &cs, &sn, &err);
-    const float c2 = (ds * cs - a) / sqrtf((a * cs - ds) * (a * cs - ds) + a * a * sn * sn);
-    if (err > 1e-5f * fmaxf(c2, 0.0f)) {
-        if (!refl_polish_df(a, ds, pu, pv, cs, sn, &cs, &sn)) refl_polish(a, ds, pu, pv, gam, cs, sn, &cs, &sn);
-    }
-    *c0 = cs; *s0 = sn;
-}
-template <typename S>
-__device__ __noinline__ void adj_refl_root(const DualT<S> &a, const DualT<S> &ds, const DualT<S> &pu,
-                                           const DualT<S> &pv, const DualT<S> &gam, DualT<S> *cs, DualT<S> *sn) {
-    typedef DualT<S> DT;
-    S c0, s0;
-    refl_root_val(a.v, ds.v, pu.v, pv.v, gam.v, &c0, &s0);
-    const DT psi(atan2(s0, c0));
-    DT s, c;
-    SinCos(psi, &s, &c);
-    const DT qx = a * c, qy = a * s;
-    const DT lS = Sqrt((qx - ds) * (qx - ds) + qy * qy);
-    const DT lP = Sqrt((qx - pu) * (qx - pu) + (qy - pv) * (qy - pv));
-    const DT gS = a * ds * s / lS, gP = a * (pu * s - pv * c) / lP;
-    DT h;
-    if constexpr (sizeof(S) == 8) {
-        h = (ds * qx - gS * gS) / lS + (pu * qx + pv * qy - gP * gP) / lP;
-    } else {
-        // d2L/dpsi2 in the product form a sum_X (u - a)(|X|^2 - a u) / |Q - X|^3,
-        // u = X.n: the difference form above cancels near grazing incidence
-        const DT uS = ds * c, uP = pu * c + pv * s;
-        h = a * ((uS - a) * (ds * ds - a * uS) / (lS * lS * lS) +
-                 (uP - a) * (pu * pu + pv * pv - a * uP) / (lP * lP * lP));
-    }
-    SinCos(psi - (gS + gP) / h, sn, cs);
-}
-
-// double-float lengths of the FP32 path pieces (no use for FP64 duals)
 __device__ __forceinline__ v3t<float> vals(const v3t<F8> &a) { return mk3(a.x.v, a.y.v, a.z.v); }
-__device__ __forceinline__ v3t<float> vals(const v3t<D8> &a) {
-    return mk3((float)a.x.v, (float)a.y.v, (float)a.z.v);
-}
 // sqrt(|X - c|^2 - a^2) from the exact squares (horiz: horizontal distance)
 __device__ __forceinline__ dfl df_tangent_len(v3t<float> X, float4 q0, bool horiz) {
     dfl q2 = df_add(df_sq_diff(X.x, q0.x), df_sq_diff(X.y, q0.y));
@@ -4111,84 +4475,23 @@ __device__ __forceinline__ dfl df_tangent_len(v3t<float> X, float4 q0, bool hori
     return df_sqrt(q2);
 }
 
-// reflection off body b (the forward construction, without decisions)
-template <typename DT>
-__device__ __noinline__ void adj_rb(const Ctx &c, int b, v3t<DT> S, v3t<DT> P, const FreqC &fq, AccAdj &acc) {
-    typedef decltype(DT().v) SC;
-    v3t<DT> cc;
-    DT a;
-    bool sphere;
-    adj_body<SC>(c, b, cc, a, sphere);
-    Frame<DT> F;
-    if (sphere) sphere_frame(S, P, cc, a, F, DT(0.0f));
-    else cyl_frame(S, P, cc.x, cc.y, a, F, DT(0.0f));
-    DT cs, sn;
-    adj_refl_root<SC>(a, F.ds, F.pu, F.pv, F.gam, &cs, &sn);
-    v3t<DT> n = F.u * cs + F.v * sn;
-    v3t<DT> Q;
-    if (sphere) {
-        Q = cc + n * a;
-    } else {
-        DT qx = a * cs, qy = a * sn;
-        DT l1 = Sqrt((qx - F.ds) * (qx - F.ds) + qy * qy);
-        DT l2 = Sqrt((qx - F.pu) * (qx - F.pu) + (qy - F.pv) * (qy - F.pv));
-        DT zq = S.z + (P.z - S.z) * l1 / (l1 + l2);
-        Q = mk3<DT>(cc.x + a * n.x, cc.y + a * n.y, zq);
-    }
-    Geo<DT> g;
-    v3t<DT> shi = unit3(Q - S);
-    DT cth = -dot3(shi, n);
-    g.dr = P - Q;
-    g.Q1 = Q;
-    g.n1 = n;
-    if (sphere) {
-        g.inv_f1 = DT(2.0f) / (a * cth);
-        g.inv_f2 = DT(2.0f) * cth / a;
-        g.rho_g = a;
-    } else {
-        g.inv_f1 = DT(2.0f) * (DT(1.0f) - shi.z * shi.z) / (a * cth);
-        g.inv_f2 = DT(0.0f);
-        DT sphi = -(shi.x * n.y) + shi.y * n.x;
-        g.rho_g = (sphi == DT(0.0f)) ? DT(INFINITY) : a * (DT(1.0f) - cth * cth) / (sphi * sphi);
-    }
-    dfl Lh = {0.0f, 0.0f};
-    if constexpr (sizeof(SC) == 4) {
-        // the forward's length: both legs to the FP32 surface point c + a n, in double-float
-        const float4 q0 = c.body[2 * b];
-        dfl ws[3], wp[3];
-        df_to_surface(vals(S), q0, q0.w, vals(n), !sphere, ws);
-        df_to_surface(vals(P), q0, q0.w, vals(n), !sphere, wp);
-        const dfl si = df_norm3(ws), sr = df_norm3(wp);
-        if (sphere) {
-            Lh = df_add(si, sr);
-        } else {
-            const dfl H = df_add(si, sr);
-            Lh = df_sqrt(df_add(df_mul(H, H), df_sq_diff(P.z.v, S.z.v)));
-        }
-    }
-    field_body_refl<DT, typename AdjLen<DT>::type, false, AccAdj>(c, acc, fq, S, P, g,
-                                                                  mk_len(norm3(Q - S) + norm3(P - Q), Lh));
-}
-
 // creeping ray round body b, dir 0 short way, 1 long way, with enc extra
 // turns; wall >= 0: fed by the reflection at face wall (the creeping ray of
 // the source's image there); false: no finite field
-template <typename DT>
-__device__ __noinline__ bool adj_creep(const Ctx &c, int b, int dir, int enc, v3t<DT> S0, v3t<DT> P, const FreqC &fq,
+__device__ __noinline__ bool adj_creep8(const Ctx &c, int b, int dir, int enc, v3t<F8> S0, v3t<F8> P, const FreqC &fq,
                                        unsigned enable, AccAdj &acc, int wall = -1) {
-    typedef decltype(DT().v) SC;
-    v3t<DT> cc;
-    DT a;
+    v3t<F8> cc;
+    F8 a;
     bool sphere;
-    adj_body<SC>(c, b, cc, a, sphere);
-    v3t<DT> S = S0;
+    adj_body8(c, b, cc, a, sphere);
+    v3t<F8> S = S0;
     v3t<float> Sval = vals(S0);            // (FP32 duals: the source point of the tangent length)
     if (wall >= 0) {
-        v3t<DT> n;
-        DT d;
-        face_plane<DT>(c, wall, &n, &d);
+        v3t<F8> n;
+        F8 d;
+        face_plane<F8>(c, wall, &n, &d);
         S = mirror_pt(S0, n, d);
-        if constexpr (sizeof(SC) == 4) {
+        {
             // the image's value from the FP64 plane, as the forward's per-transmitter table has it
             const dq4 q = c.face64[wall];
             const double X[3] = {c.S.x, c.S.y, c.S.z};
@@ -4197,16 +4500,16 @@ __device__ __noinline__ bool adj_creep(const Ctx &c, int b, int dir, int enc, v3
                        (float)(X[2] - q.z * (2.0 * dist)));
         }
     }
-    Frame<DT> F;
-    if (sphere) sphere_frame(S, P, cc, a, F, DT(0.0f));
-    else cyl_frame(S, P, cc.x, cc.y, a, F, DT(0.0f));
-    const DT TWO_PI(SC(6.283185307179586476925286766559));
-    DT dpsi = (dir == 0) ? (F.gam - F.bs - F.bp) : (TWO_PI - F.gam - F.bs - F.bp);
-    dpsi = dpsi + TWO_PI * DT(SC(enc));
-    Geo<DT> g;
-    DT psi1 = (dir == 0) ? F.bs : -F.bs;
-    DT psi2 = (dir == 0) ? F.gam - F.bp : F.gam + F.bp;
-    DT s1, c1, s2, c2;
+    Frame<F8> F;
+    if (sphere) sphere_frame(S, P, cc, a, F, F8(0.0f));
+    else cyl_frame(S, P, cc.x, cc.y, a, F, F8(0.0f));
+    const F8 TWO_PI(float(6.283185307179586476925286766559));
+    F8 dpsi = (dir == 0) ? (F.gam - F.bs - F.bp) : (TWO_PI - F.gam - F.bs - F.bp);
+    dpsi = dpsi + TWO_PI * F8(float(enc));
+    Geo<F8> g;
+    F8 psi1 = (dir == 0) ? F.bs : -F.bs;
+    F8 psi2 = (dir == 0) ? F.gam - F.bp : F.gam + F.bp;
+    F8 s1, c1, s2, c2;
     SinCos(psi1, &s1, &c1);
     SinCos(psi2, &s2, &c2);
     g.n1 = F.u * c1 + F.v * s1;
@@ -4220,46 +4523,45 @@ __device__ __noinline__ bool adj_creep(const Ctx &c, int b, int dir, int enc, v3
         g.t = a * dpsi;
         g.rho_g = a;
         g.caus = (dir == 1);
-        DT sg, cg;
+        F8 sg, cg;
         SinCos(F.gam, &sg, &cg);
         g.dperp = F.dp * sg;
-        if (!(g.dperp > DT(0.0f))) return false;
-        DT sb, cb;
+        if (!(g.dperp > F8(0.0f))) return false;
+        F8 sb, cb;
         SinCos(F.bs, &sb, &cb);
         g.amp = Sqrt(a * sb / g.dperp) / Sqrt(g.sq) / g.sp;
         if (enc & 1) g.amp = -g.amp;             // the (-1) of an odd number of extra turns
-        if constexpr (sizeof(SC) == 4) {
+        {
             const float4 q0 = c.body[2 * b];
             Lh = df_addf(df_add(df_tangent_len(Sval, q0, false), df_tangent_len(vals(P), q0, false)), g.t.v);
         }
     } else {
-        DT ds_ = F.sps, dp_ = F.sqp;
-        DT dz = P.z - S.z;
-        DT H = ds_ + a * dpsi + dp_;
-        DT ell = Sqrt(H * H + dz * dz);
-        DT sin0 = H / ell;
-        DT z1 = S.z + dz * ds_ / H, z2 = S.z + dz * (ds_ + a * dpsi) / H;
-        g.Q1 = mk3<DT>(cc.x + a * g.n1.x, cc.y + a * g.n1.y, z1);
-        g.Q2 = mk3<DT>(cc.x + a * g.n2.x, cc.y + a * g.n2.y, z2);
+        F8 ds_ = F.sps, dp_ = F.sqp;
+        F8 dz = P.z - S.z;
+        F8 H = ds_ + a * dpsi + dp_;
+        F8 ell = Sqrt(H * H + dz * dz);
+        F8 sin0 = H / ell;
+        F8 z1 = S.z + dz * ds_ / H, z2 = S.z + dz * (ds_ + a * dpsi) / H;
+        g.Q1 = mk3<F8>(cc.x + a * g.n1.x, cc.y + a * g.n1.y, z1);
+        g.Q2 = mk3<F8>(cc.x + a * g.n2.x, cc.y + a * g.n2.y, z2);
         g.sp = ds_ / sin0;
         g.t = a * dpsi / sin0;
         g.sq = dp_ / sin0;
         g.rho_g = a / (sin0 * sin0);
         g.caus = 0;
-        g.dperp = DT(0.0f);
-        g.amp = DT(1.0f) / Sqrt(g.sp * g.sq * (g.sp + g.t + g.sq));
-        if constexpr (sizeof(SC) == 4) {
+        g.dperp = F8(0.0f);
+        g.amp = F8(1.0f) / Sqrt(g.sp * g.sq * (g.sp + g.t + g.sq));
+        {
             const float4 q0 = c.body[2 * b];
             const dfl Hh = df_addf(df_add(df_tangent_len(Sval, q0, true), df_tangent_len(vals(P), q0, true)),
                                    (a * dpsi).v);
             Lh = df_sqrt(df_add(df_mul(Hh, Hh), df_sq_diff(P.z.v, Sval.z)));
         }
     }
-    typedef typename AdjLen<DT>::type LT;
     if (wall >= 0)
-        field_wcreep<DT, LT, false, AccAdj>(c, acc, fq, wall, S0, S, P, g, mk_len(g.sp + g.t + g.sq, Lh), enable);
+        field_wcreep<F8, LenF8, false, AccAdj>(c, acc, fq, wall, S0, S, P, g, LenF8{g.sp + g.t + g.sq, Lh}, enable);
     else
-        field_creep<DT, LT, false, AccAdj>(c, acc, fq, S, P, g, mk_len(g.sp + g.t + g.sq, Lh), enable);
+        field_creep<F8, LenF8, false, AccAdj>(c, acc, fq, S, P, g, LenF8{g.sp + g.t + g.sq, Lh}, enable);
     return true;
 }
 
@@ -4286,85 +4588,80 @@ __device__ __forceinline__ dfl planar_len(const Ctx &c, int order, int i, int j,
 }
 
 // direct ray and planar image paths (faces i, j; -1: none)
-template <typename DT>
-__device__ __noinline__ void adj_planar(const Ctx &c, int order, int i, int j, v3t<DT> S, v3t<DT> P,
+__device__ __noinline__ void adj_planar8(const Ctx &c, int order, int i, int j, v3t<F8> S, v3t<F8> P,
                                         const FreqC &fq, AccAdj &acc) {
-    typedef decltype(DT().v) SC;
-    dfl Lh = {0.0f, 0.0f};
-    if constexpr (sizeof(SC) == 4) Lh = planar_len(c, order, i, j, vals(P));
+    const dfl Lh = planar_len(c, order, i, j, vals(P));
     if (order == 0) {
-        v3t<DT> d = P - S;
-        DT L = norm3(d);
-        add_ray(acc, fq, src_pol(c, d * (DT(1.0f) / L)), DT(1.0f) / L, mk_len(L, Lh));
+        v3t<F8> d = P - S;
+        F8 L = norm3(d);
+        add_ray(acc, fq, src_pol(c, d * (F8(1.0f) / L)), F8(1.0f) / L, LenF8{L, Lh});
         return;
     }
-    v3t<DT> ni, nj;
-    DT di, dj;
-    face_plane<DT>(c, i, &ni, &di);
-    v3t<DT> S1 = mirror_pt(S, ni, di);
+    v3t<F8> ni, nj;
+    F8 di, dj;
+    face_plane<F8>(c, i, &ni, &di);
+    v3t<F8> S1 = mirror_pt(S, ni, di);
     if (order == 1) {
-        DT d1 = dot3(ni, S1) - di, dP = dot3(ni, P) - di;
-        v3t<DT> Q = S1 + (P - S1) * (d1 / (d1 - dP));
-        DT L = norm3(Q - S) + norm3(P - Q);
+        F8 d1 = dot3(ni, S1) - di, dP = dot3(ni, P) - di;
+        v3t<F8> Q = S1 + (P - S1) * (d1 / (d1 - dP));
+        F8 L = norm3(Q - S) + norm3(P - Q);
         if (dielectric(c, i)) {
-            const v3t<DT> s1 = unit3(Q - S), e0 = src_pol(c, s1);
-            cpx<DT> E[3] = {mkc<DT>(e0.x, DT(0.0f)), mkc<DT>(e0.y, DT(0.0f)), mkc<DT>(e0.z, DT(0.0f))};
+            const v3t<F8> s1 = unit3(Q - S), e0 = src_pol(c, s1);
+            cpx<F8> E[3] = {mkc<F8>(e0.x, F8(0.0f)), mkc<F8>(e0.y, F8(0.0f)), mkc<F8>(e0.z, F8(0.0f))};
             reflect_face(c, i, E, s1, unit3(P - Q));
-            add_ray_cx(acc, fq, E, DT(1.0f) / L, mk_len(L, Lh));
+            add_ray_cx(acc, fq, E, F8(1.0f) / L, LenF8{L, Lh});
         } else {
-            add_ray(acc, fq, pec_mirror(src_pol(c, unit3(Q - S)), ni), DT(1.0f) / L, mk_len(L, Lh));
+            add_ray(acc, fq, pec_mirror(src_pol(c, unit3(Q - S)), ni), F8(1.0f) / L, LenF8{L, Lh});
         }
         return;
     }
-    face_plane<DT>(c, j, &nj, &dj);
-    v3t<DT> S2 = mirror_pt(S1, nj, dj);
-    DT d2 = dot3(nj, S2) - dj, dP = dot3(nj, P) - dj;
-    v3t<DT> Q2 = S2 + (P - S2) * (d2 / (d2 - dP));
-    DT e1 = dot3(ni, S1) - di, eq = dot3(ni, Q2) - di;
-    v3t<DT> Q1 = S1 + (Q2 - S1) * (e1 / (e1 - eq));
-    DT L = norm3(Q1 - S) + norm3(Q2 - Q1) + norm3(P - Q2);
+    face_plane<F8>(c, j, &nj, &dj);
+    v3t<F8> S2 = mirror_pt(S1, nj, dj);
+    F8 d2 = dot3(nj, S2) - dj, dP = dot3(nj, P) - dj;
+    v3t<F8> Q2 = S2 + (P - S2) * (d2 / (d2 - dP));
+    F8 e1 = dot3(ni, S1) - di, eq = dot3(ni, Q2) - di;
+    v3t<F8> Q1 = S1 + (Q2 - S1) * (e1 / (e1 - eq));
+    F8 L = norm3(Q1 - S) + norm3(Q2 - Q1) + norm3(P - Q2);
     if (dielectric(c, i) || dielectric(c, j)) {
-        const v3t<DT> s1 = unit3(Q1 - S), s2 = unit3(Q2 - Q1), e0 = src_pol(c, s1);
-        cpx<DT> E[3] = {mkc<DT>(e0.x, DT(0.0f)), mkc<DT>(e0.y, DT(0.0f)), mkc<DT>(e0.z, DT(0.0f))};
+        const v3t<F8> s1 = unit3(Q1 - S), s2 = unit3(Q2 - Q1), e0 = src_pol(c, s1);
+        cpx<F8> E[3] = {mkc<F8>(e0.x, F8(0.0f)), mkc<F8>(e0.y, F8(0.0f)), mkc<F8>(e0.z, F8(0.0f))};
         reflect_face(c, i, E, s1, s2);
         reflect_face(c, j, E, s2, unit3(P - Q2));
-        add_ray_cx(acc, fq, E, DT(1.0f) / L, mk_len(L, Lh));
+        add_ray_cx(acc, fq, E, F8(1.0f) / L, LenF8{L, Lh});
     } else {
-        add_ray(acc, fq, pec_mirror(pec_mirror(src_pol(c, unit3(Q1 - S)), ni), nj), DT(1.0f) / L, mk_len(L, Lh));
+        add_ray(acc, fq, pec_mirror(pec_mirror(src_pol(c, unit3(Q1 - S)), ni), nj), F8(1.0f) / L, LenF8{L, Lh});
     }
 }
 
 // order-3 candidate path (faces fs, the candidate list's sequence q): the
 // images by mirroring the dual-number source, the points backwards from P
-template <typename DT>
-__device__ __noinline__ void adj_seq3(const Ctx &c, int q, int4 sq, v3t<DT> S, v3t<DT> P, const FreqC &fq,
+__device__ __noinline__ void adj_seq38(const Ctx &c, int q, int4 sq, v3t<F8> S, v3t<F8> P, const FreqC &fq,
                                       AccAdj &acc) {
-    typedef decltype(DT().v) SC;
-    v3t<DT> ni, nj, nk;
-    DT di, dj, dk;
-    face_plane<DT>(c, sq.x, &ni, &di);
-    face_plane<DT>(c, sq.y, &nj, &dj);
-    face_plane<DT>(c, sq.z, &nk, &dk);
-    const v3t<DT> S1 = mirror_pt(S, ni, di);
-    const v3t<DT> S2 = mirror_pt(S1, nj, dj);
-    const v3t<DT> S3 = mirror_pt(S2, nk, dk);
-    const DT e3 = dot3(nk, S3) - dk, p3 = dot3(nk, P) - dk;
-    const v3t<DT> Q3 = S3 + (P - S3) * (e3 / (e3 - p3));
-    const DT e2 = dot3(nj, S2) - dj, p2 = dot3(nj, Q3) - dj;
-    const v3t<DT> Q2 = S2 + (Q3 - S2) * (e2 / (e2 - p2));
-    const DT e1 = dot3(ni, S1) - di, p1 = dot3(ni, Q2) - di;
-    const v3t<DT> Q1 = S1 + (Q2 - S1) * (e1 / (e1 - p1));
-    const DT L = norm3(Q1 - S) + norm3(Q2 - Q1) + norm3(Q3 - Q2) + norm3(P - Q3);
-    const v3t<DT> s1 = unit3(Q1 - S), s2 = unit3(Q2 - Q1), s3 = unit3(Q3 - Q2), s4 = unit3(P - Q3);
-    const v3t<DT> e0 = src_pol(c, s1);
-    cpx<DT> E[3] = {mkc<DT>(e0.x, DT(0.0f)), mkc<DT>(e0.y, DT(0.0f)), mkc<DT>(e0.z, DT(0.0f))};
+    v3t<F8> ni, nj, nk;
+    F8 di, dj, dk;
+    face_plane<F8>(c, sq.x, &ni, &di);
+    face_plane<F8>(c, sq.y, &nj, &dj);
+    face_plane<F8>(c, sq.z, &nk, &dk);
+    const v3t<F8> S1 = mirror_pt(S, ni, di);
+    const v3t<F8> S2 = mirror_pt(S1, nj, dj);
+    const v3t<F8> S3 = mirror_pt(S2, nk, dk);
+    const F8 e3 = dot3(nk, S3) - dk, p3 = dot3(nk, P) - dk;
+    const v3t<F8> Q3 = S3 + (P - S3) * (e3 / (e3 - p3));
+    const F8 e2 = dot3(nj, S2) - dj, p2 = dot3(nj, Q3) - dj;
+    const v3t<F8> Q2 = S2 + (Q3 - S2) * (e2 / (e2 - p2));
+    const F8 e1 = dot3(ni, S1) - di, p1 = dot3(ni, Q2) - di;
+    const v3t<F8> Q1 = S1 + (Q2 - S1) * (e1 / (e1 - p1));
+    const F8 L = norm3(Q1 - S) + norm3(Q2 - Q1) + norm3(Q3 - Q2) + norm3(P - Q3);
+    const v3t<F8> s1 = unit3(Q1 - S), s2 = unit3(Q2 - Q1), s3 = unit3(Q3 - Q2), s4 = unit3(P - Q3);
+    const v3t<F8> e0 = src_pol(c, s1);
+    cpx<F8> E[3] = {mkc<F8>(e0.x, F8(0.0f)), mkc<F8>(e0.y, F8(0.0f)), mkc<F8>(e0.z, F8(0.0f))};
     reflect_face(c, sq.x, E, s1, s2);
     reflect_face(c, sq.y, E, s2, s3);
     reflect_face(c, sq.z, E, s3, s4);
-    dfl Lh = {0.0f, 0.0f};
-    if constexpr (sizeof(SC) == 4) Lh = df_dist_df(c.cimg[6 * q + 4], c.cimg[6 * q + 5], vals(P));
-    add_ray_cx(acc, fq, E, DT(1.0f) / L, mk_len(L, Lh));
+    const dfl Lh = df_dist_df(c.cimg[6 * q + 4], c.cimg[6 * q + 5], vals(P));
+    add_ray_cx(acc, fq, E, F8(1.0f) / L, LenF8{L, Lh});
 }
+
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -4372,84 +4669,183 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// One warp per receiver (persistent, from a queue), its lanes over the
-// receiver's listed paths.  Body gradients by atomics per path; transmitter
-// and frequency gradients summed over the warp first.
-template <typename DT>
-__global__ void __launch_bounds__(128) k_adjoint(DevScene S, const float *__restrict__ rx, int n_rx,
-                                                 const uint64_t *__restrict__ codes,
-                                                 const int32_t *__restrict__ counts, int cap,
-                                                 const float *__restrict__ gE, double *g_body, double *g_tx,
-                                                 double *g_f, unsigned long long *queue) {
-    typedef decltype(DT().v) SC;
-    Ctx c;
-    c.tri = S.tri; c.tri_aux = S.tri_alt; c.face32 = S.face32; c.face64 = S.face64;
-    c.face_rng = S.face_rng; c.face_tris = S.face_tris; c.face_box = S.face_box; c.face_occ = nullptr; c.blist = nullptr; c.n_cand_body = S.n_body; c.body = S.body;
-    c.n_tri = S.n_tri; c.n_face = S.n_face; c.n_body = S.n_body;
-    c.band = 0.0f;
-    c.S = mk3(S.tx[0], S.tx[1], S.tx[2]);
-    c.pol = mk3(S.pol[0], S.pol[1], S.pol[2]);
-    c.fock = S.fock32; c.res = S.res32; c.weid = S.weid; c.weid_L = S.weid_L;
-    c.fock64 = S.fock64; c.res64 = S.res64; c.weid64 = S.weid64;
-    c.img = S.img; c.img_pairs = S.img_pairs; c.txb = S.txb; c.occ_src = nullptr; c.occ_w = 0;
-    c.face_mat = S.face_mat;
-    c.txw = S.txw; c.bvh = S.bvh; c.bvh_tri = S.bvh_tri; c.bvh_top = nullptr; c.bvh_top_n = 0;
-    c.cand = S.cand; c.cimg = S.cimg;
-    c.n_cand = S.cand ? (S.n_cand_dev ? *S.n_cand_dev : S.n_cand) : 0;
-    const int lane = threadIdx.x & 31;
+// A block takes rpu receivers at a time from a queue and sorts their listed
+// paths by kind, the dearest first; each warp then takes 32 paths of (almost
+// always) one kind, a path per lane.
+//   What bounds it is the FP64 pipe, 2 lanes of it an SM, which a warp holds
+// for its 32 lanes whether they take part or not: with a receiver's whole list
+// over the lanes of a warp, each kind ran on 2.9 of 32 lanes (200 bodies) to
+// 6.2 (12 bodies).  Sorted, and with the FP64 fields differentiated backwards,
+// a gradient step (fields, lists and this kernel) of 4096 receivers among 200
+// bodies went from 2.58 to 1.65 ms, one of 2867 receivers, 12 bodies and three
+// frequencies with FP32 duals from 4.10 to 0.94 ms.
+constexpr int ADJ_BLOCK = 128;
+constexpr int ADJ_RX = 32;               // receivers of a unit, at most
+constexpr int ADJ_ITEMS = 1024;          // paths sorted at once
+constexpr int ADJ_KINDS = 7;
+// the sorting order of path types (dearest first); ADJ_KINDS: none
+__device__ __forceinline__ int adj_kind(int type) {
+    switch (type) {
+    case PT_RB: return 0;
+    case PT_WCP: case PT_WCM: return 1;
+    case PT_CP: case PT_CM: return 2;
+    case PT_R3: return 3;
+    case PT_R2: return 4;
+    case PT_R1: return 5;
+    case PT_LOS: return 6;
+    default: return ADJ_KINDS;
+    }
+}
+template <bool FP64>
+__global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint(DevScene S, const float *__restrict__ rx, int n_rx, int rpu,
+                                                       const uint64_t *__restrict__ codes,
+                                                       const int32_t *__restrict__ counts, int cap,
+                                                       const float *__restrict__ gE, double *g_body, double *g_tx,
+                                                       double *g_f, unsigned long long *queue) {
+    __shared__ Ctx c;
+    __shared__ int s_np[ADJ_RX], s_cnt[ADJ_KINDS], s_off[ADJ_KINDS + 1], s_max;
+    __shared__ uint16_t s_tag[ADJ_ITEMS];        // kind << 12 | rank within it (0xffff: no path)
+    __shared__ uint32_t s_item[ADJ_ITEMS];       // receiver of the unit << 16 | slot of the window
+    __shared__ unsigned long long s_unit;
+    if (threadIdx.x == 0) {
+        c = Ctx();
+        c.tri = S.tri; c.tri_aux = S.tri_alt; c.face32 = S.face32; c.face64 = S.face64;
+        c.face_rng = S.face_rng; c.face_tris = S.face_tris; c.face_box = S.face_box; c.body = S.body;
+        c.n_tri = S.n_tri; c.n_face = S.n_face; c.n_body = c.n_cand_body = S.n_body;
+        c.band = 0.0f;
+        c.S = mk3(S.tx[0], S.tx[1], S.tx[2]);
+        c.pol = mk3(S.pol[0], S.pol[1], S.pol[2]);
+        c.fock = S.fock32; c.res = S.res32; c.weid = S.weid; c.weid_L = S.weid_L;
+        c.fock64 = S.fock64; c.res64 = S.res64; c.weid64 = S.weid64;
+        c.img = S.img; c.img_pairs = S.img_pairs; c.txb = S.txb;
+        c.face_mat = S.face_mat;
+        c.txw = S.txw; c.bvh = S.bvh; c.bvh_tri = S.bvh_tri;
+        c.cand = S.cand; c.cimg = S.cimg;
+        c.n_cand = S.cand ? (S.n_cand_dev ? *S.n_cand_dev : S.n_cand) : 0;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nch = (S.n_f + NFC - 1) / NFC;
-    const v3t<DT> Sd = mk3<DT>(dvar_t<SC>(c.S.x, DS_SX), dvar_t<SC>(c.S.y, DS_SY), dvar_t<SC>(c.S.z, DS_SZ));
+    const unsigned long long n_units = ((unsigned long long)n_rx + rpu - 1) / rpu;
     double gtx[3] = {0.0, 0.0, 0.0};
     for (;;) {
-        unsigned long long q = 0;
-        if (lane == 0) q = atomicAdd(queue, 1ull);
-        q = __shfl_sync(0xffffffffu, q, 0);
-        if (q >= (unsigned long long)n_rx) break;
-        const int r = (int)q;
-        const int np = min(counts[r], cap);
-        const v3t<DT> Pd = mk3<DT>(DT(SC(rx[r])), DT(SC(rx[n_rx + r])), DT(SC(rx[2 * n_rx + r])));
-        for (int j0 = 0; j0 < np; j0 += 32) {
-            const int jj = j0 + lane;
-            for (int ch = 0; ch < nch; ++ch) {
-                const FreqC &fq = S.fqc[ch];
-                AccAdj acc;
-                acc.gE = gE; acc.n_rx = n_rx; acc.r = r; acc.f0 = ch * NFC;
-                for (int k = 0; k < ND - 1; ++k) acc.g[k] = 0.0;
-                for (int k = 0; k < NFC; ++k) acc.gf[k] = 0.0;
-                int body = -1;
-                if (jj < np) {
-                    const uint64_t code = codes[(size_t)r * cap + jj];
-                    const int type = (int)(code >> 56), id1 = (int)((code >> 28) & 0xFFFFFFFu),
-                              id2 = (int)(code & 0xFFFFFFFu);
-                    if (type == PT_LOS) adj_planar<DT>(c, 0, -1, -1, Sd, Pd, fq, acc);
-                    else if (type == PT_R1) adj_planar<DT>(c, 1, id1, -1, Sd, Pd, fq, acc);
-                    else if (type == PT_R2) adj_planar<DT>(c, 2, id1, id2, Sd, Pd, fq, acc);
-                    else if (type == PT_R3 && c.cand && id1 < c.n_cand)
-                        adj_seq3<DT>(c, id1, c.cand[id1], Sd, Pd, fq, acc);
-                    else if (type == PT_RB) {
-                        // reflection off a body: FP64 duals in both precisions (the
-                        // FP32 chain through the specular point left errors of ~1e-3
-                        // of the gradient on the test scenes)
-                        const v3t<D8> S64 = mk3<D8>(dvar(c.S.x, DS_SX), dvar(c.S.y, DS_SY), dvar(c.S.z, DS_SZ));
-                        const v3t<D8> P64 = mk3<D8>(D8((double)rx[r]), D8((double)rx[n_rx + r]),
-                                                    D8((double)rx[2 * n_rx + r]));
-                        adj_rb<D8>(c, id1, S64, P64, fq, acc);
-                        body = id1;
-                    }
-                    else if (type == PT_CP || type == PT_CM) {
-                        if (adj_creep<DT>(c, id1, type == PT_CM, id2, Sd, Pd, fq, S.enable, acc)) body = id1;
-                    } else if (type == PT_WCP || type == PT_WCM) {
-                        if (adj_creep<DT>(c, id1, type == PT_WCM, id2 & 15, Sd, Pd, fq, S.enable, acc, id2 >> 4))
-                            body = id1;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_unit = atomicAdd(queue, 1ull);
+            s_max = 0;
+        }
+        __syncthreads();
+        if (s_unit >= n_units) break;
+        const int r0 = (int)(s_unit * rpu), nr = min(rpu, n_rx - r0);
+        if (threadIdx.x < nr) {
+            const int np = min(counts[r0 + threadIdx.x], cap);
+            s_np[threadIdx.x] = np;
+            atomicMax(&s_max, np);
+        }
+        __syncthreads();
+        const int np_max = s_max;
+        for (int w0 = 0, W; w0 < np_max; w0 += W) {
+            // a window of W slots of each receiver's list: sorted by kind
+            W = min(ADJ_ITEMS / nr, np_max - w0);
+            __syncthreads();                         // (the last window's items are done with)
+            if (threadIdx.x < ADJ_KINDS) s_cnt[threadIdx.x] = 0;
+            __syncthreads();
+            for (int i = threadIdx.x; i < nr * W; i += ADJ_BLOCK) {
+                const int rl = i / W, sl = w0 + i - rl * W;
+                unsigned tag = 0xffffu;
+                if (sl < s_np[rl]) {
+                    const int k = adj_kind((int)(codes[(size_t)(r0 + rl) * cap + sl] >> 56));
+                    if (k < ADJ_KINDS) tag = (unsigned)k << 12 | (unsigned)atomicAdd(&s_cnt[k], 1);
+                }
+                s_tag[i] = (uint16_t)tag;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                s_off[0] = 0;
+                for (int k = 0; k < ADJ_KINDS; ++k) s_off[k + 1] = s_off[k] + s_cnt[k];
+            }
+            __syncthreads();
+            for (int i = threadIdx.x; i < nr * W; i += ADJ_BLOCK) {
+                const unsigned tag = s_tag[i];
+                if (tag != 0xffffu) s_item[s_off[tag >> 12] + (tag & 0xfffu)] = (unsigned)(i / W) << 16 | (unsigned)(i % W);
+            }
+            __syncthreads();
+            const int total = s_off[ADJ_KINDS];
+            for (int i0 = 32 * warp; i0 < total; i0 += ADJ_BLOCK) {
+                const bool on = i0 + lane < total;
+                const unsigned it = s_item[on ? i0 + lane : i0];
+                const int r = r0 + (int)(it >> 16);
+                const uint64_t code = codes[(size_t)r * cap + w0 + (it & 0xffffu)];
+                const int type = (int)(code >> 56), id1 = (int)((code >> 28) & 0xFFFFFFFu), id2 = (int)(code & 0xFFFFFFFu);
+                const float px = rx[r], py = rx[n_rx + r], pz = rx[2 * n_rx + r];
+                // creeping rays: way round, extra turns, feeding wall; planar: faces, order (-1: no such candidate)
+                const bool walled = type == PT_WCP || type == PT_WCM, creep = walled || type == PT_CP || type == PT_CM;
+                const int dir = type == PT_CM || type == PT_WCM, enc = walled ? id2 & 15 : id2, wall = walled ? id2 >> 4 : -1;
+                int fs[3] = {id1, id2, -1}, order = type == PT_LOS ? 0 : (type == PT_R1 ? 1 : 2);
+                if (type == PT_R3) {
+                    order = c.cand && id1 < c.n_cand ? 3 : -1;
+                    if (order == 3) {
+                        const int4 sq = c.cand[id1];
+                        fs[0] = sq.x; fs[1] = sq.y; fs[2] = sq.z;
                     }
                 }
-                if (body >= 0)
-                    for (int k = 0; k < 4; ++k)
-                        if (acc.g[k] != 0.0) atomicAdd(&g_body[4 * body + k], acc.g[k]);
-                for (int k = 0; k < 3; ++k) gtx[k] += acc.g[DS_SX + k];
-                for (int f = 0; f < fq.nf; ++f) {
-                    const double v = warp_sum(acc.gf[f]);
-                    if (lane == 0 && v != 0.0) atomicAdd(&g_f[ch * NFC + f], v);
+                for (int ch = 0; ch < nch; ++ch) {
+                    const FreqC &fq = S.fqc[ch];
+                    AccAdj acc;
+                    acc.gE = gE; acc.n_rx = n_rx; acc.r = r; acc.f0 = ch * NFC;
+                    for (int k = 0; k < 7; ++k) acc.g[k] = 0.0;
+                    for (int k = 0; k < NFC; ++k) acc.gf[k] = 0.0;
+                    int body = -1;
+                    if (on) {
+                        if (type == PT_RB) {
+                            const v3t<D7> Sd = mk3<D7>(dvar_t<double, 7>(c.S.x, DS_SX), dvar_t<double, 7>(c.S.y, DS_SY),
+                                                       dvar_t<double, 7>(c.S.z, DS_SZ));
+                            const v3t<D7> Pd = mk3<D7>(D7((double)px), D7((double)py), D7((double)pz));
+                            AdjRec R;
+                            adj_rb(c, id1, Sd, Pd, R);
+                            adj_apply<true>(c, fq, R, 0, acc);
+                            body = id1;
+                        } else if constexpr (FP64) {
+                            if (creep) {
+                                const v3t<D7> Sd = mk3<D7>(dvar_t<double, 7>(c.S.x, DS_SX), dvar_t<double, 7>(c.S.y, DS_SY),
+                                                           dvar_t<double, 7>(c.S.z, DS_SZ));
+                                const v3t<D7> Pd = mk3<D7>(D7((double)px), D7((double)py), D7((double)pz));
+                                AdjRec R;
+                                int jpow;
+                                D7 ei[2];
+                                const int parts = adj_creep(c, id1, dir, enc, Sd, Pd, S.enable, wall, R, &jpow, ei);
+#pragma unroll 1
+                                for (int p = 0; p < parts; ++p) {
+                                    if (p) { R.Es = ei[0]; R.Eh = ei[1]; }
+                                    adj_apply<false>(c, fq, R, jpow + p, acc);
+                                }
+                                if (parts) body = id1;
+                            } else if (order >= 0) {
+                                const v3t<D3> Sd = mk3<D3>(dvar_t<double, 3>(c.S.x, 0), dvar_t<double, 3>(c.S.y, 1),
+                                                           dvar_t<double, 3>(c.S.z, 2));
+                                const v3t<D3> Pd = mk3<D3>(D3((double)px), D3((double)py), D3((double)pz));
+                                adj_planar(c, order, fs, Sd, Pd, fq, acc);
+                            }
+                        } else {
+                            const v3t<F8> Sd = mk3<F8>(dvar_t<float, 8>(c.S.x, DS_SX), dvar_t<float, 8>(c.S.y, DS_SY),
+                                                       dvar_t<float, 8>(c.S.z, DS_SZ));
+                            const v3t<F8> Pd = mk3<F8>(F8(px), F8(py), F8(pz));
+                            if (creep) {
+                                if (adj_creep8(c, id1, dir, enc, Sd, Pd, fq, S.enable, acc, wall)) body = id1;
+                            } else if (order == 3) {
+                                adj_seq38(c, id1, c.cand[id1], Sd, Pd, fq, acc);
+                            } else if (order >= 0) {
+                                adj_planar8(c, order, fs[0], fs[1], Sd, Pd, fq, acc);
+                            }
+                        }
+                    }
+                    if (body >= 0)
+                        for (int k = 0; k < 4; ++k)
+                            if (acc.g[k] != 0.0) atomicAdd(&g_body[4 * body + k], acc.g[k]);
+                    for (int k = 0; k < 3; ++k) gtx[k] += acc.g[DS_SX + k];
+                    for (int f = 0; f < fq.nf; ++f) {
+                        const double v = warp_sum(acc.gf[f]);
+                        if (lane == 0 && v != 0.0) atomicAdd(&g_f[ch * NFC + f], v);
+                    }
                 }
             }
         }
@@ -4471,12 +4867,14 @@ int launch_adjoint(const DevScene &S, const float *rx_soa, int n_rx, const uint6
         int dev = 0, nsm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        long long need = ((long long)n_rx + 3) / 4;
-        int grid = (int)(need < 4LL * nsm ? need : 4LL * nsm);
+        // units of as many receivers as leave three or more for every SM: more
+        // receivers a unit fill the last warp of each kind better
+        const int rpu = max(1, min(ADJ_RX, n_rx / (3 * nsm)));
+        const int units = (n_rx + rpu - 1) / rpu, grid = min(units, 2 * nsm);
         if (precision == RT_PREC_FP64)
-            k_adjoint<D8><<<grid, 128, 0, st>>>(S, rx_soa, n_rx, codes, counts, cap, grad_e, g_body, g_tx, g_f, queue);
+            k_adjoint<true><<<grid, ADJ_BLOCK, 0, st>>>(S, rx_soa, n_rx, rpu, codes, counts, cap, grad_e, g_body, g_tx, g_f, queue);
         else
-            k_adjoint<F8><<<grid, 128, 0, st>>>(S, rx_soa, n_rx, codes, counts, cap, grad_e, g_body, g_tx, g_f, queue);
+            k_adjoint<false><<<grid, ADJ_BLOCK, 0, st>>>(S, rx_soa, n_rx, rpu, codes, counts, cap, grad_e, g_body, g_tx, g_f, queue);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
