@@ -30,7 +30,8 @@
 // membership inclusive, bodies strict).  Path lengths are accumulated as
 // double-float so that the phase 2 pi frac(L / lambda) keeps ~1e-7 rad at
 // 28 GHz over tens of metres.  Reflection points near grazing incidence are
-// refined in FP64.  RT_PREC_FP64 runs everything in FP64.
+// refined in FP64.  RT_PREC_FP64 takes every value from FP64; its decisions are
+// FP32's where those are certain by a wide margin, and FP64's otherwise.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -104,6 +105,10 @@ struct Ctx {
     // from the source to a point of body b (occ_w = 0: no masks)
     const uint32_t *occ_src;
     int occ_w;
+    // wall -> creeping kernels: the same per (face f, body b), words from (f
+    // n_body + b) occ_w on: bodies that may block the source -> f, and f ->
+    // body b, on the way of the image's ray to b (nullptr: no masks)
+    const uint32_t *occ_w1, *occ_w2;
 };
 
 template <typename T>
@@ -1436,7 +1441,8 @@ __device__ __forceinline__ dfl df_norm3(const dfl w[3]) {
 constexpr double COS_MIN = 1e-30;
 
 // body reflection candidate (sphere or vertical cylinder)
-template <typename T>
+// (VIS false: the legs are known to be clear)
+template <typename T, bool VIS = true>
 __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Frame<T> &F, Geo<T> &g,
                        const uint32_t *occ_rx = nullptr) {
     float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
@@ -1481,8 +1487,10 @@ __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Fr
     // coefficient's pole (both of order cos^(1/2)) would meet as 0 * inf: the
     // smallest positive value keeps their finite product
     const T cth = Fmax(-dot3(shi, n), T(COS_MIN));
-    if (!conj(acc, vis_to_dec(blocked_leg(c, S, Q, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
-    if (!conj(acc, vis_to_dec(blocked_leg(c, Q, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    if constexpr (VIS) {
+        if (!conj(acc, vis_to_dec(blocked_leg(c, S, Q, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
+        if (!conj(acc, vis_to_dec(blocked_leg(c, Q, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    }
     if constexpr (sizeof(T) == 4) {
         // total length s^i + s^r to the FP32 surface point c + a n, each leg in
         // double-float (the length is stationary in psi, so the FP32 root and
@@ -1520,8 +1528,9 @@ __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Fr
 }
 
 // creeping candidate, dir 0 short way, 1 long way (SRC_LEG false: the leg
-// from the source S to Q1 is the caller's, e.g. S is a source image)
-template <typename T, bool SRC_LEG = true>
+// from the source S to Q1 is the caller's, e.g. S is a source image; VIS
+// false: the legs are known to be clear)
+template <typename T, bool SRC_LEG = true, bool VIS = true>
 __device__ int cand_creep(const Ctx &c, int b, int dir, v3t<T> S, v3t<T> P, T band, const Frame<T> &F, Geo<T> &g,
                           const uint32_t *occ_rx = nullptr) {
     float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
@@ -1582,10 +1591,12 @@ __device__ int cand_creep(const Ctx &c, int b, int dir, v3t<T> S, v3t<T> P, T ba
         g.dperp = T(0);
         g.amp = T(1) / Sqrt(g.sp * g.sq * (g.sp + g.t + g.sq));
     }
-    if constexpr (SRC_LEG) {
+    if constexpr (SRC_LEG && VIS) {
         if (!conj(acc, vis_to_dec(blocked_leg(c, S, g.Q1, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
     }
-    if (!conj(acc, vis_to_dec(blocked_leg(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    if constexpr (VIS) {
+        if (!conj(acc, vis_to_dec(blocked_leg(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    }
     return acc;
 }
 
@@ -1603,16 +1614,40 @@ __device__ __forceinline__ v3t<T> wall_point(const Ctx &c, int f, v3t<T> Sw, v3t
     return Sw + (Q1 - Sw) * (dI / (dI - *dQ));
 }
 template <typename T>
-__device__ int wall_legs(const Ctx &c, int f, int b, v3t<T> S, v3t<T> Sw, v3t<T> Q1, T band) {
+__device__ __forceinline__ int wall_geo(const Ctx &c, int f, v3t<T> S, v3t<T> Sw, v3t<T> Q1, T band, v3t<T> *Qw) {
     v3t<T> n; T d;
     face_plane<T>(c, f, &n, &d);
     T dQ;
-    const v3t<T> Qw = wall_point(c, f, Sw, Q1, &dQ);
+    *Qw = wall_point(c, f, Sw, Q1, &dQ);
     int acc = D_YES;
     if (!conj(acc, side_dec(dot3(n, S) - d, dQ, band, true))) return D_NO;
-    if (!conj(acc, in_face(c, f, Qw, band))) return D_NO;
+    if (!conj(acc, in_face(c, f, *Qw, band))) return D_NO;
+    return acc;
+}
+__device__ int wall_legs(const Ctx &c, int f, int b, v3t<dx> S, v3t<dx> Sw, v3t<dx> Q1, dx band) {
+    v3t<dx> Qw;
+    int acc = wall_geo<dx>(c, f, S, Sw, Q1, band, &Qw);
+    if (acc == D_NO) return D_NO;
     if (!conj(acc, vis_to_dec(blocked(c, S, Qw, f, -1, -1, band)))) return D_NO;
     if (!conj(acc, vis_to_dec(blocked(c, Qw, Q1, f, -1, b, band)))) return D_NO;
+    return acc;
+}
+// The whole wall -> creeping candidate in FP32.  Its geometry comes first, the
+// legs last: a leg's test costs more than all of the geometry, which leaves
+// out every wall point off its wall or behind the body.  The legs on the
+// source's side first: neighbouring receivers share them, so that a blocked
+// one ends the candidate for the whole warp.
+__device__ __forceinline__ int cand_wcreep(const Ctx &c, int f, int b, int dir, v3t<float> S, v3t<float> Sw, v3t<float> P,
+                                           float band, const Frame<float> &F, Geo<float> &g, const uint32_t *occ_rx) {
+    int acc = cand_creep<float, false, false>(c, b, dir, Sw, P, band, F, g);
+    if (acc == D_NO) return D_NO;
+    v3t<float> Qw;
+    if (!conj(acc, wall_geo<float>(c, f, S, Sw, g.Q1, band, &Qw))) return D_NO;
+    const uint32_t *m1 = c.occ_w1 ? c.occ_w1 + (f * c.n_body + b) * c.occ_w : nullptr;
+    const uint32_t *m2 = c.occ_w2 ? c.occ_w2 + (f * c.n_body + b) * c.occ_w : nullptr;
+    if (!conj(acc, vis_to_dec(blocked_mask(c, S, Qw, f, -1, -1, band, m1, c.occ_w)))) return D_NO;
+    if (!conj(acc, vis_to_dec(blocked_mask(c, Qw, g.Q1, f, -1, b, band, m2, c.occ_w)))) return D_NO;
+    if (!conj(acc, vis_to_dec(blocked_leg(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
     return acc;
 }
 
@@ -1702,15 +1737,23 @@ __device__ void pekeris(const Ctx &c, dx xid, cpx<dx> &psd, cpx<dx> &phd, bool r
     cpx<double> ps, ph;
     if (xi > XI_HI) {
         cpx<double> ss = mkc(0.0, 0.0), sh = mkc(0.0, 0.0);
+        // (terms below 2^-60 of the first are left out)
+        const double x0s = c.res64[0].x, x0h = c.res64[1].x;
         for (int n = 0; n < FOCK_NRES; ++n) {
-            dq4 rs = c.res64[2 * n], rh = c.res64[2 * n + 1];
-            double sn, cs;
-            sincos(xi * rs.y, &sn, &cs);
-            double e = exp(-xi * rs.x) * rs.z;
-            ss = ss + mkc(e * cs, -e * sn);
-            sincos(xi * rh.y, &sn, &cs);
-            e = exp(-xi * rh.x) * rh.z;
-            sh = sh + mkc(e * cs, -e * sn);
+            const dq4 rs = c.res64[2 * n], rh = c.res64[2 * n + 1];
+            const bool s_on = xi * (rs.x - x0s) <= 42.0, h_on = xi * (rh.x - x0h) <= 42.0;
+            if (!s_on && !h_on) break;
+            double sn, cs, e;
+            if (s_on) {
+                sincos(xi * rs.y, &sn, &cs);
+                e = exp(-xi * rs.x) * rs.z;
+                ss = ss + mkc(e * cs, -e * sn);
+            }
+            if (h_on) {
+                sincos(xi * rh.y, &sn, &cs);
+                e = exp(-xi * rh.x) * rh.z;
+                sh = sh + mkc(e * cs, -e * sn);
+            }
         }
         cpx<double> pre = mkc(-cos(M_PI / 12.0), sin(M_PI / 12.0)) * (0.5 / sqrt(M_PI));
         ps = pre * ss;
@@ -2479,7 +2522,7 @@ __device__ __noinline__ int esc_wcreep(const Ctx &c, int wf, int b, int dir, v3t
     Frame<dx> F;
     body_frame(c, b, Sw, Pd, dx(0.0), F);
     int d = (F.dec == D_NO) ? D_NO : cand_creep<dx, false>(c, b, dir, Sw, Pd, dx(0.0), F, g);
-    if (d == D_YES) d = wall_legs<dx>(c, wf, b, Sd, Sw, g.Q1, dx(0.0));
+    if (d == D_YES) d = wall_legs(c, wf, b, Sd, Sw, g.Q1, dx(0.0));
     if (d != D_YES) return d;
     if (c.body[2 * b + 1].y == 0.0f) {
         *caustic = half_lambda_max > g.dperp.v;
@@ -2499,6 +2542,49 @@ __device__ __noinline__ int esc_wcreep(const Ctx &c, int wf, int b, int dir, v3t
         acc_zero(a);
         field_wcreep<dx, dx, true>(c, a, fq, wf, Sd, Sw, Pd, g, g.sp + g.t + g.sq, enable);
         contrib_from(out, a);
+    }
+    return d;
+}
+
+// ------------------------------------------------------------------ FP64 evaluation: FP32 filter
+// RT_PREC_FP64 decides a candidate in FP32 first, as RT_PREC_FP32 does but with
+// a band FILT times as wide, and goes to FP64 for what is left: the geometry of
+// the candidates that are certainly valid, and the whole decision of the
+// uncertain ones.  What bounds the FP64 kernels is the FP64 pipe (2 lanes an
+// SM), and most candidates are no path: 24047 receivers, 20 bodies, three
+// frequencies took 1.03 -> 0.72 ms in the planar kernel and 3.24 -> 2.97 ms in the
+// creeping one (its fields are the rest), 1.72 -> 1.83 in that of reflections.
+constexpr float FILT = 16.0f;
+__device__ __noinline__ int filt_rb(const Ctx &c, int b, v3t<float> P, const uint32_t *occ_rx) {
+    const float band = FILT * c.band;
+    Frame<float> F;
+    Geo<float> g;
+    body_frame(c, b, c.S, P, band, F);
+    return cand_rb<float>(c, b, c.S, P, band, F, g, occ_rx);
+}
+// both ways round: the decision of dir in bits 2 dir, 2 dir + 1
+__device__ __noinline__ int filt_creep(const Ctx &c, int b, v3t<float> P, const uint32_t *occ_rx) {
+    const float band = FILT * c.band;
+    Frame<float> F;
+    body_frame(c, b, c.S, P, band, F);
+    int d = 0;
+#pragma unroll 1
+    for (int dir = 0; dir < 2; ++dir) {
+        Geo<float> g;
+        d |= cand_creep<float>(c, b, dir, c.S, P, band, F, g, occ_rx) << (2 * dir);
+    }
+    return d;
+}
+__device__ __noinline__ int filt_wcreep(const Ctx &c, int wf, int b, v3t<float> P, const uint32_t *occ_rx) {
+    const float band = FILT * c.band;
+    const v3t<float> Sw = wall_img_f(c, wf);
+    Frame<float> F;
+    body_frame_tb(c, c.txw + 2 * (size_t)wf * c.n_body, b, Sw, P, band, F);
+    int d = 0;
+#pragma unroll 1
+    for (int dir = 0; dir < 2; ++dir) {
+        Geo<float> g;
+        d |= cand_wcreep(c, wf, b, dir, c.S, Sw, P, band, F, g, occ_rx) << (2 * dir);
     }
     return d;
 }
@@ -2710,8 +2796,9 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                                               int &nrec_out, const uint32_t *qmask = nullptr, unsigned lanes = 0u,
                                               uint32_t *pwm = nullptr, int *cstk = nullptr) {
     constexpr bool BODIES = (CLS & CLS_BODIES) != 0;
-    const bool fp32 = sizeof(T) == 4;
+    constexpr bool fp32 = sizeof(T) == 4;
     const T band = fp32 ? T(c.band) : T(0);
+    const float fband = fp32 ? c.band : FILT * c.band;   // the FP32 decisions' band
     // fqs[0]: the frequency chunk of the body classes' fields; the planar
     // rays take all nfq chunks (each with its own partial sums)
     const FreqC &fq = fqs[0];
@@ -2743,29 +2830,25 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
     // itself; it is the same in each)
     int inside = 0;
     for (int b = 0; b < c.n_body && !inside; ++b) {
-        float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
-        int d;
-        T ex = P.x - T((double)q0.x), ey = P.y - T((double)q0.y), ez = P.z - T((double)q0.z), a = T((double)q0.w);
-        if (fp32) {
-            T m = (q1.y == 0.0f) ? a - Sqrt(ex * ex + ey * ey + ez * ez)
-                                 : Fmin(Fmin(a - Sqrt(ex * ex + ey * ey), P.z - T((double)q0.z)),
-                                        T((double)q0.z) + T((double)q1.x) - P.z);
-            d = decide(m, band, D_YES);
-            if (d == D_UNSURE) {
+        const float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
+        const float ex = Pf.x - q0.x, ey = Pf.y - q0.y, ez = Pf.z - q0.z, a = q0.w;
+        const float m = (q1.y == 0.0f) ? a - Sqrt(ex * ex + ey * ey + ez * ez)
+                                       : Fmin(Fmin(a - Sqrt(ex * ex + ey * ey), Pf.z - q0.z), q0.z + q1.x - Pf.z);
+        int d = decide(m, fband, D_YES);
+        if (d == D_UNSURE) {
+            if constexpr (fp32) {
                 if (part == 0 && first_chunk) escalated();   // every share and chunk takes it; one counts it
                 else fl |= RT_FLAG_ESCALATED;
-                d = esc_inside(c, b, Pf);
             }
-        } else {
             d = esc_inside(c, b, Pf);
         }
         inside = (d == D_YES);
     }
 
-    // planar occluder masks (FP32 fields, enumeration): the lanes `lanes`
+    // planar occluder masks (fields, enumeration): the lanes `lanes`
     // (every lane of the warp that evaluates a receiver) share them; pnw mask
     // words per leg, 0 without masks
-    constexpr bool PM = sizeof(T) == 4 && ((!PATHS && CLS == CLS_PLANAR) || CLS == CLS_SEQ);
+    constexpr bool PM = (!PATHS && CLS == CLS_PLANAR) || (fp32 && CLS == CLS_SEQ);
     unsigned pl = 0u;
     int pnw = 0;
     float tcx = 0.0f, tcy = 0.0f, tcr = 0.0f;
@@ -2776,6 +2859,40 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
             if (!inside) lanes_box(pl, true, Pf.x, Pf.y, tcx, tcy, tcr);
         }
     }
+    // enumerated planar candidates in FP32, with the legs' masks where there are some
+    auto dec_r1 = [&](int i, Geo<float> &g) {
+        if constexpr (PM) {
+            if (pnw) {
+                int d = cand_r1_geo<float>(c, i, c.S, Pf, fband, g);
+                const bool v = d != D_NO;
+                float qx, qy, qr;
+                lanes_box(pl, v, g.Q1.x, g.Q1.y, qx, qy, qr);
+                if (qr < 0.0f) return (int)D_NO;             // (no lane: the whole warp)
+                const float cx[3] = {c.S.x, qx, tcx}, cy[3] = {c.S.y, qy, tcy}, cr[3] = {0.0f, qr, tcr};
+                leg_masks<2>(c, pl, cx, cy, cr, pwm, pnw);
+                if (v) d = cand_r1_vis(c, i, c.S, Pf, fband, g, d, pwm, pnw);
+                return d;
+            }
+        }
+        return cand_r1<float>(c, i, c.S, Pf, fband, g);
+    };
+    auto dec_r2 = [&](int i, int j, Geo<float> &g) {
+        if constexpr (PM) {
+            if (pnw) {
+                int d = cand_r2_geo<float>(c, i, j, c.S, Pf, fband, g);
+                const bool v = d != D_NO;
+                float ax, ay, ar, bx, by, br;
+                lanes_box(pl, v, g.Q1.x, g.Q1.y, ax, ay, ar);
+                lanes_box(pl, v, g.Q2.x, g.Q2.y, bx, by, br);
+                if (ar < 0.0f) return (int)D_NO;             // (no lane: the whole warp)
+                const float cx[4] = {c.S.x, ax, bx, tcx}, cy[4] = {c.S.y, ay, by, tcy}, cr[4] = {0.0f, ar, br, tcr};
+                leg_masks<3>(c, pl, cx, cy, cr, pwm, pnw);
+                if (v) d = cand_r2_vis(c, i, j, c.S, Pf, fband, g, d, pwm, pnw);
+                return d;
+            }
+        }
+        return cand_r2<float>(c, i, j, c.S, Pf, fband, g);
+    };
     if (inside) {
         fl |= RT_FLAG_INSIDE;
     } else {
@@ -2795,9 +2912,12 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                         d = cand_los<T>(c, Sx, P, band);
                     }
                 } else {
-                    d = cand_los<T>(c, Sx, P, band);
+                    d = cand_los<float>(c, c.S, Pf, fband);
                 }
-                if (d == D_UNSURE) { escalated(); d = esc_los(c, Pf); }
+                if (d == D_UNSURE) {
+                    if constexpr (fp32) escalated();
+                    d = esc_los(c, Pf);
+                }
                 if (d == D_YES) {
                     emit(PT_LOS, 0, 0);
                     if (!PATHS) {
@@ -2880,24 +3000,14 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                     if ((1 + i) % nparts != part) continue;      // candidates 1 .. n_face
                     Geo<T> g;
                     int d;
-                    if constexpr (PM) {
-                        if (pnw) {
-                            d = cand_r1_geo<T>(c, i, Sx, P, band, g);
-                            const bool v = d != D_NO;
-                            float qx, qy, qr;
-                            lanes_box(pl, v, g.Q1.x, g.Q1.y, qx, qy, qr);
-                            if (qr < 0.0f) continue;                 // (no lane: the whole warp)
-                            const float cx[3] = {c.S.x, qx, tcx}, cy[3] = {c.S.y, qy, tcy}, cr[3] = {0.0f, qr, tcr};
-                            leg_masks<2>(c, pl, cx, cy, cr, pwm, pnw);
-                            if (v) d = cand_r1_vis(c, i, Sx, P, band, g, d, pwm, pnw);
-                        } else {
-                            d = cand_r1<T>(c, i, Sx, P, band, g);
-                        }
-                    } else {
-                        d = cand_r1<T>(c, i, Sx, P, band, g);
-                    }
-                    if constexpr (sizeof(T) == 4) {
+                    if constexpr (fp32) {
+                        d = dec_r1(i, g);
                         if (d == D_UNSURE) { escalated(); d = esc_r1(c, i, Pf, &g.Q1); }
+                    } else {
+                        Geo<float> gf;
+                        d = dec_r1(i, gf);
+                        if (d == D_UNSURE) d = cand_r1<T>(c, i, Sx, P, band, g);
+                        else if (d == D_YES && !PATHS) cand_r1_geo<T>(c, i, Sx, P, band, g);
                     }
                     if (d == D_YES) {
                         emit(PT_R1, i, 0);
@@ -2926,26 +3036,14 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                         if ((1 + i * c.n_face + j) % nparts != part) continue;   // then the ordered pairs
                         Geo<T> g;
                         int d;
-                        if constexpr (PM) {
-                            if (pnw) {
-                                d = cand_r2_geo<T>(c, i, j, Sx, P, band, g);
-                                const bool v = d != D_NO;
-                                float ax, ay, ar, bx, by, br;
-                                lanes_box(pl, v, g.Q1.x, g.Q1.y, ax, ay, ar);
-                                lanes_box(pl, v, g.Q2.x, g.Q2.y, bx, by, br);
-                                if (ar < 0.0f) continue;             // (no lane: the whole warp)
-                                const float cx[4] = {c.S.x, ax, bx, tcx}, cy[4] = {c.S.y, ay, by, tcy},
-                                            cr[4] = {0.0f, ar, br, tcr};
-                                leg_masks<3>(c, pl, cx, cy, cr, pwm, pnw);
-                                if (v) d = cand_r2_vis(c, i, j, Sx, P, band, g, d, pwm, pnw);
-                            } else {
-                                d = cand_r2<T>(c, i, j, Sx, P, band, g);
-                            }
-                        } else {
-                            d = cand_r2<T>(c, i, j, Sx, P, band, g);
-                        }
-                        if constexpr (sizeof(T) == 4) {
+                        if constexpr (fp32) {
+                            d = dec_r2(i, j, g);
                             if (d == D_UNSURE) { escalated(); d = esc_r2(c, i, j, Pf, &g.Q1, &g.Q2); }
+                        } else {
+                            Geo<float> gf;
+                            d = dec_r2(i, j, gf);
+                            if (d == D_UNSURE) d = cand_r2<T>(c, i, j, Sx, P, band, g);
+                            else if (d == D_YES && !PATHS) cand_r2_geo<T>(c, i, j, Sx, P, band, g);
                         }
                         if (d == D_YES) {
                             emit(PT_R2, i, j);
@@ -3004,19 +3102,30 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                     const bool sphere = c.body[2 * bb + 1].y == 0.0f;
                     Frame<T> F;
                     v3t<T> Sw;
+                    int filt = 0;
                     if constexpr (sizeof(T) == 4) {
                         Sw = wall_img_f(c, wf);
                         body_frame_tb(c, c.txw + 2 * (size_t)wf * c.n_body, bb, Sw, P, band, F);
                     } else {
                         Sw = wall_img_d(c, wf);
-                        if (!img_outside(c, bb, Sw)) continue;
+                        filt = filt_wcreep(c, wf, bb, Pf, occ_rx);
+                        if (filt == 0 || !img_outside(c, bb, Sw)) continue;
                         body_frame(c, bb, Sw, P, band, F);
                     }
 #pragma unroll 1
                     for (int dir = 0; dir < 2; ++dir) {
                         Geo<T> g;
-                        int d = cand_creep<T, false>(c, bb, dir, Sw, P, band, F, g);
-                        if (d == D_YES) d = wall_legs<T>(c, wf, bb, Sx, Sw, g.Q1, band);
+                        int d;
+                        const int fd = (filt >> (2 * dir)) & 3;
+                        if (!fp32 && fd == D_NO) continue;
+                        if constexpr (fp32) {
+                            d = cand_wcreep(c, wf, bb, dir, Sx, Sw, P, band, F, g, occ_rx);
+                        } else if (fd == D_YES) {
+                            d = cand_creep<T, false, false>(c, bb, dir, Sw, P, band, F, g);
+                        } else {
+                            d = cand_creep<T, false>(c, bb, dir, Sw, P, band, F, g);
+                            if (d == D_YES) d = wall_legs(c, wf, bb, Sx, Sw, g.Q1, band);
+                        }
                         int cd = D_NO;
                         if (d == D_YES && sphere) {
                             if constexpr (sizeof(T) == 8) cd = (half_lambda_max > to_double(g.dperp)) ? D_YES : D_NO;
@@ -3054,12 +3163,23 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                     }
                     continue;
                 }
+                // (FP64: the FP32 filter first; each kernel has one of the two classes)
+                int filt = 0;
+                if constexpr (!fp32) {
+                    filt = (CLS & CLS_BODYREFL) != 0 ? filt_rb(c, b, Pf, occ_rx) : filt_creep(c, b, Pf, occ_rx);
+                    if (filt == 0) continue;
+                    if (PATHS && (CLS & CLS_BODYREFL) != 0 && filt == D_YES) {
+                        if (enable & RT_EN_BODYREFL) emit(PT_RB, b, 0);
+                        continue;
+                    }
+                }
                 Frame<T> F;
                 body_frame(c, b, Sx, P, band, F);
                 if constexpr ((CLS & CLS_BODYREFL) != 0) {
                     if (enable & RT_EN_BODYREFL) {
                         Geo<T> g;
-                        int d = cand_rb<T>(c, b, Sx, P, band, F, g, occ_rx);
+                        int d = !fp32 && filt == D_YES ? cand_rb<T, false>(c, b, Sx, P, band, F, g)
+                                                       : cand_rb<T>(c, b, Sx, P, band, F, g, occ_rx);
                         if constexpr (sizeof(T) == 4) {
                             if (d == D_UNSURE) {
                                 // decided in FP64, and its geometry, length and amplitude
@@ -3095,7 +3215,10 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
 #pragma unroll 1
                         for (int dir = 0; dir < 2; ++dir) {
                             Geo<T> g;
-                            int d = cand_creep<T>(c, b, dir, Sx, P, band, F, g, occ_rx);
+                            const int fd = (filt >> (2 * dir)) & 3;
+                            if (!fp32 && fd == D_NO) continue;
+                            int d = !fp32 && fd == D_YES ? cand_creep<T, true, false>(c, b, dir, Sx, P, band, F, g)
+                                                         : cand_creep<T>(c, b, dir, Sx, P, band, F, g, occ_rx);
                             int cd = D_NO;
                             if (d == D_YES && sphere) {
                                 // axial caustic flag: k d_perp < pi for some frequency, i.e. d_perp < lambda_max / 2
@@ -3185,6 +3308,43 @@ __device__ __noinline__ void occ_masks(const Ctx &c, float t0x, float t0y, float
     }
 }
 
+// wall -> creeping: the masks of every (face, body) pair, the pairs wi, wi +
+// nwarps, ...  The ray of the source's image in face f to a point of body b lies
+// in the hull of the image and b's disk; its part before the face, mirrored, in
+// that of the source and the disk of b mirrored in f (an oblique face turns a
+// cylinder's axis: every body then).
+constexpr int WALL_MASK_WORDS = 2048;      // both sets (8 KB); more pairs go without
+__device__ __noinline__ void wall_masks(const Ctx &c, uint32_t *out1, uint32_t *out2, int wi, int nwarps) {
+    const int lane = threadIdx.x & 31, nb = c.n_body;
+    const float margin = 1e-3f + 9.0f * c.band;
+#pragma unroll 1
+    for (int u = wi; u < c.n_face * nb; u += nwarps) {
+        const int f = u / nb, b = u - f * nb;
+        const float4 qb = c.body[2 * b], pl = c.face32[f];
+        const v3t<float> Sw = wall_img_f(c, f);
+        const float h2 = pl.x * pl.x + pl.y * pl.y;
+        const bool oblique = fabsf(pl.z) > 1e-6f && h2 > 1e-12f;
+        const float k = 2.0f * (pl.x * qb.x + pl.y * qb.y - pl.w) * (fabsf(pl.z) > 1e-6f ? 0.0f : 1.0f);
+        const float mx = qb.x - k * pl.x, my = qb.y - k * pl.y;     // b's axis mirrored (a horizontal face: itself)
+#pragma unroll 1
+        for (int w = 0; w < c.occ_w; ++w) {
+            const int j = 32 * w + lane;
+            bool h1 = false, h2b = false;
+            if (j < nb) {
+                const float4 qj = c.body[2 * j];
+                const float lim = qb.w + qj.w + margin;
+                h1 = oblique || seg_d2(qj.x, qj.y, c.S.x, c.S.y, mx, my) <= lim * lim;
+                h2b = j != b && seg_d2(qj.x, qj.y, Sw.x, Sw.y, qb.x, qb.y) <= lim * lim;
+            }
+            const unsigned w1 = __ballot_sync(0xffffffffu, h1), w2 = __ballot_sync(0xffffffffu, h2b);
+            if (lane == 0) {
+                out1[u * c.occ_w + w] = w1;
+                out2[u * c.occ_w + w] = w2;
+            }
+        }
+    }
+}
+
 // the occluder masks of a tile's receivers: their bounding box as a disk of
 // radius rr round the box's longer midline T0 T1; every lane of the warp
 // takes part (rok: this lane's receiver exists)
@@ -3245,7 +3405,8 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
     __shared__ Ctx s_ctx;
     __shared__ FreqC s_fqs[MAX_CHUNKS];        // frequency chunks ch0 .. ch0 + nch - 1
     // stage scene (and, for the body classes, the Fock--Pekeris table)
-    const int n_fock = BODIES ? (FOCK_N + FOCK_NP) * 2 : 0, n_res = BODIES ? FOCK_NRES * 2 : 0;
+    // (FP64 kernels read their own tables in global memory)
+    const int n_fock = BODIES && sizeof(T) == 4 ? (FOCK_N + FOCK_NP) * 2 : 0, n_res = BODIES && sizeof(T) == 4 ? FOCK_NRES * 2 : 0;
     float4 *s_fock = smem;                                   // n_fock
     float4 *s_res = s_fock + n_fock;                         // n_res
     float4 *s_face = s_res + n_res;                          // n_face
@@ -3302,7 +3463,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         c.img_pairs = S.img_pairs;
         c.face_mat = S.face_mat;
         c.txb = body_sm ? s_txb : F1.txb;
-        c.occ_src = nullptr;
+        c.occ_src = c.occ_w1 = c.occ_w2 = nullptr;
         c.occ_w = 0;
         c.enc = enc;
         c.txw = frames ? nullptr : S.txw;
@@ -3334,20 +3495,25 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         const float *rx = rx_base;
         const int n_rx = F1.n_rx;
         const unsigned long long ntiles = ((unsigned long long)n_rx + 31ull) >> 5;
-        // occluder masks (FP32 body kernels): the source side per block, the
+        // occluder masks (body kernels): the source side per block, the
         // receiver side per warp (each warp takes whole tiles)
-        constexpr bool OCC = BODIES && sizeof(T) == 4 && CLS != CLS_WCREEP;
+        constexpr bool OCC = BODIES;
         const bool occ_on = OCC && S.n_body > 0 && S.n_body <= OCC_MAX_BODIES;
         const int occ_w = occ_on ? (S.n_body + 31) >> 5 : 0;
         uint32_t *s_occ_src = reinterpret_cast<uint32_t *>(s_rec);
         uint32_t *s_occ_mine = s_occ_src + (1 + warp) * S.n_body * occ_w;
+        uint32_t *s_occ_wall = s_occ_src + (1 + NW) * S.n_body * occ_w;
+        const bool wall_on = CLS == CLS_WCREEP && occ_on && 2 * S.n_face * S.n_body * occ_w <= WALL_MASK_WORDS;
         if (threadIdx.x == 0) {
             s_ctx.occ_src = occ_on ? s_occ_src : nullptr;
             s_ctx.occ_w = occ_w;
+            s_ctx.occ_w1 = wall_on ? s_occ_wall : nullptr;
+            s_ctx.occ_w2 = wall_on ? s_occ_wall + S.n_face * S.n_body * occ_w : nullptr;
         }
         __syncthreads();
         if (occ_on) {
-            occ_masks(c, c.S.x, c.S.y, c.S.x, c.S.y, 0.0f, s_occ_src, warp, NW);
+            if (CLS != CLS_WCREEP) occ_masks(c, c.S.x, c.S.y, c.S.x, c.S.y, 0.0f, s_occ_src, warp, NW);
+            if (wall_on) wall_masks(c, s_occ_wall, s_occ_wall + S.n_face * S.n_body * occ_w, warp, NW);
             __syncthreads();
         }
         asm volatile("griddepcontrol.wait;" ::: "memory");   // the previous class kernel's lists are complete
@@ -3434,21 +3600,26 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         __shared__ unsigned long long s_unit;
         __shared__ int s_fi, s_new;
         __shared__ FrameDev s_fr;
-        // occluder masks (FP32 body kernels): the source side per frame, the
+        // occluder masks (body kernels): the source side per frame, the
         // receiver side per tile, after the path records
-        constexpr bool OCC = BODIES && sizeof(T) == 4 && CLS != CLS_WCREEP;
+        constexpr bool OCC = BODIES;
         const bool occ_on = OCC && S.n_body > 0 && S.n_body <= OCC_MAX_BODIES;
         const int occ_w = occ_on ? (S.n_body + 31) >> 5 : 0;
         uint32_t *s_occ_src = reinterpret_cast<uint32_t *>(s_rec + (RECS ? NW * rcap * REC_N * 32 : 0));
         uint32_t *s_occ_rx = s_occ_src + S.n_body * occ_w;
+        uint32_t *s_occ_wall = s_occ_rx + TPB * S.n_body * occ_w;       // (single frames only, as the wall class)
+        const bool wall_on = CLS == CLS_WCREEP && occ_on && 2 * S.n_face * S.n_body * occ_w <= WALL_MASK_WORDS;
         if (threadIdx.x == 0) {
             s_fi = -1;
             if (!frames) s_fr = F1;
             s_ctx.occ_src = occ_on ? s_occ_src : nullptr;
             s_ctx.occ_w = occ_w;
+            s_ctx.occ_w1 = wall_on ? s_occ_wall : nullptr;
+            s_ctx.occ_w2 = wall_on ? s_occ_wall + S.n_face * S.n_body * occ_w : nullptr;
         }
         __syncthreads();
-        if (occ_on && !frames) occ_masks(c, c.S.x, c.S.y, c.S.x, c.S.y, 0.0f, s_occ_src, warp, NW);
+        if (occ_on && !frames && CLS != CLS_WCREEP) occ_masks(c, c.S.x, c.S.y, c.S.x, c.S.y, 0.0f, s_occ_src, warp, NW);
+        if (wall_on) wall_masks(c, s_occ_wall, s_occ_wall + S.n_face * S.n_body * occ_w, warp, NW);
         for (;;) {
             if (threadIdx.x == 0) {
                 const unsigned long long u = atomicAdd(queue, 1ull);
@@ -3503,8 +3674,10 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
             if (occ_on) {
                 // each warp makes the masks of the bodies of its own share
                 // (b = part mod NWT), so no other warp waits for them
+                // (a wall -> creeping unit may take any body: those wait for each other)
                 tile_masks(c, rx, n_rx, r, rok, s_occ_rx + grp * S.n_body * occ_w, part, NWT);
-                __syncwarp();
+                if (CLS == CLS_WCREEP) __syncthreads();
+                else __syncwarp();
             }
             // candidate-list class: this warp's surviving candidates for the tile
             bool qm_on = false;
@@ -3589,17 +3762,18 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
 
 // dynamic shared memory of a launch: scene, tables, then the path records
 // (body classes) or the wide partial sums of wide_chunks chunks (planar)
-static size_t smem_bytes(const DevScene &S, bool bodies, bool records, int blk, int rcap, int wide_chunks,
-                         int occ_sets) {
-    size_t n = (bodies ? (FOCK_N + FOCK_NP) * 2 + FOCK_NRES * 2 : 0) + (S.n_face <= SMEM_FACE_MAX ? S.n_face : 0) +
+static size_t smem_bytes(const DevScene &S, bool tables, bool records, int blk, int rcap, int wide_chunks,
+                         int occ_sets, bool wall) {
+    size_t n = (tables ? (FOCK_N + FOCK_NP) * 2 + FOCK_NRES * 2 : 0) + (S.n_face <= SMEM_FACE_MAX ? S.n_face : 0) +
                (S.bvh ? 2 * (size_t)min(S.bvh_nodes, BVH_TOP_NODES) : 0);
     if (S.n_body <= SMEM_BODY_MAX) n += 4 * S.n_body;
     if (S.n_tri <= SMEM_TRI_MAX) n += 6 * S.n_tri;
     const int occ_w = (occ_sets > 0 && S.n_body > 0 && S.n_body <= OCC_MAX_BODIES) ? (S.n_body + 31) >> 5 : 0;
+    const size_t pairs = wall ? 2 * (size_t)S.n_face * S.n_body * occ_w : 0;      // (see wall_masks)
     return n * sizeof(float4) + WEIDEMAN_N * sizeof(float) + 16 +
            (records ? sizeof(float) * (blk / 32) * rcap * REC_N * 32 : 0) +
            sizeof(float) * (blk / 32) * wide_chunks * NFC * 6 * 32 +
-           sizeof(uint32_t) * (size_t)S.n_body * occ_w * (1 + occ_sets);
+           sizeof(uint32_t) * ((size_t)S.n_body * occ_w * (1 + occ_sets) + (pairs <= WALL_MASK_WORDS ? pairs : 0));
 }
 
 // Launch state of one evaluation: the counters (escalations, one work queue
@@ -3644,11 +3818,11 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
     int rcap = (nch > 1) ? 6 : 5;
     const bool wide = is_planar(CLS) && sizeof(T) == 4 && !PATHS;
     if (nch < 1 || nch > MAX_CHUNKS || (!wide && !bodies && nch != 1)) return cudaErrorInvalidValue;
-    // occluder masks (FP32 body kernels): one source-side set, and one
+    // occluder masks (body kernels): one source-side set, and one
     // receiver-side set per tile in flight (fields) or per warp (path lists)
-    const int occ_sets = (bodies && sizeof(T) == 4 && CLS != CLS_WCREEP) ? (PATHS ? NW : NW / nwt) : 0;
+    const int occ_sets = bodies ? (PATHS ? NW : NW / nwt) : 0;
     const bool recs = bodies && sizeof(T) == 4 && !PATHS;
-    size_t sm = smem_bytes(S, bodies, recs, blk, rcap, wide ? nch : 0, occ_sets);
+    size_t sm = smem_bytes(S, bodies && sizeof(T) == 4, recs, blk, rcap, wide ? nch : 0, occ_sets, CLS == CLS_WCREEP);
     int dev = 0, nsm = 0, occ = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -3661,7 +3835,7 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
         if ((e = cudaDeviceGetAttribute(&smax, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
         if ((e = cudaFuncGetAttributes(&fa, k_eval<T, PATHS, CLS, LIST>)) != cudaSuccess) return e;
         while (rcap > recs_per_unit(CLS) && fa.sharedSizeBytes + sm > (size_t)smax)
-            sm = smem_bytes(S, bodies, recs, blk, --rcap, wide ? nch : 0, occ_sets);
+            sm = smem_bytes(S, bodies && sizeof(T) == 4, recs, blk, --rcap, wide ? nch : 0, occ_sets, CLS == CLS_WCREEP);
     }
     e = cudaFuncSetAttribute(k_eval<T, PATHS, CLS, LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
