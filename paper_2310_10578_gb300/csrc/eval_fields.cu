@@ -2613,6 +2613,7 @@ constexpr int recs_per_unit(int cls) {
     return ((cls & CLS_CREEP) ? 2 : 0) + ((cls & CLS_BODYREFL) ? 1 : 0) + ((cls & CLS_WCREEP) ? 4 : 0);
 }
 constexpr int WARPS_PER_TILE = 4;
+constexpr int PATH_TILES = 3;
 constexpr int MAX_CHUNKS = (RT_MAX_FREQS + NFC - 1) / NFC;
 constexpr int PLANAR_CHUNKS = 4;       // frequency chunks per planar launch (FP32 fields)
 constexpr int OCC_MAX_BODIES = 256;    // occluder masks up to this many bodies (FP32 body kernels)
@@ -2785,6 +2786,31 @@ __device__ __noinline__ uint32_t list_path(uint64_t *codes, int32_t *counts, int
     return RT_FLAG_OVERFLOW;
 }
 
+// Path lists shared by the warps of a block: the candidates of an enumerated
+// class in canonical order, and the code of the one at slot i.
+constexpr bool split_paths(int cls) { return cls == CLS_PLANAR || cls == CLS_BODYREFL || cls == CLS_CREEP; }
+__host__ __device__ __forceinline__ int path_slots(int cls, int n_face, int n_body) {
+    return cls == CLS_PLANAR ? 1 + n_face + n_face * n_face : (cls == CLS_BODYREFL ? n_body : (cls == CLS_CREEP ? 2 * n_body : 0));
+}
+__device__ __forceinline__ int path_slot(const Ctx &c, int type, int a, int b) {
+    switch (type) {
+    case PT_R1: return 1 + a;
+    case PT_R2: return 1 + c.n_face + a * c.n_face + b;
+    case PT_RB: return a;
+    case PT_CP: return 2 * a;
+    case PT_CM: return 2 * a + 1;
+    default: return 0;
+    }
+}
+__device__ __forceinline__ uint64_t path_code(const Ctx &c, int cls, int i) {
+    if (cls == CLS_BODYREFL) return pcode(PT_RB, i, 0);
+    if (cls == CLS_CREEP) return pcode((i & 1) ? PT_CM : PT_CP, i >> 1, c.enc);
+    if (i == 0) return pcode(PT_LOS, 0, 0);
+    if (i <= c.n_face) return pcode(PT_R1, i - 1, 0);
+    i -= 1 + c.n_face;
+    return pcode(PT_R2, i / c.n_face, i % c.n_face);
+}
+
 template <typename T, bool PATHS, int CLS, bool LIST = false>
 __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, int nfq, unsigned enable, int max_order,
                                               const float *__restrict__ rx, int n_rx, int r,
@@ -2794,7 +2820,7 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                                               const uint32_t *occ_rx, int part, int nparts,
                                               AccS<T> acc, float *rec, uint32_t &fl, unsigned &nesc, int &npath,
                                               int &nrec_out, const uint32_t *qmask = nullptr, unsigned lanes = 0u,
-                                              uint32_t *pwm = nullptr, int *cstk = nullptr) {
+                                              uint32_t *pwm = nullptr, int *cstk = nullptr, uint32_t *found = nullptr) {
     constexpr bool BODIES = (CLS & CLS_BODIES) != 0;
     constexpr bool fp32 = sizeof(T) == 4;
     const T band = fp32 ? T(c.band) : T(0);
@@ -2812,8 +2838,12 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
     if (!PATHS) acc_zero_rows(acc, nfq * NFC * 6);
     typedef typename LenOf<T>::type LT;
 
+    // (found, path lists shared by the warps of a block: bit lane of word
+    // path_slot says that the receiver has the path)
     auto emit = [&](int type, int a, int b) {
-        if (PATHS) {
+        if (PATHS && found) {
+            atomicOr(&found[path_slot(c, type, a, b)], 1u << (threadIdx.x & 31));
+        } else if (PATHS) {
             if (npath < cap) codes[(size_t)r * cap + npath] = pcode(type, a, b);
             else fl |= RT_FLAG_OVERFLOW;
         } else if constexpr (LIST) {
@@ -2845,10 +2875,10 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
         inside = (d == D_YES);
     }
 
-    // planar occluder masks (fields, enumeration): the lanes `lanes`
+    // planar occluder masks (enumeration): the lanes `lanes`
     // (every lane of the warp that evaluates a receiver) share them; pnw mask
     // words per leg, 0 without masks
-    constexpr bool PM = (!PATHS && CLS == CLS_PLANAR) || (fp32 && CLS == CLS_SEQ);
+    constexpr bool PM = CLS == CLS_PLANAR || (fp32 && CLS == CLS_SEQ);
     unsigned pl = 0u;
     int pnw = 0;
     float tcx = 0.0f, tcy = 0.0f, tcr = 0.0f;
@@ -3517,22 +3547,41 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
             __syncthreads();
         }
         asm volatile("griddepcontrol.wait;" ::: "memory");   // the previous class kernel's lists are complete
-        // path lists: each warp takes tiles of 32 consecutive receivers from
-        // the launch's queue and lists every candidate itself (codes in the
-        // canonical order)
+        // path lists.  Many tiles: each warp takes tiles of 32 consecutive
+        // receivers from the launch's queue and lists every candidate itself
+        // (codes in the canonical order).  Few (nwt > 1): the warps of a block
+        // share a tile's candidates as in the fields kernels, mark the paths found
+        // in shared memory, and one warp lists them in order.
         __shared__ uint32_t s_qmask_p[CLS == CLS_SEQ ? NW : 1][CLS == CLS_SEQ ? SEQ_MASK_WORDS : 1];
         __shared__ int s_qlist_p[CLS == CLS_SEQ ? NW : 1][64];
         constexpr bool COOP_P = CLS == CLS_SEQ && sizeof(T) == 4;
-        __shared__ uint32_t s_pwm_p[COOP_P ? NW : 1][COOP_P ? 4 * (OCC_MAX_BODIES / 32) : 1];
+        constexpr bool LEGM_P = COOP_P || CLS == CLS_PLANAR;
+        __shared__ uint32_t s_pwm_p[LEGM_P ? NW : 1][LEGM_P ? 4 * (OCC_MAX_BODIES / 32) : 1];
         __shared__ int s_cstk_p[COOP_P ? NW : 1][COOP_P ? COOP_STACK : 1];
+        constexpr bool SPLIT = split_paths(CLS);
+        __shared__ uint32_t s_fl_p[SPLIT ? NW : 1][32];
+        __shared__ unsigned long long s_tile;
+        const bool split = SPLIT && nwt > 1;
+        const int part = split ? warp : 0, nparts = split ? NW : 1;
+        uint32_t *found = split ? s_occ_src + (1 + NW) * (occ_on ? S.n_body * occ_w : 0) : nullptr;
+        const int n_found = split ? path_slots(CLS, S.n_face, S.n_body) : 0;
+        if (split) s_occ_mine = s_occ_src + S.n_body * occ_w;        // (one set: a warp makes and reads its own bodies')
         for (;;) {
             unsigned long long t = 0;
-            if (lane == 0) t = atomicAdd(queue, 1ull);
-            t = __shfl_sync(0xffffffffu, t, 0);
+            if (split) {
+                __syncthreads();                     // (the last tile is listed)
+                if (threadIdx.x == 0) s_tile = atomicAdd(queue, 1ull);
+                for (int i = threadIdx.x; i < n_found; i += blockDim.x) found[i] = 0u;
+                __syncthreads();
+                t = s_tile;
+            } else {
+                if (lane == 0) t = atomicAdd(queue, 1ull);
+                t = __shfl_sync(0xffffffffu, t, 0);
+            }
             if (t >= ntiles) break;
             int r = (int)(t * 32ull) + lane;
             if (occ_on) {
-                tile_masks(c, rx, n_rx, r, r < n_rx, s_occ_mine, 0, 1);
+                tile_masks(c, rx, n_rx, r, r < n_rx, s_occ_mine, part, nparts);
                 __syncwarp();
             }
             bool qm_on = false;
@@ -3541,22 +3590,40 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                                       &s_qmask_p[warp][0], &s_qlist_p[warp][0]);
             }
             const unsigned lanes_p = __ballot_sync(0xffffffffu, r < n_rx);
+            uint32_t fl = 0;
+            int npath = 0;
             if (r < n_rx) {
                 AccS<T> acc{nullptr};                // no fields in this mode
-                uint32_t fl;
                 unsigned nesc;
-                int npath = accumulate ? counts[r] : 0;
+                npath = accumulate && part == 0 ? counts[r] : 0;
                 int nrec;
                 eval_receiver<T, PATHS, CLS, LIST>(c, s_fqs, 1, S.enable, S.max_order, rx, n_rx, r, codes, counts, cap,
                                                    F1.hl,
                                              0, CLS == CLS_WCREEP ? c.n_face * c.n_body : c.n_cand_body, true, false, 0,
-                                             occ_on ? s_occ_mine : nullptr, 0, 1, acc,
+                                             occ_on ? s_occ_mine : nullptr, part, nparts, acc,
                                              nullptr, fl, nesc, npath, nrec, qm_on ? &s_qmask_p[warp][0] : nullptr,
-                                             COOP_P ? lanes_p : 0u, &s_pwm_p[COOP_P ? warp : 0][0],
-                                             &s_cstk_p[COOP_P ? warp : 0][0]);
+                                             LEGM_P ? lanes_p : 0u, &s_pwm_p[LEGM_P ? warp : 0][0],
+                                             &s_cstk_p[COOP_P ? warp : 0][0], found);
+                if (nesc) atomicAdd(esc_counter, (unsigned long long)nesc);
+            }
+            if (split) {
+                s_fl_p[SPLIT ? warp : 0][lane] = fl;
+                __syncthreads();
+                if (warp != 0) continue;
+                for (int w = 1; w < NW; ++w) fl |= s_fl_p[SPLIT ? w : 0][lane];
+                if (r < n_rx) {
+                    npath = accumulate ? counts[r] : 0;
+                    for (int i = 0; i < n_found; ++i) {
+                        if (!(found[i] >> lane & 1u)) continue;
+                        if (npath < cap) codes[(size_t)r * cap + npath] = path_code(c, CLS, i);
+                        else fl |= RT_FLAG_OVERFLOW;
+                        ++npath;
+                    }
+                }
+            }
+            if (r < n_rx) {
                 counts[r] = npath;
                 if (fl_base) fl_base[r] = accumulate ? (fl_base[r] | fl) : fl;
-                if (nesc) atomicAdd(esc_counter, (unsigned long long)nesc);
             }
         }
     } else {
@@ -3826,6 +3893,17 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
     int dev = 0, nsm = 0, occ = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    bool split = false;
+    if constexpr (PATHS) {
+        // path lists: a block's warps share a tile until each warp would have
+        // PATH_TILES of its own: 11468 receivers, 20 bodies (359 tiles, for 608 and
+        // 1824 warps) took 677 us a warp per tile, 329 shared
+        split = split_paths(CLS) && (CLS != CLS_PLANAR || S.n_face <= RT_MAX_ENUM_FACES) &&
+                (long long)W.n_tiles < (long long)PATH_TILES * nsm * min_blocks(CLS, sizeof(T) == 4) * NW;
+        nwt = split ? NW : 1;
+        if (split) sm += sizeof(uint32_t) * path_slots(CLS, S.n_face, S.n_body);
+    }
     if (recs) {
         // many bodies (their data and occluder masks in shared memory): fewer
         // records per lane -- fewer bodies per geometry pass, or earlier
@@ -3841,7 +3919,6 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
     if (e != cudaSuccess) return e;
     // persistent grid: the blocks that fit on the device at once, at most
     // one per work unit
-    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_eval<T, PATHS, CLS, LIST>, blk, sm)) != cudaSuccess) return e;
     // (path lists: each warp takes whole tiles; up to one block per tile, so
     // that a few tiles spread over as many SMs)
