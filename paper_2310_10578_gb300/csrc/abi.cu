@@ -6,6 +6,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <complex>
 #include <map>
 #include <mutex>
 #include <string>
@@ -24,6 +25,7 @@ struct DevTable {
     double2 *fock64 = nullptr;
     float4 *res32 = nullptr;
     dq4 *res64 = nullptr;
+    double2 *p64 = nullptr;
     float *weid = nullptr;
     double *weid64 = nullptr;
     float weid_L = 0.f;
@@ -47,6 +49,50 @@ static void weideman(std::vector<double> &a, double *L) {
         a[n - 1] = s / (2.0 * M);
     }
 }
+
+// The polynomial pieces of P (see P64_PER) from the residue series: Chebyshev
+// interpolation on each piece, written in powers of t.  Series and sums in long
+// double: an FP64 series carries the rounding of xi alpha, 5e-15 at XI_P.
+#pragma nv_diag_suppress 20208        // (long double: host code only)
+static void fock_pieces(const FockHost &H, std::vector<double2> &out) {
+    typedef long double R;
+    typedef std::complex<R> C;
+    const int n = P64_C;
+    const R pi = 3.14159265358979323846264338327950288L, c6 = sqrtl(R(3)) / 2, w = R(1) / P64_PER;
+    const C pre = -std::polar(R(0.5) / sqrtl(pi), -pi / 12);
+    auto turn = [&](R x, R al) { return std::exp(C(-x * al * c6, -x * al / 2)); };      // e^{-x alpha e^{j pi/6}}
+    std::vector<std::vector<R>> cheb(n, std::vector<R>(n, R(0)));                       // T_k in powers of t
+    cheb[0][0] = cheb[1][1] = 1;
+    for (int k = 2; k < n; ++k)
+        for (int i = 0; i < n; ++i) cheb[k][i] = (i ? 2 * cheb[k - 1][i - 1] : R(0)) - cheb[k - 2][i];
+    std::vector<R> node(n);
+    for (int i = 0; i < n; ++i) node[i] = cosl(pi * (i + R(0.5)) / n);
+    std::vector<R> dct((size_t)n * n);
+    for (int k = 0; k < n; ++k)
+        for (int i = 0; i < n; ++i) dct[k * n + i] = cosl(pi * k * (i + R(0.5)) / n);
+    for (int kind = 0; kind < 2; ++kind) {
+        const double *al = &H.res[2 * kind * FOCK_NRES], *cf = al + FOCK_NRES;
+        std::vector<C> step((size_t)n * FOCK_NRES);      // from a piece's centre to its nodes
+        for (int i = 0; i < n; ++i)
+            for (int q = 0; q < FOCK_NRES; ++q) step[i * FOCK_NRES + q] = turn(w / 2 * node[i], al[q]);
+        for (int j = 0; j < P64_N; ++j) {
+            std::vector<C> v(n, C(0)), a(n, C(0));
+            for (int q = FOCK_NRES - 1; q >= 0; --q) {
+                const C mid = pre * R(cf[q]) * turn(R(XI_HI) + w * (j + R(0.5)), al[q]);
+                for (int i = 0; i < n; ++i) v[i] += mid * step[i * FOCK_NRES + q];
+            }
+            for (int k = 0; k < n; ++k) {
+                C ck = 0;
+                for (int i = 0; i < n; ++i) ck += v[i] * dct[k * n + i];
+                ck *= R(k ? 2 : 1) / n;
+                for (int i = 0; i <= k; ++i) a[i] += ck * cheb[k][i];
+            }
+            for (int i = 0; i < n; ++i)
+                out[((size_t)j * 2 + kind) * n + i] = make_double2((double)a[i].real(), (double)a[i].imag());
+        }
+    }
+}
+#pragma nv_diag_default 20208
 
 static int get_table(DevTable **out) {
     int dev = 0;
@@ -84,6 +130,8 @@ static int get_table(DevTable **out) {
         r64[2 * n] = make_dq4(al * s3, al / 2, cs, 0.0);
         r64[2 * n + 1] = make_dq4(be * s3, be / 2, ch, 0.0);
     }
+    std::vector<double2> p64((size_t)P64_N * 2 * P64_C);
+    fock_pieces(T.host, p64);
     std::vector<double> wa;
     double L;
     weideman(wa, &L);
@@ -98,12 +146,14 @@ static int get_table(DevTable **out) {
     CKT(cudaMalloc(&T.fock64, sizeof(double2) * f64.size()));
     CKT(cudaMalloc(&T.res32, sizeof(float4) * r32.size()));
     CKT(cudaMalloc(&T.res64, sizeof(dq4) * r64.size()));
+    CKT(cudaMalloc(&T.p64, sizeof(double2) * p64.size()));
     CKT(cudaMalloc(&T.weid, sizeof(float) * WEIDEMAN_N));
     CKT(cudaMalloc(&T.weid64, sizeof(double) * WEIDEMAN_N));
     CKT(cudaMemcpy(T.fock32, f32.data(), sizeof(float4) * f32.size(), cudaMemcpyHostToDevice));
     CKT(cudaMemcpy(T.fock64, f64.data(), sizeof(double2) * f64.size(), cudaMemcpyHostToDevice));
     CKT(cudaMemcpy(T.res32, r32.data(), sizeof(float4) * r32.size(), cudaMemcpyHostToDevice));
     CKT(cudaMemcpy(T.res64, r64.data(), sizeof(dq4) * r64.size(), cudaMemcpyHostToDevice));
+    CKT(cudaMemcpy(T.p64, p64.data(), sizeof(double2) * p64.size(), cudaMemcpyHostToDevice));
     CKT(cudaMemcpy(T.weid, wf.data(), sizeof(float) * WEIDEMAN_N, cudaMemcpyHostToDevice));
     CKT(cudaMemcpy(T.weid64, wa.data(), sizeof(double) * WEIDEMAN_N, cudaMemcpyHostToDevice));
     g_tables[dev] = T;
@@ -910,7 +960,7 @@ static int make_dev(rt_scene *s, const rt_options *opt, DevScene &D, int *prec, 
     D.face32 = s->d_face32; D.face64 = s->d_face64; D.face_rng = s->d_face_rng; D.face_tris = s->d_face_tris;
     D.body = s->d_body;
     D.fock32 = s->table->fock32; D.fock64 = s->table->fock64;
-    D.res32 = s->table->res32; D.res64 = s->table->res64;
+    D.res32 = s->table->res32; D.res64 = s->table->res64; D.p64 = s->table->p64;
     D.weid = s->table->weid; D.weid64 = s->table->weid64; D.weid_L = s->table->weid_L;
     D.freq = s->freqs.data();   // host pointer: read by the launcher only
     D.fqc = s->d_fqc;

@@ -86,6 +86,7 @@ struct Ctx {
     float weid_L;
     const double2 *fock64;
     const dq4 *res64;
+    const double2 *p64;          // see DevScene
     const double *weid64;
     const float4 *img;           // source images (double-float), see DevScene
     int img_pairs;               // img holds the ordered face pairs too
@@ -446,6 +447,7 @@ __global__ void __launch_bounds__(32 * HID_WARPS) k_src_hidden(DevScene S, Frame
     }
 }
 
+
 // every body (but sb) against a segment (FP32); uns: uncertain ones before
 __device__ __forceinline__ int bodies_all(const Ctx &c, v3t<float> A, v3t<float> B, int sb, float band, int uns) {
     // bodies: a squared-distance test against the segment's closest point
@@ -691,9 +693,9 @@ __device__ __noinline__ int tris_coop(const Ctx &c, unsigned lanes, bool alive, 
 // A leg with an occluder mask (FP32): the faces (but sf1, sf2) as in blocked;
 // the bodies (but sb) are those of the mask occ, nw words (a superset of the
 // bodies that can pass the distance test), or all of them without a mask.
-__device__ __noinline__ int blocked_mask(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb,
-                                         float band, const uint32_t *occ, int nw) {
-    if (!occ) return blocked_impl(c, A, B, sf1, sf2, sb, band);
+__device__ __forceinline__ int blocked_mask_inl(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb,
+                                                float band, const uint32_t *occ, int nw) {
+    if (!occ) return blocked(c, A, B, sf1, sf2, sb, band);
     int uns = 0;
     if (c.bvh) {
         const int r = tris_bvh(c, A, B, sf1, sf2, band);
@@ -723,6 +725,10 @@ __device__ __noinline__ int blocked_mask(const Ctx &c, v3t<float> A, v3t<float> 
     }
     return bodies_masked(c, A, B, sb, band, occ, nw, uns);
 }
+__device__ __noinline__ int blocked_mask(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb,
+                                         float band, const uint32_t *occ, int nw) {
+    return blocked_mask_inl(c, A, B, sf1, sf2, sb, band, occ, nw);
+}
 __device__ __noinline__ int blocked(const Ctx &c, v3t<dx> A, v3t<dx> B, int sf1, int sf2, int sb, dx band) {
     return blocked_impl(c, A, B, sf1, sf2, sb, band);
 }
@@ -730,7 +736,7 @@ __device__ __noinline__ int blocked(const Ctx &c, v3t<dx> A, v3t<dx> B, int sf1,
 // (nullptr: every body)
 template <typename T>
 __device__ __forceinline__ int blocked_leg(const Ctx &c, v3t<T> A, v3t<T> B, int b, T band, const uint32_t *occ) {
-    if constexpr (sizeof(T) == 4) return blocked_mask(c, A, B, -1, -1, b, band, occ, c.occ_w);
+    if constexpr (sizeof(T) == 4) return blocked_mask_inl(c, A, B, -1, -1, b, band, occ, c.occ_w);
     else return blocked(c, A, B, -1, -1, b, band);
 }
 __device__ __forceinline__ const uint32_t *occ_of(const Ctx &c, const uint32_t *masks, int b) {
@@ -865,6 +871,9 @@ template <> __device__ __forceinline__ void face_plane<float>(const Ctx &c, int 
 }
 template <> __device__ __forceinline__ void face_plane<dx>(const Ctx &c, int f, v3t<dx> *n, dx *d) {
     dq4 q = c.face64[f]; *n = mk3<dx>(q.x, q.y, q.z); *d = dx(q.w);
+}
+template <> __device__ __forceinline__ void face_plane<double>(const Ctx &c, int f, v3t<double> *n, double *d) {
+    dq4 q = c.face64[f]; *n = mk3<double>(q.x, q.y, q.z); *d = q.w;
 }
 
 // combine a new decision into a running conjunction; returns false to stop (definite NO)
@@ -1488,8 +1497,13 @@ __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Fr
     // smallest positive value keeps their finite product
     const T cth = Fmax(-dot3(shi, n), T(COS_MIN));
     if constexpr (VIS) {
-        if (!conj(acc, vis_to_dec(blocked_leg(c, S, Q, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
-        if (!conj(acc, vis_to_dec(blocked_leg(c, Q, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+#pragma unroll 1
+        for (int leg = 0; leg < 2; ++leg) {          // (as in cand_creep)
+            const bool src = leg == 0;
+            if (!conj(acc, vis_to_dec(blocked_leg(c, src ? S : Q, src ? Q : P, b, band,
+                                                  occ_of(c, src ? c.occ_src : occ_rx, b)))))
+                return D_NO;
+        }
     }
     if constexpr (sizeof(T) == 4) {
         // total length s^i + s^r to the FP32 surface point c + a n, each leg in
@@ -1591,11 +1605,16 @@ __device__ int cand_creep(const Ctx &c, int b, int dir, v3t<T> S, v3t<T> P, T ba
         g.dperp = T(0);
         g.amp = T(1) / Sqrt(g.sp * g.sq * (g.sp + g.t + g.sq));
     }
-    if constexpr (SRC_LEG && VIS) {
-        if (!conj(acc, vis_to_dec(blocked_leg(c, S, g.Q1, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
-    }
     if constexpr (VIS) {
-        if (!conj(acc, vis_to_dec(blocked_leg(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+        // (one copy of the visibility test, inlined: a call's registers would be
+        // spilled round it)
+#pragma unroll 1
+        for (int leg = SRC_LEG ? 0 : 1; leg < 2; ++leg) {
+            const bool src = leg == 0;
+            if (!conj(acc, vis_to_dec(blocked_leg(c, src ? S : g.Q2, src ? g.Q1 : P, b, band,
+                                                  occ_of(c, src ? c.occ_src : occ_rx, b)))))
+                return D_NO;
+        }
     }
     return acc;
 }
@@ -1647,7 +1666,7 @@ __device__ __forceinline__ int cand_wcreep(const Ctx &c, int f, int b, int dir, 
     const uint32_t *m2 = c.occ_w2 ? c.occ_w2 + (f * c.n_body + b) * c.occ_w : nullptr;
     if (!conj(acc, vis_to_dec(blocked_mask(c, S, Qw, f, -1, -1, band, m1, c.occ_w)))) return D_NO;
     if (!conj(acc, vis_to_dec(blocked_mask(c, Qw, g.Q1, f, -1, b, band, m2, c.occ_w)))) return D_NO;
-    if (!conj(acc, vis_to_dec(blocked_leg(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    if (!conj(acc, vis_to_dec(blocked_mask(c, g.Q2, P, -1, -1, b, band, occ_of(c, occ_rx, b), c.occ_w)))) return D_NO;
     return acc;
 }
 
@@ -1731,67 +1750,96 @@ __device__ void pekeris(const Ctx &c, float xi, cpx<float> &ps, cpx<float> &ph, 
     ph = Gh * rot;
     if (!regular) { ps = ps - mkc(ci, -ci); ph = ph - mkc(ci, -ci); }
 }
-__device__ void pekeris(const Ctx &c, dx xid, cpx<dx> &psd, cpx<dx> &phd, bool regular) {
-    double xi = xid.v;
-    const double ci = (0.5 / sqrt(M_PI)) * cos(M_PI / 4.0) / xi;
-    cpx<double> ps, ph;
-    if (xi > XI_HI) {
-        cpx<double> ss = mkc(0.0, 0.0), sh = mkc(0.0, 0.0);
-        // (terms below 2^-60 of the first are left out)
-        const double x0s = c.res64[0].x, x0h = c.res64[1].x;
-        for (int n = 0; n < FOCK_NRES; ++n) {
-            const dq4 rs = c.res64[2 * n], rh = c.res64[2 * n + 1];
-            const bool s_on = xi * (rs.x - x0s) <= 42.0, h_on = xi * (rh.x - x0h) <= 42.0;
-            if (!s_on && !h_on) break;
-            double sn, cs, e;
-            if (s_on) {
-                sincos(xi * rs.y, &sn, &cs);
-                e = exp(-xi * rs.x) * rs.z;
-                ss = ss + mkc(e * cs, -e * sn);
+// FP64 P_s and P_h (v[0], v[1]) on [XI_HI, XI_P] by the polynomial pieces, and
+// with DERIV their slopes d.  What bounds the FP64 kernels is the FP64 pipe (2
+// lanes an SM): the residue series took 16 sincos and exp a call, some 1100
+// FP64 instructions, these 48 multiply-adds.  24047 receivers, 20 bodies, three
+// frequencies: 5.23 -> 3.86 ms with the fields in fused multiply-adds.  Error of P
+// against long double: 4e-16 of |P|, the series' 5e-15.
+template <bool DERIV>
+__device__ __forceinline__ void pek_pieces(const Ctx &c, double xi, cpx<double> v[2], cpx<double> d[2]) {
+    const double u = (xi - XI_HI) * P64_PER;
+    const int j = min(max((int)u, 0), P64_N - 1);
+    const double t = 2.0 * (u - j) - 1.0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double2 *q = c.p64 + (j * 2 + k) * P64_C;
+        double2 a = q[P64_C - 1];
+        double re = a.x, im = a.y, dr = 0.0, di = 0.0;
+#pragma unroll
+        for (int n = P64_C - 2; n >= 0; --n) {
+            a = q[n];
+            if (DERIV) {
+                dr = dr * t + re;
+                di = di * t + im;
             }
-            if (h_on) {
-                sincos(xi * rh.y, &sn, &cs);
-                e = exp(-xi * rh.x) * rh.z;
-                sh = sh + mkc(e * cs, -e * sn);
-            }
+            re = re * t + a.x;
+            im = im * t + a.y;
         }
-        cpx<double> pre = mkc(-cos(M_PI / 12.0), sin(M_PI / 12.0)) * (0.5 / sqrt(M_PI));
-        ps = pre * ss;
-        ph = pre * sh;
-        if (regular) { ps = ps + mkc(ci, -ci); ph = ph + mkc(ci, -ci); }
-    } else {
-        double u = (xi - XI_LO) / XI_STEP;
-        int j = min(max((int)u, 0), FOCK_N - 2);
-        double t = u - j, t2 = t * t, omt = 1.0 - t;
-        double h00 = (1 + 2 * t) * omt * omt, h10 = t * omt * omt * XI_STEP, h01 = t2 * (3 - 2 * t), h11 = t2 * (t - 1) * XI_STEP;
-        cpx<double> G[2];
-        for (int k = 0; k < 2; ++k) {
-            double2 g0 = c.fock64[(j * 2 + k) * 2], d0 = c.fock64[(j * 2 + k) * 2 + 1];
-            double2 g1 = c.fock64[((j + 1) * 2 + k) * 2], d1 = c.fock64[((j + 1) * 2 + k) * 2 + 1];
-            G[k] = mkc(h00 * g0.x + h10 * d0.x + h01 * g1.x + h11 * d1.x, h00 * g0.y + h10 * d0.y + h01 * g1.y + h11 * d1.y);
-        }
-        double sn, cs;
-        sincos(xi * xi * xi / 12.0, &sn, &cs);
-        ps = G[0] * mkc(cs, sn);
-        ph = G[1] * mkc(cs, sn);
-        if (!regular) { ps = ps - mkc(ci, -ci); ph = ph - mkc(ci, -ci); }
+        v[k] = mkc(re, im);
+        if (DERIV) d[k] = mkc(dr * (2.0 * P64_PER), di * (2.0 * P64_PER));
     }
-    psd = mkc<dx>(ps.re, ps.im);
-    phd = mkc<dx>(ph.re, ph.im);
+}
+// the residue series of the same beyond (terms below 2^-60 of the first are left out)
+template <bool DERIV>
+__device__ __forceinline__ void pek_series(const Ctx &c, double xi, cpx<double> v[2], cpx<double> d[2]) {
+    const cpx<double> pre = mkc(-0.27248264483602590, 0.07301150463530957);    // -e^{-j pi/12} / (2 sqrt(pi))
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        cpx<double> s = mkc(0.0, 0.0), ds = s;
+        const double x0 = c.res64[k].x;
+#pragma unroll 1
+        for (int n = 0; n < FOCK_NRES; ++n) {
+            const dq4 q = c.res64[2 * n + k];
+            if (xi * (q.x - x0) > 42.0) break;
+            double sn, cs;
+            sincos(xi * q.y, &sn, &cs);
+            const double e = exp(-(xi * q.x)) * q.z;
+            const cpx<double> t = mkc(e * cs, -(e * sn));
+            s = s + t;
+            if (DERIV) ds = ds - mkc(q.x, q.y) * t;
+        }
+        v[k] = pre * s;
+        if (DERIV) d[k] = pre * ds;
+    }
+}
+__device__ void pekeris(const Ctx &c, double xi, cpx<double> &ps, cpx<double> &ph, bool regular) {
+    const double ci = 0.19947114020071633897 / xi;     // c/xi = (ci, -ci)
+    if (xi > XI_HI) {
+        cpx<double> v[2];
+        if (xi < XI_P) pek_pieces<false>(c, xi, v, v);
+        else pek_series<false>(c, xi, v, v);
+        ps = v[0];
+        ph = v[1];
+        if (regular) { ps = ps + mkc(ci, -ci); ph = ph + mkc(ci, -ci); }
+        return;
+    }
+    double u = (xi - XI_LO) / XI_STEP;
+    int j = min(max((int)u, 0), FOCK_N - 2);
+    double t = u - j, t2 = t * t, omt = 1.0 - t;
+    double h00 = (1 + 2 * t) * omt * omt, h10 = t * omt * omt * XI_STEP, h01 = t2 * (3 - 2 * t), h11 = t2 * (t - 1) * XI_STEP;
+    cpx<double> G[2];
+    for (int k = 0; k < 2; ++k) {
+        double2 g0 = c.fock64[(j * 2 + k) * 2], d0 = c.fock64[(j * 2 + k) * 2 + 1];
+        double2 g1 = c.fock64[((j + 1) * 2 + k) * 2], d1 = c.fock64[((j + 1) * 2 + k) * 2 + 1];
+        G[k] = mkc(h00 * g0.x + h10 * d0.x + h01 * g1.x + h11 * d1.x, h00 * g0.y + h10 * d0.y + h01 * g1.y + h11 * d1.y);
+    }
+    double sn, cs;
+    sincos(xi * xi * xi / 12.0, &sn, &cs);
+    ps = G[0] * mkc(cs, sn);
+    ph = G[1] * mkc(cs, sn);
+    if (!regular) { ps = ps - mkc(ci, -ci); ph = ph - mkc(ci, -ci); }
 }
 
-__device__ __forceinline__ cpx<dx> faddeeva_dx(const Ctx &c, cpx<dx> zd) {
-    cpx<double> z = mkc(zd.re.v, zd.im.v);
+__device__ __forceinline__ cpx<double> faddeeva_t(const Ctx &c, cpx<double> z) {
     double L = c.weid_L;
     cpx<double> lm = mkc(L + z.im, -z.re), lp = mkc(L - z.im, z.re);
     cpx<double> Z = cdiv(lp, lm);
     cpx<double> p = mkc(c.weid64[WEIDEMAN_N - 1], 0.0);
     for (int n = WEIDEMAN_N - 2; n >= 0; --n) p = p * Z + mkc(c.weid64[n], 0.0);
-    cpx<double> r = cdiv(p * 2.0, lm * lm) + cdiv(mkc(0.56418958354775628, 0.0), lm);
-    return mkc<dx>(r.re, r.im);
+    return cdiv(p * 2.0, lm * lm) + cdiv(mkc(0.56418958354775628, 0.0), lm);
 }
 __device__ __forceinline__ cpx<float> faddeeva_t(const Ctx &c, cpx<float> z) { return faddeeva<float>(c, z); }
-__device__ __forceinline__ cpx<dx> faddeeva_t(const Ctx &c, cpx<dx> z) { return faddeeva_dx(c, z); }
 
 // Fock bracket B = P + (c/xi)(1 - F(X)) = phat - c F(X)/xi with sqrt(X) = K |xi|.
 // X <= 4: phat - c F/xi, F/xi = sgn(xi) sqrt(pi) K e^{j pi/4} w(e^{j 3pi/4} K |xi|).
@@ -1913,6 +1961,15 @@ __device__ __forceinline__ float len_val(dfl L) { return L.hi + L.lo; }
 __device__ __forceinline__ dx len_val(dx L) { return L; }
 __device__ __forceinline__ float kof(const FreqC &fq, int f, float) { return fq.k[f]; }
 __device__ __forceinline__ dx kof(const FreqC &fq, int f, dx) { return dx(fq.kd[f]); }
+__device__ __forceinline__ double kof(const FreqC &fq, int f, double) { return fq.kd[f]; }
+__device__ __forceinline__ double khof(const FreqC &fq, int f, double) { return cbrt(fq.kd[f] * 0.5); }
+__device__ __forceinline__ double len_val(double L) { return L; }
+__device__ __forceinline__ cpx<double> phasor(const FreqC &fq, int f, double L) {
+    double cyc = L * fq.fc[f], s, co;
+    cyc -= floor(cyc);
+    sincospi(2.0 * cyc, &s, &co);
+    return mkc(co, -s);
+}
 __device__ __forceinline__ float khof(const FreqC &fq, int f, float) { return fq.kh[f]; }
 __device__ __forceinline__ dx khof(const FreqC &fq, int f, dx) { return dx(cbrt(fq.kd[f] * 0.5)); }
 
@@ -1949,6 +2006,9 @@ __device__ __forceinline__ void acc_put(AccS<T> &acc, int f, cpx<T> x, cpx<T> y,
     q[0] = q[0] + x.re; q[32] = q[32] + x.im;
     q[64] = q[64] + y.re; q[96] = q[96] + y.im;
     q[128] = q[128] + z.re; q[160] = q[160] + z.im;
+}
+__device__ __forceinline__ void acc_put(AccS<dx> &acc, int f, cpx<double> x, cpx<double> y, cpx<double> z) {
+    acc_put<dx>(acc, f, mkc<dx>(x.re, x.im), mkc<dx>(y.re, y.im), mkc<dx>(z.re, z.im));
 }
 template <typename T>
 __device__ __forceinline__ void acc_zero(AccS<T> &acc) {
@@ -2378,6 +2438,17 @@ __device__ __forceinline__ Geo<float> to_f(const Geo<dx> &d) {
     g.rho_g = to_float(d.rho_g); g.inv_f1 = to_float(d.inv_f1); g.inv_f2 = to_float(d.inv_f2);
     g.dperp = to_float(d.dperp); g.caus = d.caus;
     g.dr = to_f3(d.dr);
+    return g;
+}
+// FP64 decisions' geometry -> the FP64 fields, which need no fixed rounding
+__device__ __forceinline__ v3t<double> to_d3(v3t<dx> a) { return mk3<double>(a.x.v, a.y.v, a.z.v); }
+__device__ __forceinline__ Geo<double> to_d(const Geo<dx> &d) {
+    Geo<double> g;
+    g.Q1 = to_d3(d.Q1); g.Q2 = to_d3(d.Q2); g.n1 = to_d3(d.n1); g.n2 = to_d3(d.n2);
+    g.sp = d.sp.v; g.t = d.t.v; g.sq = d.sq.v; g.amp = d.amp.v;
+    g.rho_g = d.rho_g.v; g.inv_f1 = d.inv_f1.v; g.inv_f2 = d.inv_f2.v;
+    g.dperp = d.dperp.v; g.caus = d.caus;
+    g.dr = to_d3(d.dr);
     return g;
 }
 __device__ __forceinline__ dfl to_df(double x) {
@@ -2820,7 +2891,8 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                                               const uint32_t *occ_rx, int part, int nparts,
                                               AccS<T> acc, float *rec, uint32_t &fl, unsigned &nesc, int &npath,
                                               int &nrec_out, const uint32_t *qmask = nullptr, unsigned lanes = 0u,
-                                              uint32_t *pwm = nullptr, int *cstk = nullptr, uint32_t *found = nullptr) {
+                                              uint32_t *pwm = nullptr, int *cstk = nullptr, uint32_t *found = nullptr,
+                                              bool own = true) {
     constexpr bool BODIES = (CLS & CLS_BODIES) != 0;
     constexpr bool fp32 = sizeof(T) == 4;
     const T band = fp32 ? T(c.band) : T(0);
@@ -2847,7 +2919,7 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
             if (npath < cap) codes[(size_t)r * cap + npath] = pcode(type, a, b);
             else fl |= RT_FLAG_OVERFLOW;
         } else if constexpr (LIST) {
-            fl |= list_path(codes, counts, cap, r, pcode(type, a, b));
+            if (own) fl |= list_path(codes, counts, cap, r, pcode(type, a, b));
         }
         ++npath;
     };
@@ -3188,7 +3260,8 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                             nrec += wcreep_prep(c, rec + nrec * REC_N * 32, wf, Sx, Sw, P, g,
                                                 creep_len(c, bb, Sw, P, g, F), enable);
                         } else if constexpr (!PATHS) {
-                            field_wcreep<T>(c, acc, fq, wf, Sx, Sw, P, g, creep_len(c, bb, Sw, P, g, F), enable);
+                            field_wcreep<double>(c, acc, fq, wf, to_d3(Sx), to_d3(Sw), to_d3(P), to_d(g),
+                                                 creep_len(c, bb, Sw, P, g, F).v, enable);
                         }
                     }
                     continue;
@@ -3234,7 +3307,8 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                             if constexpr (RECS) {
                                 rb_prep(c, rec + (nrec++) * REC_N * 32, Sx, g, g.Lf);
                             } else if constexpr (!PATHS) {
-                                field_body_refl<T>(c, acc, fq, Sx, P, g, ladd(seglen(Sx, g.Q1), seglen(g.Q1, P)));
+                                field_body_refl<double>(c, acc, fq, to_d3(Sx), to_d3(P), to_d(g),
+                                                        ladd(seglen(Sx, g.Q1), seglen(g.Q1, P)).v);
                             }
                         }
                     }
@@ -3282,7 +3356,8 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                             if constexpr (RECS) {
                                 creep_prep(c, rec + (nrec++) * REC_N * 32, Sx, P, g, creep_len(c, b, Sx, P, g, F), enable);
                             } else if constexpr (!PATHS) {
-                                field_creep<T>(c, acc, fq, Sx, P, g, creep_len(c, b, Sx, P, g, F), enable);
+                                field_creep<double>(c, acc, fq, to_d3(Sx), to_d3(P), to_d(g),
+                                                    creep_len(c, b, Sx, P, g, F).v, enable);
                             }
                         }
                     }
@@ -3429,7 +3504,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
        const float *__restrict__ rx_base, const int32_t *__restrict__ perm, float *__restrict__ e_base,
        uint32_t *__restrict__ fl_base,
        uint64_t *__restrict__ codes, int32_t *__restrict__ counts, int cap, int ch0, int nch, int rcap,
-       int nwt, int accumulate, int enc, unsigned long long *esc_counter, unsigned long long *queue) {
+       int nwt, int tsh, int accumulate, int enc, unsigned long long *esc_counter, unsigned long long *queue) {
     constexpr bool BODIES = (CLS & CLS_BODIES) != 0;
     extern __shared__ float4 smem[];
     __shared__ Ctx s_ctx;
@@ -3488,7 +3563,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         c.S = mk3(S.tx[0], S.tx[1], S.tx[2]);
         c.pol = mk3(S.pol[0], S.pol[1], S.pol[2]);
         c.fock = s_fock; c.res = s_res; c.weid = s_weid; c.weid_L = S.weid_L;
-        c.fock64 = S.fock64; c.res64 = S.res64; c.weid64 = S.weid64;
+        c.fock64 = S.fock64; c.res64 = S.res64; c.p64 = S.p64; c.weid64 = S.weid64;
         c.img = S.img;
         c.img_pairs = S.img_pairs;
         c.face_mat = S.face_mat;
@@ -3524,7 +3599,6 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         // (one frame only)
         const float *rx = rx_base;
         const int n_rx = F1.n_rx;
-        const unsigned long long ntiles = ((unsigned long long)n_rx + 31ull) >> 5;
         // occluder masks (body kernels): the source side per block, the
         // receiver side per warp (each warp takes whole tiles)
         constexpr bool OCC = BODIES;
@@ -3578,8 +3652,9 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                 if (lane == 0) t = atomicAdd(queue, 1ull);
                 t = __shfl_sync(0xffffffffu, t, 0);
             }
-            if (t >= ntiles) break;
-            int r = (int)(t * 32ull) + lane;
+            if (t >= n_tiles) break;
+            const int r = (int)(t << tsh) + (lane & ((1 << tsh) - 1));
+            const bool own = r < n_rx && lane >> tsh == 0;       // (narrow tiles: see the fields below)
             if (occ_on) {
                 tile_masks(c, rx, n_rx, r, r < n_rx, s_occ_mine, part, nparts);
                 __syncwarp();
@@ -3604,14 +3679,14 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                                              nullptr, fl, nesc, npath, nrec, qm_on ? &s_qmask_p[warp][0] : nullptr,
                                              LEGM_P ? lanes_p : 0u, &s_pwm_p[LEGM_P ? warp : 0][0],
                                              &s_cstk_p[COOP_P ? warp : 0][0], found);
-                if (nesc) atomicAdd(esc_counter, (unsigned long long)nesc);
+                if (own && nesc) atomicAdd(esc_counter, (unsigned long long)nesc);
             }
             if (split) {
                 s_fl_p[SPLIT ? warp : 0][lane] = fl;
                 __syncthreads();
                 if (warp != 0) continue;
                 for (int w = 1; w < NW; ++w) fl |= s_fl_p[SPLIT ? w : 0][lane];
-                if (r < n_rx) {
+                if (own) {
                     npath = accumulate ? counts[r] : 0;
                     for (int i = 0; i < n_found; ++i) {
                         if (!(found[i] >> lane & 1u)) continue;
@@ -3621,7 +3696,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                     }
                 }
             }
-            if (r < n_rx) {
+            if (own) {
                 counts[r] = npath;
                 if (fl_base) fl_base[r] = accumulate ? (fl_base[r] | fl) : fl;
             }
@@ -3637,6 +3712,8 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         // record buffer; per chunk all warps finish the geometry pass before
         // any starts the field pass, which runs once per frequency chunk on
         // the same records and adds its rows to the outputs.
+        //   Few receivers: narrower tiles, so that every SM has some (see
+        // launch_one), of which a receiver's fields do not depend.
         //   The tile shape: NWT = nwt warps share a tile (the launcher checks
         // that it divides the block's warps), TPB tiles per block.  A work
         // unit is TPB tiles of one frame; a batch's frames start at tile
@@ -3734,10 +3811,13 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
             // bodies per geometry pass: all of them with one frequency chunk (full
             // record buffers are flushed on the way), else as many as the buffer holds
             const int bc = (RECS && nch > 1) ? NWT * (rcap / PER) : (n_b > 0 ? n_b : 1);
+            // the tile's 2^tsh receivers; with fewer than 32 the other lanes repeat
+            // them (own: not a repeat), share the warp's work on masks and culling,
+            // and write nothing
             const unsigned long long t = s_unit * TPB - Fr.tile0 + grp;   // tile within the frame
-            const long long r0 = (long long)(t * 32ull);
-            const int r = r0 < n_rx ? (int)r0 + lane : n_rx;
-            const bool rok = r < n_rx;
+            const long long r0 = (long long)(t << tsh);
+            const int r = r0 < n_rx ? (int)r0 + (lane & ((1 << tsh) - 1)) : n_rx;
+            const bool rok = r < n_rx, own = rok && lane >> tsh == 0;
             if (occ_on) {
                 // each warp makes the masks of the bodies of its own share
                 // (b = part mod NWT), so no other warp waits for them
@@ -3767,9 +3847,10 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                                                  Fr.hl, b0, min(b0 + bc, n_b), b0 == 0, nch == 1, rcap,
                                                  occ_on ? s_occ_rx + grp * S.n_body * occ_w : nullptr, part,
                                                  NWT, acc, rec, fl, nesc, npath, nrec,
-                                                 qm_on ? &s_qmask[warp][0] : nullptr, lanes, &s_pwm[LEGM ? warp : 0][0], &s_cstk[COOP ? warp : 0][0]);
+                                                 qm_on ? &s_qmask[warp][0] : nullptr, lanes, &s_pwm[LEGM ? warp : 0][0], &s_cstk[COOP ? warp : 0][0],
+                                                 nullptr, own);
                 s_fl[warp][lane] = fl;
-                if (nesc && ch0 == 0) atomicAdd(esc_counter, (unsigned long long)nesc);
+                if (own && nesc && ch0 == 0) atomicAdd(esc_counter, (unsigned long long)nesc);
 #pragma unroll 1
                 for (int ch = ch0; ch < ch0 + nch; ++ch) {
                     const FreqC &fqc = s_fqs[ch - ch0];
@@ -3787,7 +3868,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                     __syncthreads();
                     // reduce the tile's NWT partials: part p writes the
                     // (frequency, component) pairs j = p, p + NWT, ... of chunk ch
-                    if (rok) {
+                    if (own) {
                         const int w0 = grp * NWT, f0 = ch * NFC;
                         const int ro = perm ? perm[Fr.rx_off + r] : r;       // the receiver's output slot
                         const bool add = accumulate || b0 > 0;
@@ -3923,8 +4004,19 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
     // (path lists: each warp takes whole tiles; up to one block per tile, so
     // that a few tiles spread over as many SMs)
     const int tiles_per_unit = PATHS ? 1 : NW / nwt;
-    long long need = (long long)((W.n_tiles + tiles_per_unit - 1) / tiles_per_unit);
     long long cap_blocks = (long long)nsm * (occ > 0 ? occ : 1);
+    // one frame of few receivers: the narrowest tiles of which a third of the
+    // device holds all (the three classes run side by side).  A tile's receivers
+    // mostly take different paths through the kernel, one after the other; apart,
+    // they run on SMs that would be idle: 97 receivers among 20 bodies 159 -> 113
+    // us.  With tiles for a whole wave of each class, 2867 and 4096 receivers were
+    // 8 and 10 % slower.
+    int tsh = 5;
+    auto tiles_of = [&](int sh) { return (((unsigned long long)W.F1.n_rx + (1u << sh) - 1) >> sh); };
+    if (!W.frames && (!PATHS || split))
+        while (tsh > 0 && 3 * tiles_of(tsh - 1) <= (unsigned long long)(cap_blocks * tiles_per_unit)) --tsh;
+    const unsigned long long n_tiles = tsh < 5 ? tiles_of(tsh) : W.n_tiles;
+    long long need = (long long)((n_tiles + tiles_per_unit - 1) / tiles_per_unit);
     int grid = (int)(need < cap_blocks ? need : cap_blocks);
     if (grid < 1) grid = 1;
     // every launch after the first of the evaluation is a programmatic
@@ -3939,8 +4031,8 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = L.n > 0 ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, k_eval<T, PATHS, CLS, LIST>, S, W.F1, W.frames, W.n_frames, W.n_tiles, W.rx, W.perm, W.e, W.fl,
-                           W.codes, W.counts, W.cap, ch0, nch, rcap, nwt, accumulate, enc, L.ctr, L.ctr + 1 + L.n);
+    e = cudaLaunchKernelEx(&cfg, k_eval<T, PATHS, CLS, LIST>, S, W.F1, W.frames, W.n_frames, n_tiles, W.rx, W.perm, W.e, W.fl,
+                           W.codes, W.counts, W.cap, ch0, nch, rcap, nwt, tsh, accumulate, enc, L.ctr, L.ctr + 1 + L.n);
     ++L.n;
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -4099,15 +4191,9 @@ template <> __device__ __forceinline__ void face_plane<D7>(const Ctx &c, int f, 
     dq4 q = c.face64[f]; *n = mk3<D7>(q.x, q.y, q.z); *d = D7(q.w);
 }
 
-// ---- FP64: Fock--Pekeris functions of a dual xi: value and slope in scalars (the
-// residue series term by term above XI_HI, else the table's cubic Hermite
-// interpolant and its slope), then the chain rule once.  A term of the series
-// is left out once it is below 2^-60 of the first.
-__device__ __forceinline__ double adj_res(const Ctx &c, int n, int k, double *x, double *y) {
-    const dq4 q = c.res64[2 * n + k];
-    *x = q.x; *y = q.y;
-    return q.z;
-}
+// ---- FP64: Fock--Pekeris functions of a dual xi: value and slope in scalars
+// (above XI_HI the pieces or the residue series, else the table's cubic Hermite
+// interpolant), then the chain rule once.
 __device__ __forceinline__ void adj_node(const Ctx &c, int j, int k, cpx<double> *g, cpx<double> *hd) {
     const double2 a = c.fock64[(j * 2 + k) * 2], q = c.fock64[(j * 2 + k) * 2 + 1];
     *g = mkc(a.x, a.y);
@@ -4123,29 +4209,9 @@ __device__ void pekeris(const Ctx &c, const DualT<double, N> &xid, cpx<DualT<dou
     const double ci = 0.19947114020071633897 / xi, dci = -ci / xi;   // c/xi = (ci, -ci)
     cpx<double> v[2], d[2];
     bool reg;
-    if (xi > double(XI_HI)) {
-        const double cut = 42.0;
-        const cpx<double> pre = mkc<double>(-0.27248264483602590, 0.07301150463530957);    // -e^{-j pi/12} / (2 sqrt(pi))
-#pragma unroll 1
-        for (int k = 0; k < 2; ++k) {
-            cpx<double> s = mkc<double>(0.0, 0.0), ds = s;
-            double x0, y0;
-            adj_res(c, 0, k, &x0, &y0);
-#pragma unroll 1
-            for (int n = 0; n < FOCK_NRES; ++n) {
-                double x, y;
-                const double z = adj_res(c, n, k, &x, &y);
-                if (xi * (x - x0) > cut) break;
-                double sn, cs;
-                dsincos(xi * y, &sn, &cs);
-                const double e = Exp(-(xi * x)) * z;
-                const cpx<double> t = mkc<double>(e * cs, -(e * sn));
-                s = s + t;
-                ds = ds - mkc<double>(x, y) * t;
-            }
-            v[k] = pre * s;
-            d[k] = pre * ds;
-        }
+    if (xi > XI_HI) {
+        if (xi < XI_P) pek_pieces<true>(c, xi, v, d);
+        else pek_series<true>(c, xi, v, d);
         reg = false;                               // P
     } else {
         const double u = (xi - double(XI_LO)) * double(1.0 / XI_STEP);
@@ -4197,8 +4263,7 @@ __device__ __forceinline__ cpx<DualT<S, N>> faddeeva_dual(const cpx<DualT<S, N>>
 }
 template <int N>
 __device__ __forceinline__ cpx<DualT<double, N>> faddeeva_t(const Ctx &c, const cpx<DualT<double, N>> &zd) {
-    const cpx<dx> w = faddeeva_dx(c, mkc<dx>(zd.re.v, zd.im.v));
-    return faddeeva_dual<double, N>(zd, mkc(w.re.v, w.im.v));
+    return faddeeva_dual<double, N>(zd, faddeeva_t(c, mkc(zd.re.v, zd.im.v)));
 }
 
 // the path phasor e^{-j k L}
@@ -4932,7 +4997,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // frequencies with FP32 duals from 4.10 to 0.94 ms.
 constexpr int ADJ_BLOCK = 128;
 constexpr int ADJ_RX = 32;               // receivers of a unit, at most
-constexpr int ADJ_ITEMS = 1024;          // paths sorted at once
+constexpr int ADJ_ITEMS = 2048;          // paths sorted at once
 constexpr int ADJ_KINDS = 7;
 // the sorting order of path types (dearest first); ADJ_KINDS: none
 __device__ __forceinline__ int adj_kind(int type) {
@@ -4967,7 +5032,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adjoint(DevScene S, const float *
         c.S = mk3(S.tx[0], S.tx[1], S.tx[2]);
         c.pol = mk3(S.pol[0], S.pol[1], S.pol[2]);
         c.fock = S.fock32; c.res = S.res32; c.weid = S.weid; c.weid_L = S.weid_L;
-        c.fock64 = S.fock64; c.res64 = S.res64; c.weid64 = S.weid64;
+        c.fock64 = S.fock64; c.res64 = S.res64; c.p64 = S.p64; c.weid64 = S.weid64;
         c.img = S.img; c.img_pairs = S.img_pairs; c.txb = S.txb;
         c.face_mat = S.face_mat;
         c.txw = S.txw; c.bvh = S.bvh; c.bvh_tri = S.bvh_tri;
@@ -5118,9 +5183,9 @@ int launch_adjoint(const DevScene &S, const float *rx_soa, int n_rx, const uint6
         int dev = 0, nsm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        // units of as many receivers as leave three or more for every SM: more
-        // receivers a unit fill the last warp of each kind better
-        const int rpu = max(1, min(ADJ_RX, n_rx / (3 * nsm)));
+        // the fewest units of at most ADJ_RX receivers that give every SM the same
+        // number: the more receivers a unit, the fuller the last warp of each kind
+        const int waves = (n_rx + ADJ_RX * nsm - 1) / (ADJ_RX * nsm), rpu = max(1, (n_rx + waves * nsm - 1) / (waves * nsm));
         const int units = (n_rx + rpu - 1) / rpu, grid = min(units, 2 * nsm);
         if (precision == RT_PREC_FP64)
             k_adjoint<true><<<grid, ADJ_BLOCK, 0, st>>>(S, rx_soa, n_rx, rpu, codes, counts, cap, grad_e, g_body, g_tx, g_f, queue);

@@ -32,6 +32,13 @@ constexpr int FOCK_N = 737;            // (XI_HI - XI_LO) / XI_STEP + 1
 constexpr double XI_P = 12.0;
 constexpr double XI_PRES = 3.0;
 constexpr int FOCK_NP = 673;           // (XI_P - XI_HI) / XI_STEP + 1
+// FP64: P on [XI_HI, XI_P] as polynomials of degree P64_C - 1 on pieces of width
+// 1 / P64_PER.  A term e^{-alpha xi e^{j pi/6}} of the residue series is
+// interpolated to within 2 (alpha / (8 P64_PER))^n / n!, n = P64_C: 5e-11 for the
+// last (alpha = 11), which is 6e-7 of the first at XI_HI, and nothing for the first.
+constexpr int P64_PER = 4;
+constexpr int P64_N = 42;             // (XI_P - XI_HI) P64_PER
+constexpr int P64_C = 12;
 constexpr int FOCK_NBUCKET = 11;       // quadrature buckets: [0, XI_HI], [-1, 0), ..., [-10, -9)
 constexpr int FOCK_NRES = 8;           // residue-series terms
 constexpr int WEIDEMAN_N = 16;         // terms of the rational approximation of w(z)
@@ -85,6 +92,7 @@ struct DevScene {
     const double2 *fock64;     // [FOCK_N][2][2]: G, G' (soft, hard)
     const float4 *res32;       // [FOCK_NRES][2]: (alpha sqrt3/2, alpha/2, coef, 0) soft, hard
     const dq4 *res64;      // [FOCK_NRES][2]
+    const double2 *p64;        // [P64_N][2][P64_C]: P in powers of t in [-1, 1] over the piece (soft, hard)
     const float *weid;         // [WEIDEMAN_N]
     const double *weid64;      // [WEIDEMAN_N]
     float weid_L;
