@@ -39,7 +39,20 @@
 #include "dual.cuh"
 #include "internal.h"
 
+// This file is compiled twice: as it is, and by eval_small.cu with CREEP_SMALL
+// for the scenes without a BVH and without a candidate list, whose kernels then
+// carry none of the large scenes' code: they wait for instructions as long as for
+// anything else.  65536 receivers, 20 bodies, three frequencies 1.21 -> 1.04 ms,
+// 521473 receivers, 7 bodies 4.08 -> 3.84 ms, wall -> creeping paths of 16637
+// receivers 3.53 -> 3.17 ms.
+#ifdef CREEP_SMALL
 namespace creep {
+namespace small {
+constexpr bool LARGE = false;
+#else
+namespace creep {
+constexpr bool LARGE = true;
+#endif
 
 #define EPS_TRIM 1e-6
 enum { D_NO = 0, D_YES = 1, D_UNSURE = 2 };
@@ -76,7 +89,11 @@ struct Ctx {
     int n_tri, n_face, n_body;
     // the bodies that get candidates: all n_body of them, or (scenes with a
     // BVH, body classes) the n_cand_body of blist that the source may see
+#ifdef CREEP_SMALL
+    static constexpr const uint16_t *blist = nullptr;
+#else
     const uint16_t *blist;
+#endif
     int n_cand_body;
     float band;
     v3t<float> S, pol;
@@ -92,10 +109,16 @@ struct Ctx {
     int img_pairs;               // img holds the ordered face pairs too
     const float4 *txb;           // [n_body][2] source-side body frame, see DevScene
     const float4 *txw;           // [n_face][n_body][2] the same for each face's source image (or nullptr)
+#ifdef CREEP_SMALL
+    static constexpr const float4 *bvh = nullptr, *bvh_top = nullptr;
+    static constexpr const int *bvh_tri = nullptr;
+    static constexpr int bvh_top_n = 0;
+#else
     const float4 *bvh;           // triangle BVH, see DevScene (nullptr: every triangle is tested)
     const int *bvh_tri;
     const float4 *bvh_top;       // its first bvh_top_n nodes (the top levels) staged in shared memory
     int bvh_top_n;
+#endif
     const int4 *cand;            // candidate face sequences, see DevScene (n_cand = 0: every face and pair)
     const float4 *cimg;
     int n_cand;
@@ -391,6 +414,7 @@ __device__ __noinline__ bool occludes(const Ctx &c, int t, const Box &X, const B
 // alone is some 100 us of dependent loads, ahead of everything else.  0.07 ms
 // for 110 bodies among 193 572 triangles; with most of those bodies out, the
 // body kernels of 1 M receivers went from 31 and 32 ms to 2.2 and 1.7 ms.
+#ifndef CREEP_SMALL
 constexpr int HID_WARPS = 4;
 constexpr int HID_STACK = 1088;
 __global__ void __launch_bounds__(32 * HID_WARPS) k_src_hidden(DevScene S, FrameDev F1, const FrameDev *frames) {
@@ -447,6 +471,7 @@ __global__ void __launch_bounds__(32 * HID_WARPS) k_src_hidden(DevScene S, Frame
     }
 }
 
+#endif
 
 // every body (but sb) against a segment (FP32); uns: uncertain ones before
 __device__ __forceinline__ int bodies_all(const Ctx &c, v3t<float> A, v3t<float> B, int sb, float band, int uns) {
@@ -3522,7 +3547,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
     float4 *s_tri = s_body + (body_sm ? 2 * S.n_body : 0);   // n_tri * 3 (if staged)
     float4 *s_aux = s_tri + (tri_sm ? 3 * S.n_tri : 0);      // n_tri * 3 (if staged)
     float4 *s_txb = s_aux + (tri_sm ? 3 * S.n_tri : 0);      // n_body * 2 (if staged)
-    const int n_top = S.bvh ? min(S.bvh_nodes, BVH_TOP_NODES) : 0;
+    const int n_top = LARGE && S.bvh ? min(S.bvh_nodes, BVH_TOP_NODES) : 0;
     float4 *s_bvh = s_txb + (body_sm ? 2 * S.n_body : 0);    // n_top * 2: the BVH's top treelet
     float *s_weid = (float *)(s_bvh + 2 * n_top);
     float *s_rec = s_weid + WEIDEMAN_N;                      // path records (FP32 fields of the body classes)
@@ -3572,8 +3597,10 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         c.occ_w = 0;
         c.enc = enc;
         c.txw = frames ? nullptr : S.txw;
+#ifndef CREEP_SMALL
         c.bvh = S.bvh; c.bvh_tri = S.bvh_tri;
         c.bvh_top = s_bvh; c.bvh_top_n = n_top;
+#endif
         c.cand = S.cand; c.cimg = S.cimg;
         c.n_cand = S.cand ? (S.n_cand_dev ? *S.n_cand_dev : S.n_cand) : 0;
     }
@@ -3587,10 +3614,12 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int NW = blk_of(CLS, sizeof(T) == 4) / 32;
     // scenes with a BVH: the bodies not hidden from the source (body_list)
-    constexpr bool BLIST = BODIES && CLS != CLS_WCREEP;
+    constexpr bool BLIST = LARGE && BODIES && CLS != CLS_WCREEP;
     __shared__ uint16_t s_blist[BLIST ? RT_MAX_BODIES : 1];
     if (threadIdx.x == 0) {
+#ifndef CREEP_SMALL
         s_ctx.blist = BLIST && S.bvh ? s_blist : nullptr;
+#endif
         s_ctx.n_cand_body = s_ctx.n_body;
     }
     __syncthreads();
@@ -4056,8 +4085,12 @@ static cudaError_t launch_all(const DevScene &S, const Work &W, int nchunks, Lau
                                                                                                   : PLANAR_CHUNKS);
     for (int ch = 0; ch < nchunks && e == cudaSuccess; ch += pstep) {
         const int n = nchunks - ch < pstep ? nchunks - ch : pstep;
-        e = (S.cand && S.n_cand > 0) ? launch_one<T, PATHS, CLS_SEQ, LIST>(S, W, ch, n, 0, L)
-                                     : launch_one<T, PATHS, CLS_PLANAR, LIST>(S, W, ch, n, 0, L);
+        if constexpr (LARGE) {
+            e = (S.cand && S.n_cand > 0) ? launch_one<T, PATHS, CLS_SEQ, LIST>(S, W, ch, n, 0, L)
+                                         : launch_one<T, PATHS, CLS_PLANAR, LIST>(S, W, ch, n, 0, L);
+        } else {
+            e = launch_one<T, PATHS, CLS_PLANAR, LIST>(S, W, ch, n, 0, L);
+        }
         if (chunked_bodies && e == cudaSuccess) e = launch_one<T, PATHS, CLS_BODYREFL, LIST>(S, W, ch, 1, 1, L);
         for (int enc = 0; chunked_bodies && enc <= S.max_enc && e == cudaSuccess; ++enc)
             e = launch_one<T, PATHS, CLS_CREEP, LIST>(S, W, ch, 1, 1, L, enc);
@@ -4080,7 +4113,8 @@ static int run(const DevScene &S, const Work &W, int precision, bool paths, bool
     const int nchunks = paths ? 1 : (S.n_f + NFC - 1) / NFC;
     cudaError_t e;
     // scenes with a BVH: the bodies hidden from the transmitter first
-    const int hid = S.bvh && S.n_body > 0 && (S.enable & (RT_EN_BODYREFL | RT_EN_CREEP_SOFT | RT_EN_CREEP_HARD)) ? 1 : 0;
+    const int hid = LARGE && S.bvh && S.n_body > 0 && (S.enable & (RT_EN_BODYREFL | RT_EN_CREEP_SOFT | RT_EN_CREEP_HARD)) ? 1 : 0;
+#ifndef CREEP_SMALL
     if (hid) {
         k_src_hidden<<<dim3((S.n_body + HID_WARPS - 1) / HID_WARPS, W.frames ? W.n_frames : 1), 32 * HID_WARPS, 0,
                        stream>>>(S, W.F1, W.frames);
@@ -4089,6 +4123,7 @@ static int run(const DevScene &S, const Work &W, int precision, bool paths, bool
             return RT_ERR_CUDA;
         }
     }
+#endif
     if (precision == RT_PREC_FP64) {
         e = paths ? launch_all<dx, true>(S, W, nchunks, L) : launch_all<dx, false>(S, W, nchunks, L);
         if (list && e == cudaSuccess) e = launch_all<dx, true>(S, W, 1, L);
@@ -4105,9 +4140,17 @@ static int run(const DevScene &S, const Work &W, int precision, bool paths, bool
     return RT_OK;
 }
 
+#ifndef CREEP_SMALL
+static bool small_scene(const DevScene &S) { return !S.bvh && !(S.cand && S.n_cand > 0); }
+#endif
+
 int launch_eval(const DevScene &S, const float *rx_soa, int n_rx, float *e_out, uint32_t *flags,
                 uint64_t *codes, int32_t *counts, int cap, int precision, const int *shape, unsigned long long *ctr,
                 cudaStream_t stream, int *n_launches) {
+#ifndef CREEP_SMALL
+    if (small_scene(S))
+        return small::launch_eval(S, rx_soa, n_rx, e_out, flags, codes, counts, cap, precision, shape, ctr, stream, n_launches);
+#endif
     *n_launches = 0;
     // fields and a path list (unordered): counts zeroed first
     const bool paths = codes != nullptr && e_out == nullptr;
@@ -4146,6 +4189,11 @@ int launch_eval_batch(const DevScene &S, const FrameDev *frames_dev, const Frame
                       unsigned long long n_tiles, const float *rx_soa, const int32_t *perm, float *e_out,
                       uint32_t *flags, int precision, const int shape[3], unsigned long long *ctr,
                       cudaStream_t stream, int *n_launches) {
+#ifndef CREEP_SMALL
+    if (small_scene(S))
+        return small::launch_eval_batch(S, frames_dev, frames_host, n_frames, n_tiles, rx_soa, perm, e_out, flags, precision,
+                                        shape, ctr, stream, n_launches);
+#endif
     *n_launches = 0;
     if (n_frames <= 0 || n_tiles == 0) return RT_OK;
     Work W = {};
@@ -4158,6 +4206,10 @@ int launch_eval_batch(const DevScene &S, const FrameDev *frames_dev, const Frame
     return run(S, W, precision, false, false, ctr, stream, n_launches);
 }
 
+#ifdef CREEP_SMALL
+}  // namespace small
+}  // namespace creep
+#else
 // ============================================================== adjoint
 // Gradient of a scalar loss through the fields (the vector-Jacobian product
 // of the evaluation): given dLoss/dE (real and imaginary parts) at every
@@ -5201,3 +5253,4 @@ int launch_adjoint(const DevScene &S, const float *rx_soa, int n_rx, const uint6
 }
 
 }  // namespace creep
+#endif

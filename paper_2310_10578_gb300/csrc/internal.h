@@ -197,6 +197,18 @@ int launch_eval_batch(const DevScene &S, const FrameDev *frames_dev, const Frame
                       uint32_t *flags, int precision, const int shape[3], unsigned long long *ctr,
                       cudaStream_t stream, int *n_launches);
 
+// The same two for scenes without a BVH and without a candidate list
+// (eval_small.cu); the two above pass those on.
+namespace small {
+int launch_eval(const DevScene &S, const float *rx_soa, int n_rx, float *e_out, uint32_t *flags,
+                uint64_t *codes, int32_t *counts, int cap, int precision, const int *shape, unsigned long long *ctr,
+                cudaStream_t stream, int *n_launches);
+int launch_eval_batch(const DevScene &S, const FrameDev *frames_dev, const FrameDev *frames_host, int n_frames,
+                      unsigned long long n_tiles, const float *rx_soa, const int32_t *perm, float *e_out,
+                      uint32_t *flags, int precision, const int shape[3], unsigned long long *ctr,
+                      cudaStream_t stream, int *n_launches);
+}  // namespace small
+
 // Gradient of a loss through the fields (adjoint pass, eval_fields.cu): for
 // the n_rx receivers' listed paths (codes/counts/cap as rt_paths wrote
 // them), the sums of dLoss/dE (grad_e, as the fields) times each path's
