@@ -78,12 +78,41 @@ __device__ __forceinline__ int decide(T m, T band, int tie) {
 }
 
 
-// scene view (pointers into shared or global memory)
+// The scene view's arrays: pointers into shared or global memory; in small
+// scenes all of them staged, as offsets into shared memory, so that the compiler
+// reads them as such (a generic load takes longer, waits as one from memory does,
+// and its address is 64 bits): the reflection kernel's spills went from 208 to 92
+// bytes, the creeping one's from 464 to 344, wall -> creeping paths of 16637
+// receivers from 3.17 to 3.00 ms, 24 frames of 16 frequencies from 16.8 to 16.3,
+// 521473 receivers, 7 bodies from 3.84 to 3.76.
+#ifdef CREEP_SMALL
+template <typename T>
+struct View {
+    uint32_t off;
+    __device__ __forceinline__ const T &operator[](int i) const {
+        extern __shared__ float4 smem[];
+        return *reinterpret_cast<const T *>(reinterpret_cast<const char *>(smem) + off + (uint32_t)i * (uint32_t)sizeof(T));
+    }
+    __device__ __forceinline__ View operator+(int i) const { return View{off + (uint32_t)i * (uint32_t)sizeof(T)}; }
+};
+template <typename T>
+__device__ __forceinline__ View<T> view(const T *staged, const T *) {
+    extern __shared__ float4 smem[];
+    return View<T>{(uint32_t)(reinterpret_cast<const char *>(staged) - reinterpret_cast<const char *>(smem))};
+}
+#else
+template <typename T>
+using View = const T *;
+template <typename T>
+__device__ __forceinline__ const T *view(const T *staged, const T *global) { return staged ? staged : global; }
+#endif
+
+// scene view
 struct Ctx {
-    const float4 *tri, *tri_aux, *face32, *body;
+    View<float4> tri, tri_aux, face32, body;
     const dq4 *face64;
-    const int2 *face_rng;
-    const int *face_tris;
+    View<int2> face_rng;
+    View<int> face_tris;
     const float4 *face_box;      // see DevScene
     const float4 *face_occ;      // see DevScene (with bvh)
     int n_tri, n_face, n_body;
@@ -97,9 +126,9 @@ struct Ctx {
     int n_cand_body;
     float band;
     v3t<float> S, pol;
-    const float4 *fock;          // [FOCK_N][2], then the P segment [FOCK_NP][2] (see DevScene)
-    const float4 *res;           // [FOCK_NRES][2]
-    const float *weid;
+    View<float4> fock;           // [FOCK_N][2], then the P segment [FOCK_NP][2] (see DevScene)
+    View<float4> res;            // [FOCK_NRES][2]
+    View<float> weid;
     float weid_L;
     const double2 *fock64;
     const dq4 *res64;
@@ -107,7 +136,7 @@ struct Ctx {
     const double *weid64;
     const float4 *img;           // source images (double-float), see DevScene
     int img_pairs;               // img holds the ordered face pairs too
-    const float4 *txb;           // [n_body][2] source-side body frame, see DevScene
+    View<float4> txb;            // [n_body][2] source-side body frame, see DevScene
     const float4 *txw;           // [n_face][n_body][2] the same for each face's source image (or nullptr)
 #ifdef CREEP_SMALL
     static constexpr const float4 *bvh = nullptr, *bvh_top = nullptr;
@@ -134,6 +163,15 @@ struct Ctx {
     // body b, on the way of the image's ray to b (nullptr: no masks)
     const uint32_t *occ_w1, *occ_w2;
 };
+
+// Out-of-line functions get the context by reference, which they would read
+// by generic loads: small scenes name the block's shared one (CTX).
+#ifdef CREEP_SMALL
+__shared__ Ctx s_ctx;
+#define CTX(c, arg) const Ctx &c = s_ctx
+#else
+#define CTX(c, arg) const Ctx &c = arg
+#endif
 
 template <typename T>
 __device__ __forceinline__ v3t<T> ld3(float4 q) { return mk3<T>(T((double)q.x), T((double)q.y), T((double)q.z)); }
@@ -376,6 +414,7 @@ __device__ __forceinline__ Box body_box(const Ctx &c, int b) {
     return box_of(lo, hi);
 }
 // triangle t (its face's polygon where the face is one) blocks X -> Y
+#ifndef CREEP_SMALL
 __device__ __noinline__ bool occludes(const Ctx &c, int t, const Box &X, const Box &Y) {
     const float m = hull_margin(c);
     const float4 nq = c.tri_aux[3 * t];
@@ -414,7 +453,6 @@ __device__ __noinline__ bool occludes(const Ctx &c, int t, const Box &X, const B
 // alone is some 100 us of dependent loads, ahead of everything else.  0.07 ms
 // for 110 bodies among 193 572 triangles; with most of those bodies out, the
 // body kernels of 1 M receivers went from 31 and 32 ms to 2.2 and 1.7 ms.
-#ifndef CREEP_SMALL
 constexpr int HID_WARPS = 4;
 constexpr int HID_STACK = 1088;
 __global__ void __launch_bounds__(32 * HID_WARPS) k_src_hidden(DevScene S, FrameDev F1, const FrameDev *frames) {
@@ -580,8 +618,15 @@ __device__ __forceinline__ int blocked_impl(const Ctx &c, v3t<T> A, v3t<T> B, in
 }
 // One out-of-line copy per precision: the visibility loop is called from ten
 // places per receiver; inlining it everywhere overflows the instruction cache.
-__device__ __noinline__ int blocked(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb, float band) {
+__device__ __noinline__ int blocked(const Ctx &ctx, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb, float band) {
+    CTX(c, ctx);
     return blocked_impl(c, A, B, sf1, sf2, sb, band);
+}
+// a mask word, always in shared memory
+__device__ __forceinline__ unsigned ld_shared(const uint32_t *p) {
+    unsigned v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"((unsigned)__cvta_generic_to_shared(p)) : "memory");
+    return v;
 }
 // The bodies (but sb) of the mask occ, nw words, against a segment (FP32): uns
 // tells of uncertain ones among the triangles before
@@ -594,7 +639,7 @@ __device__ __forceinline__ int bodies_masked(const Ctx &c, v3t<float> A, v3t<flo
     const float tlo = (float)EPS_TRIM, thi = 1.0f - (float)EPS_TRIM;
 #pragma unroll 1
     for (int w = 0; w < nw; ++w) {
-        unsigned cand = occ[w];
+        unsigned cand = ld_shared(occ + w);
         if (sb >= 0 && sb >> 5 == w) cand &= ~(1u << (sb & 31));
         while (cand) {
             const int b = 32 * w + __ffs(cand) - 1;
@@ -750,11 +795,13 @@ __device__ __forceinline__ int blocked_mask_inl(const Ctx &c, v3t<float> A, v3t<
     }
     return bodies_masked(c, A, B, sb, band, occ, nw, uns);
 }
-__device__ __noinline__ int blocked_mask(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb,
+__device__ __noinline__ int blocked_mask(const Ctx &ctx, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb,
                                          float band, const uint32_t *occ, int nw) {
+    CTX(c, ctx);
     return blocked_mask_inl(c, A, B, sf1, sf2, sb, band, occ, nw);
 }
-__device__ __noinline__ int blocked(const Ctx &c, v3t<dx> A, v3t<dx> B, int sf1, int sf2, int sb, dx band) {
+__device__ __noinline__ int blocked(const Ctx &ctx, v3t<dx> A, v3t<dx> B, int sf1, int sf2, int sb, dx band) {
+    CTX(c, ctx);
     return blocked_impl(c, A, B, sf1, sf2, sb, band);
 }
 // a leg from or to a point of body b; FP32 legs take the occluder mask occ
@@ -1142,7 +1189,8 @@ __device__ void cyl_frame(v3t<T> S, v3t<T> P, T cx, T cy, T a, Frame<T> &F, T ba
 // rays.  FP32: the source-only quantities (u, |S - c|, beta_s, s' or d_s, and
 // whether the source is over a cylinder's footprint) come precomputed in FP64
 // per transmitter (Ctx::txb); FP64: computed here as the definition does.
-__device__ __forceinline__ void body_frame_tb(const Ctx &c, const float4 *tb, int b, v3t<float> S, v3t<float> P,
+template <typename TB>
+__device__ __forceinline__ void body_frame_tb(const Ctx &c, TB tb, int b, v3t<float> S, v3t<float> P,
                                               float band, Frame<float> &F) {
     float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1], t0 = tb[2 * b], t1 = tb[2 * b + 1];
     float a = q0.w;
@@ -1721,7 +1769,7 @@ __device__ void pekeris(const Ctx &c, float xi, cpx<float> &ps, cpx<float> &ph, 
         const float t = u - (float)j, t2 = t * t, omt = 1.0f - t;
         const float h00 = (1.0f + 2.0f * t) * omt * omt, h10 = t * omt * omt, h01 = t2 * (3.0f - 2.0f * t),
                     h11 = t2 * (t - 1.0f);
-        const float4 *tp = c.fock + 2 * FOCK_N;
+        const View<float4> tp = c.fock + 2 * FOCK_N;
         const float4 a0 = tp[2 * j], a1 = tp[2 * j + 2], b0 = tp[2 * j + 1], b1 = tp[2 * j + 3];
         ps = mkc(h00 * a0.x + h10 * a0.z + h01 * a1.x + h11 * a1.z, h00 * a0.y + h10 * a0.w + h01 * a1.y + h11 * a1.w);
         ph = mkc(h00 * b0.x + h10 * b0.z + h01 * b1.x + h11 * b1.z, h00 * b0.y + h10 * b0.w + h01 * b1.y + h11 * b1.w);
@@ -2506,7 +2554,8 @@ __device__ __forceinline__ void acc_zero(Acc<dx> &a) {
 }
 __device__ __forceinline__ v3t<dx> dxv(v3t<float> a) { return mk3<dx>((double)a.x, (double)a.y, (double)a.z); }
 
-__device__ __noinline__ int esc_inside(const Ctx &c, int b, v3t<float> Pf) {
+__device__ __noinline__ int esc_inside(const Ctx &ctx, int b, v3t<float> Pf) {
+    CTX(c, ctx);
     float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
     dx ex = dx((double)Pf.x) - dx((double)q0.x), ey = dx((double)Pf.y) - dx((double)q0.y),
        ez = dx((double)Pf.z) - dx((double)q0.z), a = dx((double)q0.w);
@@ -2514,16 +2563,19 @@ __device__ __noinline__ int esc_inside(const Ctx &c, int b, v3t<float> Pf) {
     return (ex * ex + ey * ey <= a * a && dx((double)Pf.z) >= dx((double)q0.z) &&
             dx((double)Pf.z) <= dx((double)q0.z) + dx((double)q1.x)) ? D_YES : D_NO;
 }
-__device__ __noinline__ int esc_los(const Ctx &c, v3t<float> Pf) {
+__device__ __noinline__ int esc_los(const Ctx &ctx, v3t<float> Pf) {
+    CTX(c, ctx);
     return cand_los<dx>(c, dxv(c.S), dxv(Pf), dx(0.0));
 }
-__device__ __noinline__ int esc_r1(const Ctx &c, int i, v3t<float> Pf, v3t<float> *Q) {
+__device__ __noinline__ int esc_r1(const Ctx &ctx, int i, v3t<float> Pf, v3t<float> *Q) {
+    CTX(c, ctx);
     Geo<dx> g;
     int d = cand_r1<dx>(c, i, dxv(c.S), dxv(Pf), dx(0.0), g);
     if (d == D_YES) *Q = to_f3(g.Q1);
     return d;
 }
-__device__ __noinline__ int esc_r2(const Ctx &c, int i, int j, v3t<float> Pf, v3t<float> *Q1, v3t<float> *Q2) {
+__device__ __noinline__ int esc_r2(const Ctx &ctx, int i, int j, v3t<float> Pf, v3t<float> *Q1, v3t<float> *Q2) {
+    CTX(c, ctx);
     Geo<dx> g;
     int d = cand_r2<dx>(c, i, j, dxv(c.S), dxv(Pf), dx(0.0), g);
     if (d == D_YES) { *Q1 = to_f3(g.Q1); *Q2 = to_f3(g.Q2); }
@@ -2537,8 +2589,9 @@ __device__ __noinline__ int esc_seq(const Ctx &c, int q, int4 sq, v3t<float> Pf,
     return d;
 }
 // body reflection decided and (field = true) evaluated in FP64
-__device__ __noinline__ int esc_rb(const Ctx &c, int b, v3t<float> Pf, const FreqC &fq, bool field, Contrib *out,
+__device__ __noinline__ int esc_rb(const Ctx &ctx, int b, v3t<float> Pf, const FreqC &fq, bool field, Contrib *out,
                                    float *rec) {
+    CTX(c, ctx);
     Geo<dx> g;
     v3t<dx> Sd = dxv(c.S), Pd = dxv(Pf);
     Frame<dx> F;
@@ -2557,9 +2610,10 @@ __device__ __noinline__ int esc_rb(const Ctx &c, int b, v3t<float> Pf, const Fre
     return d;
 }
 // creeping ray decided, its caustic flag taken, and (field) evaluated in FP64
-__device__ __noinline__ int esc_creep(const Ctx &c, int b, int dir, v3t<float> Pf, const FreqC &fq, bool field,
+__device__ __noinline__ int esc_creep(const Ctx &ctx, int b, int dir, v3t<float> Pf, const FreqC &fq, bool field,
                                       double half_lambda_max, unsigned enable, Contrib *out, int *caustic,
                                       float *rec = nullptr, int *n_rec = nullptr) {
+    CTX(c, ctx);
     Geo<dx> g;
     v3t<dx> Sd = dxv(c.S), Pd = dxv(Pf);
     Frame<dx> F;
@@ -2607,9 +2661,10 @@ __device__ __forceinline__ v3t<dx> wall_img_d(const Ctx &c, int wf) {
 }
 // wall -> creeping candidate decided, its caustic flag taken, and (field)
 // evaluated in FP64, or its records written (rec)
-__device__ __noinline__ int esc_wcreep(const Ctx &c, int wf, int b, int dir, v3t<float> Pf, const FreqC &fq,
+__device__ __noinline__ int esc_wcreep(const Ctx &ctx, int wf, int b, int dir, v3t<float> Pf, const FreqC &fq,
                                        bool field, double half_lambda_max, unsigned enable, Contrib *out,
                                        int *caustic, float *rec, int *n_rec) {
+    CTX(c, ctx);
     Geo<dx> g;
     const v3t<dx> Sd = dxv(c.S), Pd = dxv(Pf), Sw = wall_img_d(c, wf);
     *caustic = 0;
@@ -2651,7 +2706,8 @@ __device__ __noinline__ int esc_wcreep(const Ctx &c, int wf, int b, int dir, v3t
 // frequencies took 1.03 -> 0.72 ms in the planar kernel and 3.24 -> 2.97 ms in the
 // creeping one (its fields are the rest), 1.72 -> 1.83 in that of reflections.
 constexpr float FILT = 16.0f;
-__device__ __noinline__ int filt_rb(const Ctx &c, int b, v3t<float> P, const uint32_t *occ_rx) {
+__device__ __noinline__ int filt_rb(const Ctx &ctx, int b, v3t<float> P, const uint32_t *occ_rx) {
+    CTX(c, ctx);
     const float band = FILT * c.band;
     Frame<float> F;
     Geo<float> g;
@@ -2659,7 +2715,8 @@ __device__ __noinline__ int filt_rb(const Ctx &c, int b, v3t<float> P, const uin
     return cand_rb<float>(c, b, c.S, P, band, F, g, occ_rx);
 }
 // both ways round: the decision of dir in bits 2 dir, 2 dir + 1
-__device__ __noinline__ int filt_creep(const Ctx &c, int b, v3t<float> P, const uint32_t *occ_rx) {
+__device__ __noinline__ int filt_creep(const Ctx &ctx, int b, v3t<float> P, const uint32_t *occ_rx) {
+    CTX(c, ctx);
     const float band = FILT * c.band;
     Frame<float> F;
     body_frame(c, b, c.S, P, band, F);
@@ -2671,7 +2728,8 @@ __device__ __noinline__ int filt_creep(const Ctx &c, int b, v3t<float> P, const 
     }
     return d;
 }
-__device__ __noinline__ int filt_wcreep(const Ctx &c, int wf, int b, v3t<float> P, const uint32_t *occ_rx) {
+__device__ __noinline__ int filt_wcreep(const Ctx &ctx, int wf, int b, v3t<float> P, const uint32_t *occ_rx) {
+    CTX(c, ctx);
     const float band = FILT * c.band;
     const v3t<float> Sw = wall_img_f(c, wf);
     Frame<float> F;
@@ -3414,8 +3472,9 @@ __device__ __forceinline__ float tri_d2(float px, float py, float ax, float ay, 
 // masks of every body for the region (T0, T1, rr): out[b * occ_w + w]; the
 // calling warp (index wi of nwarps that share the work) takes bodies wi,
 // wi + nwarps, ...; every lane of the warp takes part
-__device__ __noinline__ void occ_masks(const Ctx &c, float t0x, float t0y, float t1x, float t1y, float rr, uint32_t *out, int wi,
+__device__ __noinline__ void occ_masks(const Ctx &ctx, float t0x, float t0y, float t1x, float t1y, float rr, uint32_t *out, int wi,
                           int nwarps) {
+    CTX(c, ctx);
     const int lane = threadIdx.x & 31, nb = c.n_body;
     const float margin = 1e-3f + 8.0f * c.band;
 #pragma unroll 1
@@ -3444,7 +3503,8 @@ __device__ __noinline__ void occ_masks(const Ctx &c, float t0x, float t0y, float
 // that of the source and the disk of b mirrored in f (an oblique face turns a
 // cylinder's axis: every body then).
 constexpr int WALL_MASK_WORDS = 2048;      // both sets (8 KB); more pairs go without
-__device__ __noinline__ void wall_masks(const Ctx &c, uint32_t *out1, uint32_t *out2, int wi, int nwarps) {
+__device__ __noinline__ void wall_masks(const Ctx &ctx, uint32_t *out1, uint32_t *out2, int wi, int nwarps) {
+    CTX(c, ctx);
     const int lane = threadIdx.x & 31, nb = c.n_body;
     const float margin = 1e-3f + 9.0f * c.band;
 #pragma unroll 1
@@ -3532,7 +3592,9 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
        int nwt, int tsh, int accumulate, int enc, unsigned long long *esc_counter, unsigned long long *queue) {
     constexpr bool BODIES = (CLS & CLS_BODIES) != 0;
     extern __shared__ float4 smem[];
+#ifndef CREEP_SMALL
     __shared__ Ctx s_ctx;
+#endif
     __shared__ FreqC s_fqs[MAX_CHUNKS];        // frequency chunks ch0 .. ch0 + nch - 1
     // stage scene (and, for the body classes, the Fock--Pekeris table)
     // (FP64 kernels read their own tables in global memory)
@@ -3547,8 +3609,10 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
     float4 *s_tri = s_body + (body_sm ? 2 * S.n_body : 0);   // n_tri * 3 (if staged)
     float4 *s_aux = s_tri + (tri_sm ? 3 * S.n_tri : 0);      // n_tri * 3 (if staged)
     float4 *s_txb = s_aux + (tri_sm ? 3 * S.n_tri : 0);      // n_body * 2 (if staged)
+    int2 *s_rng = reinterpret_cast<int2 *>(s_txb + (body_sm ? 2 * S.n_body : 0));   // (small scenes) n_face, then n_tri
+    int *s_ftri = reinterpret_cast<int *>(s_rng + (LARGE ? 0 : S.n_face));
     const int n_top = LARGE && S.bvh ? min(S.bvh_nodes, BVH_TOP_NODES) : 0;
-    float4 *s_bvh = s_txb + (body_sm ? 2 * S.n_body : 0);    // n_top * 2: the BVH's top treelet
+    float4 *s_bvh = reinterpret_cast<float4 *>(s_rng) + (LARGE ? 0 : (2 * S.n_face + S.n_tri + 3) / 4);   // n_top * 2: the BVH's top treelet
     float *s_weid = (float *)(s_bvh + 2 * n_top);
     float *s_rec = s_weid + WEIDEMAN_N;                      // path records (FP32 fields of the body classes)
     for (int i = threadIdx.x; i < 2 * n_top; i += blockDim.x) s_bvh[i] = S.bvh[i];
@@ -3570,29 +3634,34 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
             s_tri[i] = S.tri[i];
             s_aux[i] = S.tri_alt[i];
         }
+    if (!LARGE) {
+        for (int i = threadIdx.x; i < S.n_face; i += blockDim.x) s_rng[i] = S.face_rng[i];
+        for (int i = threadIdx.x; i < S.n_tri; i += blockDim.x) s_ftri[i] = S.face_tris[i];
+    }
     if (BODIES)
         for (int i = threadIdx.x; i < WEIDEMAN_N; i += blockDim.x) s_weid[i] = S.weid[i];
     if (threadIdx.x == 0) {
         Ctx &c = s_ctx;
-        c.tri = tri_sm ? s_tri : S.tri;
-        c.tri_aux = tri_sm ? s_aux : S.tri_alt;
-        c.face32 = face_sm ? s_face : S.face32;
+        c.tri = view<float4>(tri_sm ? s_tri : nullptr, S.tri);
+        c.tri_aux = view<float4>(tri_sm ? s_aux : nullptr, S.tri_alt);
+        c.face32 = view<float4>(face_sm ? s_face : nullptr, S.face32);
         c.face64 = S.face64;
-        c.face_rng = S.face_rng;
-        c.face_tris = S.face_tris;
+        c.face_rng = view<int2>(LARGE ? nullptr : s_rng, S.face_rng);
+        c.face_tris = view<int>(LARGE ? nullptr : s_ftri, S.face_tris);
         c.face_box = S.face_box;
         c.face_occ = S.face_occ;
-        c.body = body_sm ? s_body : F1.body;
+        c.body = view<float4>(body_sm ? s_body : nullptr, F1.body);
         c.n_tri = S.n_tri; c.n_face = S.n_face; c.n_body = frames ? 0 : F1.n_body;
         c.band = S.band_len;
         c.S = mk3(S.tx[0], S.tx[1], S.tx[2]);
         c.pol = mk3(S.pol[0], S.pol[1], S.pol[2]);
-        c.fock = s_fock; c.res = s_res; c.weid = s_weid; c.weid_L = S.weid_L;
+        c.fock = view<float4>(s_fock, nullptr); c.res = view<float4>(s_res, nullptr); c.weid = view<float>(s_weid, nullptr);
+        c.weid_L = S.weid_L;
         c.fock64 = S.fock64; c.res64 = S.res64; c.p64 = S.p64; c.weid64 = S.weid64;
         c.img = S.img;
         c.img_pairs = S.img_pairs;
         c.face_mat = S.face_mat;
-        c.txb = body_sm ? s_txb : F1.txb;
+        c.txb = view<float4>(body_sm ? s_txb : nullptr, F1.txb);
         c.occ_src = c.occ_w1 = c.occ_w2 = nullptr;
         c.occ_w = 0;
         c.enc = enc;
@@ -3818,8 +3887,8 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                     }
                 stage_words(s_fqs, s_fr.fqc + ch0, nch * sizeof(FreqC));
                 if (threadIdx.x == 0) {
-                    s_ctx.body = body_sm ? s_body : s_fr.body;
-                    s_ctx.txb = body_sm ? s_txb : s_fr.txb;
+                    s_ctx.body = view<float4>(body_sm ? s_body : nullptr, s_fr.body);
+                    s_ctx.txb = view<float4>(body_sm ? s_txb : nullptr, s_fr.txb);
                     s_ctx.n_body = s_fr.n_body;
                     s_ctx.band = s_fr.band;
                     s_ctx.n_cand_body = s_fr.n_body;
@@ -3945,6 +4014,7 @@ static size_t smem_bytes(const DevScene &S, bool tables, bool records, int blk, 
                (S.bvh ? 2 * (size_t)min(S.bvh_nodes, BVH_TOP_NODES) : 0);
     if (S.n_body <= SMEM_BODY_MAX) n += 4 * S.n_body;
     if (S.n_tri <= SMEM_TRI_MAX) n += 6 * S.n_tri;
+    if (!LARGE) n += (2 * S.n_face + S.n_tri + 3) / 4;
     const int occ_w = (occ_sets > 0 && S.n_body > 0 && S.n_body <= OCC_MAX_BODIES) ? (S.n_body + 31) >> 5 : 0;
     const size_t pairs = wall ? 2 * (size_t)S.n_face * S.n_body * occ_w : 0;      // (see wall_masks)
     return n * sizeof(float4) + WEIDEMAN_N * sizeof(float) + 16 +
@@ -4141,7 +4211,10 @@ static int run(const DevScene &S, const Work &W, int precision, bool paths, bool
 }
 
 #ifndef CREEP_SMALL
-static bool small_scene(const DevScene &S) { return !S.bvh && !(S.cand && S.n_cand > 0); }
+static bool small_scene(const DevScene &S) {
+    return !S.bvh && !(S.cand && S.n_cand > 0) && S.n_body <= SMEM_BODY_MAX && S.n_face <= SMEM_FACE_MAX &&
+           S.n_tri <= SMEM_TRI_MAX;
+}
 #endif
 
 int launch_eval(const DevScene &S, const float *rx_soa, int n_rx, float *e_out, uint32_t *flags,
