@@ -1758,6 +1758,20 @@ __device__ cpx<float> faddeeva<float>(const Ctx &c, cpx<float> z) {
     cpx<float> r = cdiv(p * 2.0f, lm * lm) + cdiv(mkc(0.56418958354775628f, 0.0f), lm);
     return r;
 }
+// phat on the table's first segment, XI_LO to XI_HI; rot = e^{+j xi^3/12}
+__device__ __forceinline__ void pek_low(const Ctx &c, float xi, cpx<float> rot, cpx<float> &ps, cpx<float> &ph) {
+    const float u = (xi - (float)XI_LO) * (float)(1.0 / XI_STEP);
+    const int j = min(max((int)u, 0), FOCK_N - 2);
+    const float t = u - (float)j;
+    const float t2 = t * t, omt = 1.0f - t;
+    const float h00 = (1.0f + 2.0f * t) * omt * omt, h10 = t * omt * omt, h01 = t2 * (3.0f - 2.0f * t), h11 = t2 * (t - 1.0f);
+    const float4 a0 = c.fock[2 * j], a1 = c.fock[2 * j + 2];
+    const float4 b0 = c.fock[2 * j + 1], b1 = c.fock[2 * j + 3];
+    const cpx<float> Gs = mkc(h00 * a0.x + h10 * a0.z + h01 * a1.x + h11 * a1.z, h00 * a0.y + h10 * a0.w + h01 * a1.y + h11 * a1.w);
+    const cpx<float> Gh = mkc(h00 * b0.x + h10 * b0.z + h01 * b1.x + h11 * b1.z, h00 * b0.y + h10 * b0.w + h01 * b1.y + h11 * b1.w);
+    ps = Gs * rot;
+    ph = Gh * rot;
+}
 // Fock--Pekeris functions at xi >= XI_LO.  regular = true returns phat = P + c/xi,
 // false returns P itself (each computed without cancellation in its domain).
 __device__ void pekeris(const Ctx &c, float xi, cpx<float> &ps, cpx<float> &ph, bool regular) {
@@ -1807,20 +1821,9 @@ __device__ void pekeris(const Ctx &c, float xi, cpx<float> &ps, cpx<float> &ph, 
         if (regular) { ps = ps + mkc(ci, -ci); ph = ph + mkc(ci, -ci); }
         return;
     }
-    float u = (xi - (float)XI_LO) * (float)(1.0 / XI_STEP);
-    int j = min(max((int)u, 0), FOCK_N - 2);
-    float t = u - (float)j;
-    float t2 = t * t, omt = 1.0f - t;
-    float h00 = (1.0f + 2.0f * t) * omt * omt, h10 = t * omt * omt, h01 = t2 * (3.0f - 2.0f * t), h11 = t2 * (t - 1.0f);
-    float4 a0 = c.fock[2 * j], a1 = c.fock[2 * j + 2];
-    float4 b0 = c.fock[2 * j + 1], b1 = c.fock[2 * j + 3];
-    cpx<float> Gs = mkc(h00 * a0.x + h10 * a0.z + h01 * a1.x + h11 * a1.z, h00 * a0.y + h10 * a0.w + h01 * a1.y + h11 * a1.w);
-    cpx<float> Gh = mkc(h00 * b0.x + h10 * b0.z + h01 * b1.x + h11 * b1.z, h00 * b0.y + h10 * b0.w + h01 * b1.y + h11 * b1.w);
     float sn, cs;
     sincospif(xi * xi * xi * (float)(1.0 / (12.0 * M_PI)), &sn, &cs);   // e^{+j xi^3/12}
-    cpx<float> rot = mkc(cs, sn);
-    ps = Gs * rot;
-    ph = Gh * rot;
+    pek_low(c, xi, mkc(cs, sn), ps, ph);
     if (!regular) { ps = ps - mkc(ci, -ci); ph = ph - mkc(ci, -ci); }
 }
 // FP64 P_s and P_h (v[0], v[1]) on [XI_HI, XI_P] by the polynomial pieces, and
@@ -1919,14 +1922,15 @@ __device__ __forceinline__ cpx<float> faddeeva_t(const Ctx &c, cpx<float> z) { r
 // X > 4: P + (c/xi)(1 - F), 1 - F from w (X < 30) or from the asymptotic series
 // 1 - F ~ -sum_{n>=1} (2n-1)!! (j/(2X))^n (X >= 30, 8 terms): no cancellation
 // between two O(c/xi) terms.
-template <typename T>
-__device__ __forceinline__ void fock_bracket_impl(const Ctx &c, T xi, T K, cpx<T> &Bs, cpx<T> &Bh) {
+// (fock(ps, ph, regular): the Fock--Pekeris functions at xi)
+template <typename T, typename FOCK>
+__device__ __forceinline__ void fock_bracket_of(const Ctx &c, T xi, T K, FOCK fock, cpx<T> &Bs, cpx<T> &Bh) {
     const T r2 = T(0.70710678118654752440), spi = T(1.7724538509055160273), cc = T(0.19947114020071633897);
     T sx = K * Fabs(xi);
     T X = sx * sx;
     cpx<T> ps, ph;
     if (!(X > T(4))) {
-        pekeris(c, xi, ps, ph, true);
+        fock(ps, ph, true);
         cpx<T> w = faddeeva_t(c, mkc<T>(-(sx * r2), sx * r2));
         T s = (xi >= T(0) ? T(1) : T(-1)) * spi * K * r2;
         cpx<T> fx = w * mkc<T>(s, s);                      // F/xi
@@ -1935,7 +1939,7 @@ __device__ __forceinline__ void fock_bracket_impl(const Ctx &c, T xi, T K, cpx<T
         Bh = ph - cf;
         return;
     }
-    pekeris(c, xi, ps, ph, false);
+    fock(ps, ph, false);
     cpx<T> omf;                                            // 1 - F(X)
     if (X >= T(30)) {
         T u = T(0.5) / X;                                  // j/(2X) = j u
@@ -1957,6 +1961,10 @@ __device__ __forceinline__ void fock_bracket_impl(const Ctx &c, T xi, T K, cpx<T
     Bh = ph + cterm;
 }
 
+template <typename T>
+__device__ __forceinline__ void fock_bracket_impl(const Ctx &c, T xi, T K, cpx<T> &Bs, cpx<T> &Bh) {
+    fock_bracket_of<T>(c, xi, K, [&](cpx<T> &ps, cpx<T> &ph, bool regular) { pekeris(c, xi, ps, ph, regular); }, Bs, Bh);
+}
 struct Bpair {
     cpx<float> s, h;
 };
@@ -2402,11 +2410,21 @@ __device__ __forceinline__ void rb_apply(const Ctx &c, AccS<float> &acc, const F
         if (!(xi >= (float)XI_LO)) {
             Rs = mkc<float>(-1, 0); Rh = mkc<float>(1, 0);
         } else {
+            // (xi < 0: the table's first segment, whose turn e^{+j xi^3/12} is the
+            // coefficient's conjugate: one sincospi for both, 24 frames of 16
+            // frequencies 16.3 -> 16.1 ms)
             cpx<float> Bs, Bh;
-            fock_bracket<float>(c, xi, fq.sk[f] * sLr, Bs, Bh);
             float sn, cs;
-            sincospif(-xi * xi * xi * (float)(1.0 / (12.0 * M_PI)), &sn, &cs);
-            cpx<float> pre = mkc<float>(cs, sn) * (-sqrtf(-4.0f / xi));
+            sincospif(xi * xi * xi * (float)(1.0 / (12.0 * M_PI)), &sn, &cs);
+            fock_bracket_of<float>(c, xi, fq.sk[f] * sLr, [&](cpx<float> &ps, cpx<float> &ph, bool regular) {
+                pek_low(c, xi, mkc(cs, sn), ps, ph);
+                if (!regular) {
+                    const float ci = 0.19947114f / xi;
+                    ps = ps - mkc(ci, -ci);
+                    ph = ph - mkc(ci, -ci);
+                }
+            }, Bs, Bh);
+            cpx<float> pre = mkc<float>(cs, -sn) * (-sqrtf(-4.0f / xi));
             Rs = pre * Bs; Rh = pre * Bh;
         }
         cpx<float> ph = phasor(fq, f, len) * A;
@@ -2757,10 +2775,13 @@ constexpr int CLS_BODIES = CLS_BODYREFL | CLS_CREEP | CLS_WCREEP;
 // tiles at a time, four warps per tile; a block barrier between the geometry
 // pass and the field pass keeps all warps of the SM in the same pass, so the
 // instruction cache holds one pass's code at a time.  The planar class, and
-// the FP64 path, run 4-warp blocks, several per SM.
+// the FP64 path, run 4-warp blocks, several per SM: the planar class of small
+// scenes is bound by its waits for instructions and dependent results, so that
+// five blocks at 96 registers (some spilled) do better than four at 128 or three
+// at 166: 521473 receivers, 7 bodies 3.66 against 3.76 and 3.93 ms.
 constexpr int blk_of(int cls, bool fp32) { return ((cls & CLS_BODIES) && fp32) ? 384 : BLOCK; }
 constexpr int min_blocks(int cls, bool fp32) {
-    return ((cls & CLS_BODIES) && fp32) ? 1 : (is_planar(cls) ? 4 : 3);
+    return ((cls & CLS_BODIES) && fp32) ? 1 : (is_planar(cls) ? (fp32 && !LARGE ? 5 : 4) : 3);
 }
 // records per work unit of a body class (FP32 fields)
 constexpr int recs_per_unit(int cls) {
@@ -2770,7 +2791,16 @@ constexpr int WARPS_PER_TILE = 4;
 constexpr int PATH_TILES = 3;
 constexpr int MAX_CHUNKS = (RT_MAX_FREQS + NFC - 1) / NFC;
 constexpr int PLANAR_CHUNKS = 4;       // frequency chunks per planar launch (FP32 fields)
-constexpr int OCC_MAX_BODIES = 256;    // occluder masks up to this many bodies (FP32 body kernels)
+constexpr int OCC_MAX_BODIES = 256;    // occluder masks up to this many bodies
+// Wall -> creeping kernels: at most so many words (4.5 KB) of the bodies' masks, and
+// of the (face, body) pairs' again, beside the path records; more go without.
+constexpr int WALL_MASK_WORDS = 1152;
+// words per body of the occluder masks (0: none): one source-side set and sets
+// receiver-side ones
+__host__ __device__ __forceinline__ int occ_words(int n_body, int sets, bool wall) {
+    const int w = n_body > 0 && n_body <= OCC_MAX_BODIES ? (n_body + 31) >> 5 : 0;
+    return wall && n_body * w * (1 + sets) > WALL_MASK_WORDS ? 0 : w;
+}
 
 // Field pass over one lane's records for the frequency chunk fq.
 template <int CLS>
@@ -3502,7 +3532,6 @@ __device__ __noinline__ void occ_masks(const Ctx &ctx, float t0x, float t0y, flo
 // in the hull of the image and b's disk; its part before the face, mirrored, in
 // that of the source and the disk of b mirrored in f (an oblique face turns a
 // cylinder's axis: every body then).
-constexpr int WALL_MASK_WORDS = 2048;      // both sets (8 KB); more pairs go without
 __device__ __noinline__ void wall_masks(const Ctx &ctx, uint32_t *out1, uint32_t *out2, int wi, int nwarps) {
     CTX(c, ctx);
     const int lane = threadIdx.x & 31, nb = c.n_body;
@@ -3700,8 +3729,8 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         // occluder masks (body kernels): the source side per block, the
         // receiver side per warp (each warp takes whole tiles)
         constexpr bool OCC = BODIES;
-        const bool occ_on = OCC && S.n_body > 0 && S.n_body <= OCC_MAX_BODIES;
-        const int occ_w = occ_on ? (S.n_body + 31) >> 5 : 0;
+        const int occ_w = OCC ? occ_words(S.n_body, NW, CLS == CLS_WCREEP) : 0;
+        const bool occ_on = occ_w > 0;
         uint32_t *s_occ_src = reinterpret_cast<uint32_t *>(s_rec);
         uint32_t *s_occ_mine = s_occ_src + (1 + warp) * S.n_body * occ_w;
         uint32_t *s_occ_wall = s_occ_src + (1 + NW) * S.n_body * occ_w;
@@ -3845,8 +3874,8 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         // occluder masks (body kernels): the source side per frame, the
         // receiver side per tile, after the path records
         constexpr bool OCC = BODIES;
-        const bool occ_on = OCC && S.n_body > 0 && S.n_body <= OCC_MAX_BODIES;
-        const int occ_w = occ_on ? (S.n_body + 31) >> 5 : 0;
+        const int occ_w = OCC ? occ_words(S.n_body, TPB, CLS == CLS_WCREEP) : 0;
+        const bool occ_on = occ_w > 0;
         uint32_t *s_occ_src = reinterpret_cast<uint32_t *>(s_rec + (RECS ? NW * rcap * REC_N * 32 : 0));
         uint32_t *s_occ_rx = s_occ_src + S.n_body * occ_w;
         uint32_t *s_occ_wall = s_occ_rx + TPB * S.n_body * occ_w;       // (single frames only, as the wall class)
@@ -4015,7 +4044,7 @@ static size_t smem_bytes(const DevScene &S, bool tables, bool records, int blk, 
     if (S.n_body <= SMEM_BODY_MAX) n += 4 * S.n_body;
     if (S.n_tri <= SMEM_TRI_MAX) n += 6 * S.n_tri;
     if (!LARGE) n += (2 * S.n_face + S.n_tri + 3) / 4;
-    const int occ_w = (occ_sets > 0 && S.n_body > 0 && S.n_body <= OCC_MAX_BODIES) ? (S.n_body + 31) >> 5 : 0;
+    const int occ_w = occ_sets > 0 ? occ_words(S.n_body, occ_sets, wall) : 0;
     const size_t pairs = wall ? 2 * (size_t)S.n_face * S.n_body * occ_w : 0;      // (see wall_masks)
     return n * sizeof(float4) + WEIDEMAN_N * sizeof(float) + 16 +
            (records ? sizeof(float) * (blk / 32) * rcap * REC_N * 32 : 0) +
