@@ -808,7 +808,8 @@ __device__ __noinline__ int blocked(const Ctx &ctx, v3t<dx> A, v3t<dx> B, int sf
 // (nullptr: every body)
 template <typename T>
 __device__ __forceinline__ int blocked_leg(const Ctx &c, v3t<T> A, v3t<T> B, int b, T band, const uint32_t *occ) {
-    if constexpr (sizeof(T) == 4) return blocked_mask_inl(c, A, B, -1, -1, b, band, occ, c.occ_w);
+    if constexpr (sizeof(T) == 4 && LARGE) return blocked_mask(c, A, B, -1, -1, b, band, occ, c.occ_w);
+    else if constexpr (sizeof(T) == 4) return blocked_mask_inl(c, A, B, -1, -1, b, band, occ, c.occ_w);
     else return blocked(c, A, B, -1, -1, b, band);
 }
 __device__ __forceinline__ const uint32_t *occ_of(const Ctx &c, const uint32_t *masks, int b) {
@@ -1569,7 +1570,10 @@ __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Fr
     // coefficient's pole (both of order cos^(1/2)) would meet as 0 * inf: the
     // smallest positive value keeps their finite product
     const T cth = Fmax(-dot3(shi, n), T(COS_MIN));
-    if constexpr (VIS) {
+    if constexpr (VIS && LARGE) {
+        if (!conj(acc, vis_to_dec(blocked_leg(c, S, Q, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
+        if (!conj(acc, vis_to_dec(blocked_leg(c, Q, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    } else if constexpr (VIS) {
 #pragma unroll 1
         for (int leg = 0; leg < 2; ++leg) {          // (as in cand_creep)
             const bool src = leg == 0;
@@ -1678,9 +1682,14 @@ __device__ int cand_creep(const Ctx &c, int b, int dir, v3t<T> S, v3t<T> P, T ba
         g.dperp = T(0);
         g.amp = T(1) / Sqrt(g.sp * g.sq * (g.sp + g.t + g.sq));
     }
-    if constexpr (VIS) {
+    if constexpr (VIS && LARGE) {
+        if constexpr (SRC_LEG) {
+            if (!conj(acc, vis_to_dec(blocked_leg(c, S, g.Q1, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
+        }
+        if (!conj(acc, vis_to_dec(blocked_leg(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    } else if constexpr (VIS) {
         // (one copy of the visibility test, inlined: a call's registers would be
-        // spilled round it)
+        // spilled round it; large scenes walk a BVH, out of line)
 #pragma unroll 1
         for (int leg = SRC_LEG ? 0 : 1; leg < 2; ++leg) {
             const bool src = leg == 0;
@@ -5147,9 +5156,10 @@ __device__ __forceinline__ double warp_sum(double v) {
 // over the lanes of a warp, each kind ran on 2.9 of 32 lanes (200 bodies) to
 // 6.2 (12 bodies).  Sorted, and with the FP64 fields differentiated backwards,
 // a gradient step (fields, lists and this kernel) of 4096 receivers among 200
-// bodies went from 2.58 to 1.65 ms, one of 2867 receivers, 12 bodies and three
-// frequencies with FP32 duals from 4.10 to 0.94 ms.
-constexpr int ADJ_BLOCK = 128;
+// bodies went from 2.58 to 1.38 ms, one of 2867 receivers, 12 bodies and three
+// frequencies with FP32 duals from 4.20 to 0.73 ms (0.96 with two blocks of four
+// warps an SM in place of one of eight: fewer receivers to sort among).
+constexpr int ADJ_BLOCK = 256;
 constexpr int ADJ_RX = 32;               // receivers of a unit, at most
 constexpr int ADJ_ITEMS = 2048;          // paths sorted at once
 constexpr int ADJ_KINDS = 7;
@@ -5340,7 +5350,7 @@ int launch_adjoint(const DevScene &S, const float *rx_soa, int n_rx, const uint6
         // the fewest units of at most ADJ_RX receivers that give every SM the same
         // number: the more receivers a unit, the fuller the last warp of each kind
         const int waves = (n_rx + ADJ_RX * nsm - 1) / (ADJ_RX * nsm), rpu = max(1, (n_rx + waves * nsm - 1) / (waves * nsm));
-        const int units = (n_rx + rpu - 1) / rpu, grid = min(units, 2 * nsm);
+        const int units = (n_rx + rpu - 1) / rpu, grid = min(units, nsm);
         if (precision == RT_PREC_FP64)
             k_adjoint<true><<<grid, ADJ_BLOCK, 0, st>>>(S, rx_soa, n_rx, rpu, codes, counts, cap, grad_e, g_body, g_tx, g_f, queue);
         else
