@@ -2798,6 +2798,8 @@ constexpr int recs_per_unit(int cls) {
 }
 constexpr int WARPS_PER_TILE = 4;
 constexpr int PATH_TILES = 3;
+constexpr uint16_t NO_BODY = 0xffffu;  // see body_list
+constexpr int BLIST_MAX = RT_MAX_BODIES + 32;
 constexpr int MAX_CHUNKS = (RT_MAX_FREQS + NFC - 1) / NFC;
 constexpr int PLANAR_CHUNKS = 4;       // frequency chunks per planar launch (FP32 fields)
 constexpr int OCC_MAX_BODIES = 256;    // occluder masks up to this many bodies
@@ -3309,6 +3311,7 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
             for (int bi = b_begin + part; bi < b_end; bi += nparts) {
                 // (scenes with a BVH: bi counts the bodies the source may see)
                 const int b = (CLS != CLS_WCREEP && c.blist) ? c.blist[bi] : bi;
+                if (CLS != CLS_WCREEP && c.blist && b == NO_BODY) continue;
                 if constexpr (RECS) {
                     // one frequency chunk: records that could overflow are turned
                     // into fields here (with several chunks the caller sizes the
@@ -3519,6 +3522,7 @@ __device__ __noinline__ void occ_masks(const Ctx &ctx, float t0x, float t0y, flo
 #pragma unroll 1
     for (int bi = wi; bi < c.n_cand_body; bi += nwarps) {
         const int b = c.blist ? c.blist[bi] : bi;
+        if (c.blist && b == NO_BODY) continue;
         const float4 qb = c.body[2 * b];
         const float rad = fmaxf(rr, qb.w) + c.band + margin;
 #pragma unroll 1
@@ -3597,20 +3601,30 @@ __device__ __forceinline__ void tile_masks(const Ctx &c, const float *rx, int n_
     }
 }
 
-// the whole block: the bodies without their bit in hid, in order; ends with a
-// barrier.  (An office's walls hide most of its bodies from a transmitter: the
-// warps of a tile share the rest evenly, where a skipped body in its owner's
-// loop left the others waiting.)
-__device__ __noinline__ void body_list(Ctx &c, const uint32_t *hid, uint16_t *list) {
+// the whole block: the bodies without their bit in hid, share by share (body b
+// belongs to share b mod np, np <= 32, and keeps its place in that share's sum):
+// entry p + np k is the k-th of share p, NO_BODY past the share's last; ends with
+// a barrier.  (An office's walls hide most of its bodies from a transmitter: a
+// skipped body in its owner's loop left the other lanes and warps waiting.)
+__device__ __noinline__ void body_list(Ctx &c, const uint32_t *hid, uint16_t *list, int np) {
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
-        int n = 0;
-        for (int b0 = 0; b0 < c.n_body; b0 += 32) {
-            const unsigned word = ~hid[b0 >> 5] & (b0 + 32 <= c.n_body ? 0xffffffffu : (1u << (c.n_body - b0)) - 1u);
-            if (word >> lane & 1u) list[n + __popc(word & ((1u << lane) - 1u))] = (uint16_t)(b0 + lane);
-            n += __popc(word);
+        int most = 0, mine = 0;
+        for (int p = 0; p < np; ++p) {
+            int n = 0;
+            for (int k0 = 0; p + np * k0 < c.n_body; k0 += 32) {
+                const int b = p + np * (k0 + lane);
+                const bool seen = b < c.n_body && !(hid[b >> 5] >> (b & 31) & 1u);
+                const unsigned word = __ballot_sync(0xffffffffu, seen);
+                if (seen) list[p + np * (n + __popc(word & ((1u << lane) - 1u)))] = (uint16_t)b;
+                n += __popc(word);
+            }
+            most = max(most, n);
+            if (lane == p) mine = n;
         }
-        if (lane == 0) c.n_cand_body = n;
+        for (int p = 0; p < np; ++p)
+            for (int k = __shfl_sync(0xffffffffu, mine, p) + lane; k < most; k += 32) list[p + np * k] = NO_BODY;
+        if (lane == 0) c.n_cand_body = np * most;
     }
     __syncthreads();
 }
@@ -3722,7 +3736,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
     constexpr int NW = blk_of(CLS, sizeof(T) == 4) / 32;
     // scenes with a BVH: the bodies not hidden from the source (body_list)
     constexpr bool BLIST = LARGE && BODIES && CLS != CLS_WCREEP;
-    __shared__ uint16_t s_blist[BLIST ? RT_MAX_BODIES : 1];
+    __shared__ uint16_t s_blist[BLIST ? BLIST_MAX : 1];
     if (threadIdx.x == 0) {
 #ifndef CREEP_SMALL
         s_ctx.blist = BLIST && S.bvh ? s_blist : nullptr;
@@ -3730,7 +3744,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
         s_ctx.n_cand_body = s_ctx.n_body;
     }
     __syncthreads();
-    if (BLIST && S.bvh && !frames) body_list(s_ctx, F1.hid, s_blist);
+    if (BLIST && S.bvh && !frames) body_list(s_ctx, F1.hid, s_blist, PATHS ? (split_paths(CLS) && nwt > 1 ? NW : 1) : nwt);
     if constexpr (PATHS) {
         // (one frame only)
         const float *rx = rx_base;
@@ -3932,7 +3946,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                     s_ctx.n_cand_body = s_fr.n_body;
                 }
                 __syncthreads();
-                if (BLIST && S.bvh) body_list(s_ctx, s_fr.hid, s_blist);
+                if (BLIST && S.bvh) body_list(s_ctx, s_fr.hid, s_blist, nwt);
                 if (occ_on) {
                     occ_masks(c, c.S.x, c.S.y, c.S.x, c.S.y, 0.0f, s_occ_src, warp, NW);
                     __syncthreads();
