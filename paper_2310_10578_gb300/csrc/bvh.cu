@@ -60,7 +60,8 @@ inline int float_bits(float f) {
 // boxes and 24 triangles to their first hit or end; with this split 68 and 11).
 // The median split stays for nodes that no plane divides, and where a node's
 // depth and the levels that median splits still need below it reach MAX_DEPTH:
-// the device walks' stacks count on that.
+// the device walks' stacks count on that.  An axis on which the centroids' spread
+// or its reciprocal is not finite has no bins (vertices may be any finite floats).
 constexpr int SAH_BINS = 16;
 constexpr int MAX_DEPTH = 32;
 
@@ -96,15 +97,15 @@ struct Builder {
         float sc[3];
         const int nb = hi - lo <= 2 * SAH_BINS ? SAH_BINS / 2 : SAH_BINS;       // (most nodes are small)
         for (int k = 0; k < 3; ++k) {
-            sc[k] = cmax[k] > cmin[k] ? nb / (cmax[k] - cmin[k]) : 0.0f;
+            const float ext = cmax[k] - cmin[k];
+            sc[k] = std::isfinite(ext) && ext > 0.0f && std::isfinite(nb / ext) ? nb / ext : 0.0f;
             for (int s = 0; s < nb; ++s) { empty(bin[k][s].b); bin[k][s].n = 0; }
         }
-        auto slot = [&](const Item &q, int k) {
-            const int s = (int)((q.c[k] - cmin[k]) * sc[k]);
-            return s < nb - 1 ? s : nb - 1;
-        };
+        // (an axis with sc > 0: its centroids are finite, (c - cmin) sc within a rounding of [0, nb])
+        auto slot = [&](const Item &q, int k) { return std::min((int)((q.c[k] - cmin[k]) * sc[k]), nb - 1); };
         for (int i = lo; i < hi; ++i)
             for (int k = 0; k < 3; ++k) {
+                if (sc[k] == 0.0f) continue;
                 Bin &q = bin[k][slot(it[i], k)];
                 grow(q.b, it[i].b);
                 ++q.n;
