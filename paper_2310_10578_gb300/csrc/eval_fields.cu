@@ -30,8 +30,9 @@
 // membership inclusive, bodies strict).  Path lengths are accumulated as
 // double-float so that the phase 2 pi frac(L / lambda) keeps ~1e-7 rad at
 // 28 GHz over tens of metres.  Reflection points near grazing incidence are
-// refined in FP64.  RT_PREC_FP64 takes every value from FP64; its decisions are
-// FP32's where those are certain by a wide margin, and FP64's otherwise.
+// refined in FP64.  RT_PREC_FP64 runs everything in FP64 but for tests on given
+// or exact points (a triangle or a body against a leg, a point in a triangle),
+// which FP32 takes where it is certain with the points' rounding in its band.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -357,10 +358,10 @@ __device__ __forceinline__ bool bvh_walk(const Ctx &c, v3t<float> A, v3t<float> 
 template <typename T>
 __device__ __forceinline__ int tris_bvh(const Ctx &c, v3t<T> A, v3t<T> B, int sf1, int sf2, T band) {
     v3t<float> Af, Bf;
-    float box_m = 0.0f;
+    float box_m = 0.0f, tri_b = c.band;          // (tri_b: the FP32 test's band)
     if constexpr (sizeof(T) == 4) {
         Af = A; Bf = B;
-        box_m = band;
+        box_m = tri_b = band;
     } else {
         Af = mk3<float>(to_float(A.x), to_float(A.y), to_float(A.z));
         Bf = mk3<float>(to_float(B.x), to_float(B.y), to_float(B.z));
@@ -369,7 +370,7 @@ __device__ __forceinline__ int tris_bvh(const Ctx &c, v3t<T> A, v3t<T> B, int sf
     const bool hit = bvh_walk(c, Af, Bf, box_m, [&](int t) {
         const int f = __float_as_int(c.tri[3 * t].w);
         if (f == sf1 || f == sf2) return false;
-        int r = seg_tri(c, t, Af, Bf, c.band);
+        int r = seg_tri(c, t, Af, Bf, tri_b);
         if constexpr (sizeof(T) == 8) {
             if (r == D_UNSURE) r = seg_tri(c, t, A, B, band);
         }
@@ -717,7 +718,7 @@ __device__ __forceinline__ int coop_walk(const Ctx &c, unsigned lanes, v3t<float
             const int t = c.bvh_tri[first + j];
             const int f = __float_as_int(c.tri[3 * t].w);
             if (f == sf1 || f == sf2) continue;
-            const int r = seg_tri(c, t, a, b, c.band);
+            const int r = seg_tri(c, t, a, b, band);
             if (r == D_YES) hit = t;
             u = u || r == D_UNSURE;
         }
@@ -804,13 +805,28 @@ __device__ __noinline__ int blocked(const Ctx &ctx, v3t<dx> A, v3t<dx> B, int sf
     CTX(c, ctx);
     return blocked_impl(c, A, B, sf1, sf2, sb, band);
 }
-// a leg from or to a point of body b; FP32 legs take the occluder mask occ
-// (nullptr: every body)
-template <typename T>
+// A leg with an occluder mask in either precision.  FP64 (exact end points): FP32
+// on the rounded ones first, whose band covers that rounding, and FP64 only where
+// it is uncertain.
+__device__ __forceinline__ int leg(const Ctx &c, v3t<float> A, v3t<float> B, int sf1, int sf2, int sb, float band,
+                                   const uint32_t *occ, int nw) {
+    return blocked_mask(c, A, B, sf1, sf2, sb, band, occ, nw);
+}
+__device__ __forceinline__ int leg(const Ctx &c, v3t<dx> A, v3t<dx> B, int sf1, int sf2, int sb, dx band,
+                                   const uint32_t *occ, int nw) {
+    const v3t<float> Af = mk3<float>(to_float(A.x), to_float(A.y), to_float(A.z));
+    const v3t<float> Bf = mk3<float>(to_float(B.x), to_float(B.y), to_float(B.z));
+    const int r = blocked_mask(c, Af, Bf, sf1, sf2, sb, c.band, occ, nw);
+    return r != D_UNSURE ? r : blocked(c, A, B, sf1, sf2, sb, band);
+}
+// a leg from or to a point of body b, with the occluder mask occ (nullptr: every
+// body); REDO: FP32 was uncertain of this candidate, FP64 straight away
+template <typename T, bool REDO>
 __device__ __forceinline__ int blocked_leg(const Ctx &c, v3t<T> A, v3t<T> B, int b, T band, const uint32_t *occ) {
-    if constexpr (sizeof(T) == 4 && LARGE) return blocked_mask(c, A, B, -1, -1, b, band, occ, c.occ_w);
+    if constexpr (REDO) return blocked(c, A, B, -1, -1, b, band);
+    else if constexpr (sizeof(T) == 4 && LARGE) return blocked_mask(c, A, B, -1, -1, b, band, occ, c.occ_w);
     else if constexpr (sizeof(T) == 4) return blocked_mask_inl(c, A, B, -1, -1, b, band, occ, c.occ_w);
-    else return blocked(c, A, B, -1, -1, b, band);
+    else return leg(c, A, B, -1, -1, b, band, occ, c.occ_w);
 }
 __device__ __forceinline__ const uint32_t *occ_of(const Ctx &c, const uint32_t *masks, int b) {
     return (masks && c.occ_w) ? masks + b * c.occ_w : nullptr;
@@ -991,8 +1007,8 @@ __device__ int cand_los(const Ctx &c, v3t<T> S, v3t<T> P, T band) {
 }
 
 // planar candidates: the geometric part (sides, reflection points in their
-// faces; the points in g), then the visibility of the legs (FP32: with the
-// legs' occluder masks wm, or none)
+// faces; the points in g), then the visibility of the legs (with the legs'
+// occluder masks wm, or none)
 template <typename T>
 __device__ __forceinline__ int cand_r1_geo(const Ctx &c, int i, v3t<T> S, v3t<T> P, T band, Geo<T> &g) {
     v3t<T> n; T d;
@@ -1007,10 +1023,11 @@ __device__ __forceinline__ int cand_r1_geo(const Ctx &c, int i, v3t<T> S, v3t<T>
     if (!conj(acc, in_face(c, i, g.Q1, band))) return D_NO;
     return acc;
 }
-__device__ __forceinline__ int cand_r1_vis(const Ctx &c, int i, v3t<float> S, v3t<float> P, float band,
-                                           const Geo<float> &g, int acc, const uint32_t *wm, int nw) {
-    if (!conj(acc, vis_to_dec(blocked_mask(c, S, g.Q1, i, -1, -1, band, wm, nw)))) return D_NO;
-    if (!conj(acc, vis_to_dec(blocked_mask(c, g.Q1, P, i, -1, -1, band, wm ? wm + nw : nullptr, nw)))) return D_NO;
+template <typename T>
+__device__ __forceinline__ int cand_r1_vis(const Ctx &c, int i, v3t<T> S, v3t<T> P, T band,
+                                           const Geo<T> &g, int acc, const uint32_t *wm, int nw) {
+    if (!conj(acc, vis_to_dec(leg(c, S, g.Q1, i, -1, -1, band, wm, nw)))) return D_NO;
+    if (!conj(acc, vis_to_dec(leg(c, g.Q1, P, i, -1, -1, band, wm ? wm + nw : nullptr, nw)))) return D_NO;
     return acc;
 }
 template <typename T>
@@ -1043,11 +1060,12 @@ __device__ __forceinline__ int cand_r2_geo(const Ctx &c, int i, int j, v3t<T> S,
     if (!conj(acc, in_face(c, i, Q1, band))) return D_NO;
     return acc;
 }
-__device__ __forceinline__ int cand_r2_vis(const Ctx &c, int i, int j, v3t<float> S, v3t<float> P, float band,
-                                           const Geo<float> &g, int acc, const uint32_t *wm, int nw) {
-    if (!conj(acc, vis_to_dec(blocked_mask(c, S, g.Q1, i, -1, -1, band, wm, nw)))) return D_NO;
-    if (!conj(acc, vis_to_dec(blocked_mask(c, g.Q1, g.Q2, i, j, -1, band, wm ? wm + nw : nullptr, nw)))) return D_NO;
-    if (!conj(acc, vis_to_dec(blocked_mask(c, g.Q2, P, j, -1, -1, band, wm ? wm + 2 * nw : nullptr, nw)))) return D_NO;
+template <typename T>
+__device__ __forceinline__ int cand_r2_vis(const Ctx &c, int i, int j, v3t<T> S, v3t<T> P, T band,
+                                           const Geo<T> &g, int acc, const uint32_t *wm, int nw) {
+    if (!conj(acc, vis_to_dec(leg(c, S, g.Q1, i, -1, -1, band, wm, nw)))) return D_NO;
+    if (!conj(acc, vis_to_dec(leg(c, g.Q1, g.Q2, i, j, -1, band, wm ? wm + nw : nullptr, nw)))) return D_NO;
+    if (!conj(acc, vis_to_dec(leg(c, g.Q2, P, j, -1, -1, band, wm ? wm + 2 * nw : nullptr, nw)))) return D_NO;
     return acc;
 }
 template <typename T>
@@ -1523,9 +1541,8 @@ __device__ __forceinline__ dfl df_norm3(const dfl w[3]) {
 // smallest incidence cosine of a reflection off a body (see cand_rb)
 constexpr double COS_MIN = 1e-30;
 
-// body reflection candidate (sphere or vertical cylinder)
-// (VIS false: the legs are known to be clear)
-template <typename T, bool VIS = true>
+// body reflection candidate (sphere or vertical cylinder; REDO: see blocked_leg)
+template <typename T, bool REDO = false>
 __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Frame<T> &F, Geo<T> &g,
                        const uint32_t *occ_rx = nullptr) {
     float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
@@ -1570,14 +1587,14 @@ __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Fr
     // coefficient's pole (both of order cos^(1/2)) would meet as 0 * inf: the
     // smallest positive value keeps their finite product
     const T cth = Fmax(-dot3(shi, n), T(COS_MIN));
-    if constexpr (VIS && LARGE) {
-        if (!conj(acc, vis_to_dec(blocked_leg(c, S, Q, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
-        if (!conj(acc, vis_to_dec(blocked_leg(c, Q, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
-    } else if constexpr (VIS) {
+    if constexpr (LARGE) {
+        if (!conj(acc, vis_to_dec(blocked_leg<T, REDO>(c, S, Q, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
+        if (!conj(acc, vis_to_dec(blocked_leg<T, REDO>(c, Q, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+    } else {
 #pragma unroll 1
-        for (int leg = 0; leg < 2; ++leg) {          // (as in cand_creep)
-            const bool src = leg == 0;
-            if (!conj(acc, vis_to_dec(blocked_leg(c, src ? S : Q, src ? Q : P, b, band,
+        for (int k = 0; k < 2; ++k) {                // (as in cand_creep)
+            const bool src = k == 0;
+            if (!conj(acc, vis_to_dec(blocked_leg<T, REDO>(c, src ? S : Q, src ? Q : P, b, band,
                                                   occ_of(c, src ? c.occ_src : occ_rx, b)))))
                 return D_NO;
         }
@@ -1620,8 +1637,8 @@ __device__ int cand_rb(const Ctx &c, int b, v3t<T> S, v3t<T> P, T band, const Fr
 
 // creeping candidate, dir 0 short way, 1 long way (SRC_LEG false: the leg
 // from the source S to Q1 is the caller's, e.g. S is a source image; VIS
-// false: the legs are known to be clear)
-template <typename T, bool SRC_LEG = true, bool VIS = true>
+// false: both legs are the caller's)
+template <typename T, bool SRC_LEG = true, bool VIS = true, bool REDO = false>
 __device__ int cand_creep(const Ctx &c, int b, int dir, v3t<T> S, v3t<T> P, T band, const Frame<T> &F, Geo<T> &g,
                           const uint32_t *occ_rx = nullptr) {
     float4 q0 = c.body[2 * b], q1 = c.body[2 * b + 1];
@@ -1684,16 +1701,16 @@ __device__ int cand_creep(const Ctx &c, int b, int dir, v3t<T> S, v3t<T> P, T ba
     }
     if constexpr (VIS && LARGE) {
         if constexpr (SRC_LEG) {
-            if (!conj(acc, vis_to_dec(blocked_leg(c, S, g.Q1, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
+            if (!conj(acc, vis_to_dec(blocked_leg<T, REDO>(c, S, g.Q1, b, band, occ_of(c, c.occ_src, b))))) return D_NO;
         }
-        if (!conj(acc, vis_to_dec(blocked_leg(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
+        if (!conj(acc, vis_to_dec(blocked_leg<T, REDO>(c, g.Q2, P, b, band, occ_of(c, occ_rx, b))))) return D_NO;
     } else if constexpr (VIS) {
         // (one copy of the visibility test, inlined: a call's registers would be
         // spilled round it; large scenes walk a BVH, out of line)
 #pragma unroll 1
-        for (int leg = SRC_LEG ? 0 : 1; leg < 2; ++leg) {
-            const bool src = leg == 0;
-            if (!conj(acc, vis_to_dec(blocked_leg(c, src ? S : g.Q2, src ? g.Q1 : P, b, band,
+        for (int k = SRC_LEG ? 0 : 1; k < 2; ++k) {
+            const bool src = k == 0;
+            if (!conj(acc, vis_to_dec(blocked_leg<T, REDO>(c, src ? S : g.Q2, src ? g.Q1 : P, b, band,
                                                   occ_of(c, src ? c.occ_src : occ_rx, b)))))
                 return D_NO;
         }
@@ -1733,22 +1750,23 @@ __device__ int wall_legs(const Ctx &c, int f, int b, v3t<dx> S, v3t<dx> Sw, v3t<
     if (!conj(acc, vis_to_dec(blocked(c, Qw, Q1, f, -1, b, band)))) return D_NO;
     return acc;
 }
-// The whole wall -> creeping candidate in FP32.  Its geometry comes first, the
+// The whole wall -> creeping candidate.  Its geometry comes first, the
 // legs last: a leg's test costs more than all of the geometry, which leaves
 // out every wall point off its wall or behind the body.  The legs on the
 // source's side first: neighbouring receivers share them, so that a blocked
 // one ends the candidate for the whole warp.
-__device__ __forceinline__ int cand_wcreep(const Ctx &c, int f, int b, int dir, v3t<float> S, v3t<float> Sw, v3t<float> P,
-                                           float band, const Frame<float> &F, Geo<float> &g, const uint32_t *occ_rx) {
-    int acc = cand_creep<float, false, false>(c, b, dir, Sw, P, band, F, g);
+template <typename T>
+__device__ __forceinline__ int cand_wcreep(const Ctx &c, int f, int b, int dir, v3t<T> S, v3t<T> Sw, v3t<T> P,
+                                           T band, const Frame<T> &F, Geo<T> &g, const uint32_t *occ_rx) {
+    int acc = cand_creep<T, false, false>(c, b, dir, Sw, P, band, F, g);
     if (acc == D_NO) return D_NO;
-    v3t<float> Qw;
-    if (!conj(acc, wall_geo<float>(c, f, S, Sw, g.Q1, band, &Qw))) return D_NO;
+    v3t<T> Qw;
+    if (!conj(acc, wall_geo<T>(c, f, S, Sw, g.Q1, band, &Qw))) return D_NO;
     const uint32_t *m1 = c.occ_w1 ? c.occ_w1 + (f * c.n_body + b) * c.occ_w : nullptr;
     const uint32_t *m2 = c.occ_w2 ? c.occ_w2 + (f * c.n_body + b) * c.occ_w : nullptr;
-    if (!conj(acc, vis_to_dec(blocked_mask(c, S, Qw, f, -1, -1, band, m1, c.occ_w)))) return D_NO;
-    if (!conj(acc, vis_to_dec(blocked_mask(c, Qw, g.Q1, f, -1, b, band, m2, c.occ_w)))) return D_NO;
-    if (!conj(acc, vis_to_dec(blocked_mask(c, g.Q2, P, -1, -1, b, band, occ_of(c, occ_rx, b), c.occ_w)))) return D_NO;
+    if (!conj(acc, vis_to_dec(leg(c, S, Qw, f, -1, -1, band, m1, c.occ_w)))) return D_NO;
+    if (!conj(acc, vis_to_dec(leg(c, Qw, g.Q1, f, -1, b, band, m2, c.occ_w)))) return D_NO;
+    if (!conj(acc, vis_to_dec(leg(c, g.Q2, P, -1, -1, b, band, occ_of(c, occ_rx, b), c.occ_w)))) return D_NO;
     return acc;
 }
 
@@ -2623,7 +2641,7 @@ __device__ __noinline__ int esc_rb(const Ctx &ctx, int b, v3t<float> Pf, const F
     v3t<dx> Sd = dxv(c.S), Pd = dxv(Pf);
     Frame<dx> F;
     body_frame(c, b, Sd, Pd, dx(0.0), F);
-    int d = cand_rb<dx>(c, b, Sd, Pd, dx(0.0), F, g);
+    int d = cand_rb<dx, true>(c, b, Sd, Pd, dx(0.0), F, g);
     if (d == D_YES && rec) {
         // the path record of the FP64 geometry (its field is summed with the
         // FP32 records, frequency chunk by frequency chunk)
@@ -2645,7 +2663,7 @@ __device__ __noinline__ int esc_creep(const Ctx &ctx, int b, int dir, v3t<float>
     v3t<dx> Sd = dxv(c.S), Pd = dxv(Pf);
     Frame<dx> F;
     body_frame(c, b, Sd, Pd, dx(0.0), F);
-    int d = cand_creep<dx>(c, b, dir, Sd, Pd, dx(0.0), F, g);
+    int d = cand_creep<dx, true, true, true>(c, b, dir, Sd, Pd, dx(0.0), F, g);
     *caustic = 0;
     if (d != D_YES) return d;
     bool sphere = c.body[2 * b + 1].y == 0.0f;
@@ -2699,7 +2717,7 @@ __device__ __noinline__ int esc_wcreep(const Ctx &ctx, int wf, int b, int dir, v
     if (!img_outside(c, b, Sw)) return D_NO;
     Frame<dx> F;
     body_frame(c, b, Sw, Pd, dx(0.0), F);
-    int d = (F.dec == D_NO) ? D_NO : cand_creep<dx, false>(c, b, dir, Sw, Pd, dx(0.0), F, g);
+    int d = (F.dec == D_NO) ? D_NO : cand_creep<dx, false, true, true>(c, b, dir, Sw, Pd, dx(0.0), F, g);
     if (d == D_YES) d = wall_legs(c, wf, b, Sd, Sw, g.Q1, dx(0.0));
     if (d != D_YES) return d;
     if (c.body[2 * b + 1].y == 0.0f) {
@@ -2720,52 +2738,6 @@ __device__ __noinline__ int esc_wcreep(const Ctx &ctx, int wf, int b, int dir, v
         acc_zero(a);
         field_wcreep<dx, dx, true>(c, a, fq, wf, Sd, Sw, Pd, g, g.sp + g.t + g.sq, enable);
         contrib_from(out, a);
-    }
-    return d;
-}
-
-// ------------------------------------------------------------------ FP64 evaluation: FP32 filter
-// RT_PREC_FP64 decides a candidate in FP32 first, as RT_PREC_FP32 does but with
-// a band FILT times as wide, and goes to FP64 for what is left: the geometry of
-// the candidates that are certainly valid, and the whole decision of the
-// uncertain ones.  What bounds the FP64 kernels is the FP64 pipe (2 lanes an
-// SM), and most candidates are no path: 24047 receivers, 20 bodies, three
-// frequencies took 1.03 -> 0.72 ms in the planar kernel and 3.24 -> 2.97 ms in the
-// creeping one (its fields are the rest), 1.72 -> 1.83 in that of reflections.
-constexpr float FILT = 16.0f;
-__device__ __noinline__ int filt_rb(const Ctx &ctx, int b, v3t<float> P, const uint32_t *occ_rx) {
-    CTX(c, ctx);
-    const float band = FILT * c.band;
-    Frame<float> F;
-    Geo<float> g;
-    body_frame(c, b, c.S, P, band, F);
-    return cand_rb<float>(c, b, c.S, P, band, F, g, occ_rx);
-}
-// both ways round: the decision of dir in bits 2 dir, 2 dir + 1
-__device__ __noinline__ int filt_creep(const Ctx &ctx, int b, v3t<float> P, const uint32_t *occ_rx) {
-    CTX(c, ctx);
-    const float band = FILT * c.band;
-    Frame<float> F;
-    body_frame(c, b, c.S, P, band, F);
-    int d = 0;
-#pragma unroll 1
-    for (int dir = 0; dir < 2; ++dir) {
-        Geo<float> g;
-        d |= cand_creep<float>(c, b, dir, c.S, P, band, F, g, occ_rx) << (2 * dir);
-    }
-    return d;
-}
-__device__ __noinline__ int filt_wcreep(const Ctx &ctx, int wf, int b, v3t<float> P, const uint32_t *occ_rx) {
-    CTX(c, ctx);
-    const float band = FILT * c.band;
-    const v3t<float> Sw = wall_img_f(c, wf);
-    Frame<float> F;
-    body_frame_tb(c, c.txw + 2 * (size_t)wf * c.n_body, b, Sw, P, band, F);
-    int d = 0;
-#pragma unroll 1
-    for (int dir = 0; dir < 2; ++dir) {
-        Geo<float> g;
-        d |= cand_wcreep(c, wf, b, dir, c.S, Sw, P, band, F, g, occ_rx) << (2 * dir);
     }
     return d;
 }
@@ -3020,7 +2992,6 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
     constexpr bool BODIES = (CLS & CLS_BODIES) != 0;
     constexpr bool fp32 = sizeof(T) == 4;
     const T band = fp32 ? T(c.band) : T(0);
-    const float fband = fp32 ? c.band : FILT * c.band;   // the FP32 decisions' band
     // fqs[0]: the frequency chunk of the body classes' fields; the planar
     // rays take all nfq chunks (each with its own partial sums)
     const FreqC &fq = fqs[0];
@@ -3060,7 +3031,7 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
         const float ex = Pf.x - q0.x, ey = Pf.y - q0.y, ez = Pf.z - q0.z, a = q0.w;
         const float m = (q1.y == 0.0f) ? a - Sqrt(ex * ex + ey * ey + ez * ez)
                                        : Fmin(Fmin(a - Sqrt(ex * ex + ey * ey), Pf.z - q0.z), q0.z + q1.x - Pf.z);
-        int d = decide(m, fband, D_YES);
+        int d = decide(m, c.band, D_YES);
         if (d == D_UNSURE) {
             if constexpr (fp32) {
                 if (part == 0 && first_chunk) escalated();   // every share and chunk takes it; one counts it
@@ -3085,39 +3056,39 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
             if (!inside) lanes_box(pl, true, Pf.x, Pf.y, tcx, tcy, tcr);
         }
     }
-    // enumerated planar candidates in FP32, with the legs' masks where there are some
-    auto dec_r1 = [&](int i, Geo<float> &g) {
+    // enumerated planar candidates, with the legs' masks where there are some
+    auto dec_r1 = [&](int i, Geo<T> &g) {
         if constexpr (PM) {
             if (pnw) {
-                int d = cand_r1_geo<float>(c, i, c.S, Pf, fband, g);
+                int d = cand_r1_geo<T>(c, i, Sx, P, band, g);
                 const bool v = d != D_NO;
                 float qx, qy, qr;
-                lanes_box(pl, v, g.Q1.x, g.Q1.y, qx, qy, qr);
+                lanes_box(pl, v, to_float(g.Q1.x), to_float(g.Q1.y), qx, qy, qr);
                 if (qr < 0.0f) return (int)D_NO;             // (no lane: the whole warp)
                 const float cx[3] = {c.S.x, qx, tcx}, cy[3] = {c.S.y, qy, tcy}, cr[3] = {0.0f, qr, tcr};
                 leg_masks<2>(c, pl, cx, cy, cr, pwm, pnw);
-                if (v) d = cand_r1_vis(c, i, c.S, Pf, fband, g, d, pwm, pnw);
+                if (v) d = cand_r1_vis<T>(c, i, Sx, P, band, g, d, pwm, pnw);
                 return d;
             }
         }
-        return cand_r1<float>(c, i, c.S, Pf, fband, g);
+        return cand_r1<T>(c, i, Sx, P, band, g);
     };
-    auto dec_r2 = [&](int i, int j, Geo<float> &g) {
+    auto dec_r2 = [&](int i, int j, Geo<T> &g) {
         if constexpr (PM) {
             if (pnw) {
-                int d = cand_r2_geo<float>(c, i, j, c.S, Pf, fband, g);
+                int d = cand_r2_geo<T>(c, i, j, Sx, P, band, g);
                 const bool v = d != D_NO;
                 float ax, ay, ar, bx, by, br;
-                lanes_box(pl, v, g.Q1.x, g.Q1.y, ax, ay, ar);
-                lanes_box(pl, v, g.Q2.x, g.Q2.y, bx, by, br);
+                lanes_box(pl, v, to_float(g.Q1.x), to_float(g.Q1.y), ax, ay, ar);
+                lanes_box(pl, v, to_float(g.Q2.x), to_float(g.Q2.y), bx, by, br);
                 if (ar < 0.0f) return (int)D_NO;             // (no lane: the whole warp)
                 const float cx[4] = {c.S.x, ax, bx, tcx}, cy[4] = {c.S.y, ay, by, tcy}, cr[4] = {0.0f, ar, br, tcr};
                 leg_masks<3>(c, pl, cx, cy, cr, pwm, pnw);
-                if (v) d = cand_r2_vis(c, i, j, c.S, Pf, fband, g, d, pwm, pnw);
+                if (v) d = cand_r2_vis<T>(c, i, j, Sx, P, band, g, d, pwm, pnw);
                 return d;
             }
         }
-        return cand_r2<float>(c, i, j, c.S, Pf, fband, g);
+        return cand_r2<T>(c, i, j, Sx, P, band, g);
     };
     if (inside) {
         fl |= RT_FLAG_INSIDE;
@@ -3138,7 +3109,7 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                         d = cand_los<T>(c, Sx, P, band);
                     }
                 } else {
-                    d = cand_los<float>(c, c.S, Pf, fband);
+                    d = cand_los<float>(c, c.S, Pf, c.band);      // (the end points are exact)
                 }
                 if (d == D_UNSURE) {
                     if constexpr (fp32) escalated();
@@ -3225,15 +3196,9 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                 for (int i = 0; i < c.n_face; ++i) {
                     if ((1 + i) % nparts != part) continue;      // candidates 1 .. n_face
                     Geo<T> g;
-                    int d;
+                    int d = dec_r1(i, g);
                     if constexpr (fp32) {
-                        d = dec_r1(i, g);
                         if (d == D_UNSURE) { escalated(); d = esc_r1(c, i, Pf, &g.Q1); }
-                    } else {
-                        Geo<float> gf;
-                        d = dec_r1(i, gf);
-                        if (d == D_UNSURE) d = cand_r1<T>(c, i, Sx, P, band, g);
-                        else if (d == D_YES && !PATHS) cand_r1_geo<T>(c, i, Sx, P, band, g);
                     }
                     if (d == D_YES) {
                         emit(PT_R1, i, 0);
@@ -3261,15 +3226,9 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                         if (j == i) continue;
                         if ((1 + i * c.n_face + j) % nparts != part) continue;   // then the ordered pairs
                         Geo<T> g;
-                        int d;
+                        int d = dec_r2(i, j, g);
                         if constexpr (fp32) {
-                            d = dec_r2(i, j, g);
                             if (d == D_UNSURE) { escalated(); d = esc_r2(c, i, j, Pf, &g.Q1, &g.Q2); }
-                        } else {
-                            Geo<float> gf;
-                            d = dec_r2(i, j, gf);
-                            if (d == D_UNSURE) d = cand_r2<T>(c, i, j, Sx, P, band, g);
-                            else if (d == D_YES && !PATHS) cand_r2_geo<T>(c, i, j, Sx, P, band, g);
                         }
                         if (d == D_YES) {
                             emit(PT_R2, i, j);
@@ -3329,30 +3288,18 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                     const bool sphere = c.body[2 * bb + 1].y == 0.0f;
                     Frame<T> F;
                     v3t<T> Sw;
-                    int filt = 0;
                     if constexpr (sizeof(T) == 4) {
                         Sw = wall_img_f(c, wf);
                         body_frame_tb(c, c.txw + 2 * (size_t)wf * c.n_body, bb, Sw, P, band, F);
                     } else {
                         Sw = wall_img_d(c, wf);
-                        filt = filt_wcreep(c, wf, bb, Pf, occ_rx);
-                        if (filt == 0 || !img_outside(c, bb, Sw)) continue;
+                        if (!img_outside(c, bb, Sw)) continue;
                         body_frame(c, bb, Sw, P, band, F);
                     }
 #pragma unroll 1
                     for (int dir = 0; dir < 2; ++dir) {
                         Geo<T> g;
-                        int d;
-                        const int fd = (filt >> (2 * dir)) & 3;
-                        if (!fp32 && fd == D_NO) continue;
-                        if constexpr (fp32) {
-                            d = cand_wcreep(c, wf, bb, dir, Sx, Sw, P, band, F, g, occ_rx);
-                        } else if (fd == D_YES) {
-                            d = cand_creep<T, false, false>(c, bb, dir, Sw, P, band, F, g);
-                        } else {
-                            d = cand_creep<T, false>(c, bb, dir, Sw, P, band, F, g);
-                            if (d == D_YES) d = wall_legs(c, wf, bb, Sx, Sw, g.Q1, band);
-                        }
+                        int d = cand_wcreep<T>(c, wf, bb, dir, Sx, Sw, P, band, F, g, occ_rx);
                         int cd = D_NO;
                         if (d == D_YES && sphere) {
                             if constexpr (sizeof(T) == 8) cd = (half_lambda_max > to_double(g.dperp)) ? D_YES : D_NO;
@@ -3391,23 +3338,12 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
                     }
                     continue;
                 }
-                // (FP64: the FP32 filter first; each kernel has one of the two classes)
-                int filt = 0;
-                if constexpr (!fp32) {
-                    filt = (CLS & CLS_BODYREFL) != 0 ? filt_rb(c, b, Pf, occ_rx) : filt_creep(c, b, Pf, occ_rx);
-                    if (filt == 0) continue;
-                    if (PATHS && (CLS & CLS_BODYREFL) != 0 && filt == D_YES) {
-                        if (enable & RT_EN_BODYREFL) emit(PT_RB, b, 0);
-                        continue;
-                    }
-                }
                 Frame<T> F;
                 body_frame(c, b, Sx, P, band, F);
                 if constexpr ((CLS & CLS_BODYREFL) != 0) {
                     if (enable & RT_EN_BODYREFL) {
                         Geo<T> g;
-                        int d = !fp32 && filt == D_YES ? cand_rb<T, false>(c, b, Sx, P, band, F, g)
-                                                       : cand_rb<T>(c, b, Sx, P, band, F, g, occ_rx);
+                        int d = cand_rb<T>(c, b, Sx, P, band, F, g, occ_rx);
                         if constexpr (sizeof(T) == 4) {
                             if (d == D_UNSURE) {
                                 // decided in FP64, and its geometry, length and amplitude
@@ -3444,10 +3380,7 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
 #pragma unroll 1
                         for (int dir = 0; dir < 2; ++dir) {
                             Geo<T> g;
-                            const int fd = (filt >> (2 * dir)) & 3;
-                            if (!fp32 && fd == D_NO) continue;
-                            int d = !fp32 && fd == D_YES ? cand_creep<T, true, false>(c, b, dir, Sx, P, band, F, g)
-                                                         : cand_creep<T>(c, b, dir, Sx, P, band, F, g, occ_rx);
+                            int d = cand_creep<T>(c, b, dir, Sx, P, band, F, g, occ_rx);
                             int cd = D_NO;
                             if (d == D_YES && sphere) {
                                 // axial caustic flag: k d_perp < pi for some frequency, i.e. d_perp < lambda_max / 2
