@@ -2815,9 +2815,12 @@ __device__ __forceinline__ void apply_records(const Ctx &c, AccS<float> &acc, co
 // points of the whole box lie in the hull of the corners' (the central
 // projection keeps convexity on that half-space), and the face box is grown
 // so that a point outside it is outside every triangle of the face by more
-// than the band.  Such candidates are decided "no" for every receiver of the
-// tile by the per-receiver test too (FP32 with its band, or FP64), so
-// leaving them out changes no decision and no field.
+// than the band.  The corners' crossing points are FP32's: each is taken as
+// uncertain by its distance from the image, times the rounding of the two
+// plane distances over their sum (centimetres, with both a fraction of a
+// millimetre from the plane).  Such candidates are decided "no" for every
+// receiver of the tile in FP64, so leaving them out changes no decision and no
+// field.
 constexpr int SEQ_MASK_WORDS = 512;      // culling up to 16384 candidates (a larger list is not culled)
 // the points where the segments from the image I (after reflection m of
 // sequence sq, face f) to the box [lo, hi] cross f's plane, within f's box:
@@ -2826,9 +2829,13 @@ __device__ __forceinline__ bool cross_box(const Ctx &c, float4 I, int f, float l
     const float4 pl = c.face32[f];
     const float4 b0 = c.face_box[2 * f], b1 = c.face_box[2 * f + 1];
     const float di = pl.x * I.x + pl.y * I.y + pl.z * I.z - pl.w;
-    const float m = 2.0f * c.band;
+    // bounds the rounding of a plane distance (per term its factors', the product's and the sums': 4e-7 of it)
+    const float err = 1e-6f * (fabsf(I.x) + fabsf(I.y) + fabsf(I.z) + fabsf(pl.w) + fmaxf(fabsf(lo[0]), fabsf(hi[0])) +
+                               fmaxf(fabsf(lo[1]), fabsf(hi[1])) + fmaxf(fabsf(lo[2]), fabsf(hi[2])));
+    const float m = 2.0f * c.band + err;
     const float sg = di > 0.0f ? 1.0f : -1.0f;
     bool same = fabsf(di) > m, opp = same;
+    float near = INFINITY;                      // the corners' least distance from the plane
     float qlo[3] = {INFINITY, INFINITY, INFINITY}, qhi[3] = {-INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
     for (int cc = 0; cc < 8; ++cc) {
@@ -2836,6 +2843,7 @@ __device__ __forceinline__ bool cross_box(const Ctx &c, float4 I, int f, float l
         const float dp = pl.x * px + pl.y * py + pl.z * pz - pl.w;
         same = same && (dp * sg > m);
         opp = opp && (-dp * sg > m);
+        near = fminf(near, -dp * sg);
         const float t = di / (di - dp);
         const float x = I.x + (px - I.x) * t, y = I.y + (py - I.y) * t, z = I.z + (pz - I.z) * t;
         qlo[0] = fminf(qlo[0], x); qhi[0] = fmaxf(qhi[0], x);
@@ -2844,14 +2852,16 @@ __device__ __forceinline__ bool cross_box(const Ctx &c, float4 I, int f, float l
     }
     if (same) return false;
     const float bl[3] = {b0.x, b0.y, b0.z}, bh[3] = {b1.x, b1.y, b1.z};
-    const float g = hull_margin(c);             // (the crossing points' own rounding)
+    const float g = hull_margin(c), dt = err / (fabsf(di) + near);
+    const float Ik[3] = {I.x, I.y, I.z};
     bool any = true;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
+        const float e = fmaxf(fabsf(lo[k] - Ik[k]), fabsf(hi[k] - Ik[k])) * dt;
         // the box straddles the plane: nothing but the face's box is known
-        if (opp) any = any && qlo[k] <= bh[k] && qhi[k] >= bl[k];
-        lo[k] = opp ? fmaxf(qlo[k] - g, bl[k]) : bl[k];
-        hi[k] = opp ? fminf(qhi[k] + g, bh[k]) : bh[k];
+        if (opp) any = any && qlo[k] - e <= bh[k] && qhi[k] + e >= bl[k];
+        lo[k] = opp ? fmaxf(qlo[k] - e - g, bl[k]) : bl[k];
+        hi[k] = opp ? fminf(qhi[k] + e + g, bh[k]) : bh[k];
     }
     return any;
 }
