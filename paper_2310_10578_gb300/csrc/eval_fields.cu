@@ -3956,9 +3956,13 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                     }
                     // the previous class kernel's fields and flags are complete (a
                     // no-op when this grid was not launched as a dependent, and
-                    // after its first return)
-                    asm volatile("griddepcontrol.wait;" ::: "memory");
+                    // after its first return).  After the barrier: a lane that
+                    // came here alone would hold its warp's others back, too, so
+                    // that this kernel's work began when the last one's ended (854
+                    // receivers among 42 faces, six frequencies in FP64: 5.19 against
+                    // 3.23 ms)
                     __syncthreads();
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
                     // reduce the tile's NWT partials: part p writes the
                     // (frequency, component) pairs j = p, p + NWT, ... of chunk ch
                     if (own) {
