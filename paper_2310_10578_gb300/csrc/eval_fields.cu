@@ -4028,6 +4028,7 @@ struct LaunchCtx {
     unsigned long long *ctr;
     int n;
     cudaStream_t stream;
+    int total;                  // launches of the evaluation's fields or lists
 };
 
 // What one evaluation covers: one frame (F1, frames == nullptr) or a batch
@@ -4103,16 +4104,32 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
     // that a few tiles spread over as many SMs)
     const int tiles_per_unit = PATHS ? 1 : NW / nwt;
     long long cap_blocks = (long long)nsm * (occ > 0 ? occ : 1);
-    // one frame of few receivers: the narrowest tiles of which a third of the
-    // device holds all (the three classes run side by side).  A tile's receivers
-    // mostly take different paths through the kernel, one after the other; apart,
-    // they run on SMs that would be idle: 97 receivers among 20 bodies 159 -> 113
-    // us.  With tiles for a whole wave of each class, 2867 and 4096 receivers were
-    // 8 and 10 % slower.
+    // One frame of few receivers: narrower tiles.  A tile's receivers mostly take
+    // different paths through the kernel, one after the other; apart, they run on
+    // SMs that would be idle: 97 receivers among 20 bodies 159 -> 97 us.  A repeated
+    // lane costs as much as any other, though, so that the tiles of all launches
+    // that run side by side (side) have to fit the device (room).
+    //   In general every launch of the evaluation, six at most, and 3/2 tiles an SM in
+    // FP32 (1112 receivers, 2 frequencies: 110 us at 70 tiles, 126 at 139), one in
+    // FP64, where two tiles of an SM share its FP64 pipe (576 receivers, 20 bodies: 305
+    // us at 36 tiles, 380 at 72, 707 at 144; 676 receivers, 13 frequencies, 20
+    // launches: 515 us at 22 tiles, 809 at 43).
+    //   FP32 kernels that outlast the others, where a lane walks a BVH or has a
+    // candidate list or many wall -> creeping pairs: a third of the blocks the device
+    // holds (683 receivers of an office, 6 frequencies: 627 us at 22 tiles, 443 at 86;
+    // 1924 receivers, 30 bodies, off walls: 3.31 ms at 61 tiles, 2.92 at 121).  FP64
+    // with a BVH: a third of a tile an SM, of two for candidate lists (814 receivers:
+    // 2.44 ms at 26 tiles, 2.10 at 51, 2.83 at 102).  Path lists, whose launches run
+    // one after the other: a third of the blocks, too.
     int tsh = 5;
+    const bool bvh = LARGE && S.bvh;
+    const bool lasts = sizeof(T) == 4 ? bvh || CLS == CLS_SEQ || (CLS == CLS_WCREEP && S.n_face * S.n_body >= 16) : bvh;
+    const unsigned long long side = PATHS || lasts ? 3 : (L.total < 6 ? L.total : 6);
+    const unsigned long long room = PATHS || (lasts && sizeof(T) == 4) ? (unsigned long long)(cap_blocks * tiles_per_unit)
+                                    : sizeof(T) == 4 ? 3ull * nsm / 2 : (bvh && CLS == CLS_SEQ ? 2ull : 1ull) * nsm;
     auto tiles_of = [&](int sh) { return (((unsigned long long)W.F1.n_rx + (1u << sh) - 1) >> sh); };
     if (!W.frames && (!PATHS || split))
-        while (tsh > 0 && 3 * tiles_of(tsh - 1) <= (unsigned long long)(cap_blocks * tiles_per_unit)) --tsh;
+        while (tsh > 0 && side * tiles_of(tsh - 1) <= room) --tsh;
     const unsigned long long n_tiles = tsh < 5 ? tiles_of(tsh) : W.n_tiles;
     long long need = (long long)((n_tiles + tiles_per_unit - 1) / tiles_per_unit);
     int grid = (int)(need < cap_blocks ? need : cap_blocks);
@@ -4152,6 +4169,8 @@ static cudaError_t launch_all(const DevScene &S, const Work &W, int nchunks, Lau
     // geometry pass
     const int pstep = chunked_bodies ? 1 : (W.planar_chunks >= 1 && W.planar_chunks <= MAX_CHUNKS ? W.planar_chunks
                                                                                                   : PLANAR_CHUNKS);
+    const int per = 1 + (S.max_enc + 1) * (wall ? 2 : 1), nplanar = (nchunks + pstep - 1) / pstep;
+    L.total = nplanar + (chunked_bodies ? nplanar * per : per);
     for (int ch = 0; ch < nchunks && e == cudaSuccess; ch += pstep) {
         const int n = nchunks - ch < pstep ? nchunks - ch : pstep;
         if constexpr (LARGE) {
@@ -4178,7 +4197,7 @@ static cudaError_t launch_all(const DevScene &S, const Work &W, int nchunks, Lau
 // same kernels, unordered; FP64: the fields, then the path-list kernels)
 static int run(const DevScene &S, const Work &W, int precision, bool paths, bool list, unsigned long long *ctr,
                cudaStream_t stream, int *n_launches) {
-    LaunchCtx L{ctr, 0, stream};
+    LaunchCtx L{ctr, 0, stream, 0};
     const int nchunks = paths ? 1 : (S.n_f + NFC - 1) / NFC;
     cudaError_t e;
     // scenes with a BVH: the bodies hidden from the transmitter first
