@@ -2769,7 +2769,6 @@ constexpr int recs_per_unit(int cls) {
     return ((cls & CLS_CREEP) ? 2 : 0) + ((cls & CLS_BODYREFL) ? 1 : 0) + ((cls & CLS_WCREEP) ? 4 : 0);
 }
 constexpr int WARPS_PER_TILE = 4;
-constexpr int PATH_TILES = 3;
 constexpr uint16_t NO_BODY = 0xffffu;  // see body_list
 constexpr int BLIST_MAX = RT_MAX_BODIES + 32;
 constexpr int MAX_CHUNKS = (RT_MAX_FREQS + NFC - 1) / NFC;
@@ -4076,11 +4075,17 @@ static cudaError_t launch_one(const DevScene &S, const Work &W, int ch0, int nch
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     bool split = false;
     if constexpr (PATHS) {
-        // path lists: a block's warps share a tile until each warp would have
-        // PATH_TILES of its own: 11468 receivers, 20 bodies (359 tiles, for 608 and
-        // 1824 warps) took 677 us a warp per tile, 329 shared
-        split = split_paths(CLS) && (CLS != CLS_PLANAR || S.n_face <= RT_MAX_ENUM_FACES) &&
-                (long long)W.n_tiles < (long long)PATH_TILES * nsm * min_blocks(CLS, sizeof(T) == 4) * NW;
+        // path lists: a block's warps share a tile's candidates where that is less
+        // than a warp for each tile, counted in candidates one after the other (of
+        // the body classes: in bodies).  A shared tile costs two barriers more, in
+        // FP32 half of its own time.  One body takes a warp a tile sooner than 40, and
+        // planar candidates from 0.65 tiles a warp on: 11468 receivers, 20 bodies 677
+        // us a warp a tile, 323 shared; 40000 receivers, one body 281 us, 284 with
+        // both classes shared, 209 with the planar one; 80000 319, 500 and 367.
+        const double blocks = (double)nsm * min_blocks(CLS, sizeof(T) == 4), tiles = (double)W.n_tiles;
+        const int units = bodies ? S.n_body : path_slots(CLS, S.n_face, S.n_body);
+        split = split_paths(CLS) && (CLS != CLS_PLANAR || S.n_face <= RT_MAX_ENUM_FACES) && tiles < blocks * NW &&
+                fmax(1.0, (sizeof(T) == 4 ? 1.5 : 1.0) * tiles / blocks) * ((units + NW - 1) / NW) <= units;
         nwt = split ? NW : 1;
         if (split) sm += sizeof(uint32_t) * path_slots(CLS, S.n_face, S.n_body);
     }
