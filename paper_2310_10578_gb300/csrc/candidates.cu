@@ -101,7 +101,8 @@ __device__ __forceinline__ unsigned long long seq_key(int k, const int fs[3]) {
 // scale, the largest |coordinate| of the ray and the triangle) and that of
 // some ten operations, 1e-5 (|s| + scale) |edge| in all, two orders above it.
 // (The FP64 test divides by det; the signs of its u, v and 1 - u - v are those
-// of the numerators here.)
+// of the numerators here.)  FP64 decides, too, where a product overflows, with
+// coordinates from 1e12 m on (vertices may be any finite floats).
 __device__ __forceinline__ bool ray_tri_may(const float o[3], const float d[3], float4 a, float4 b, float4 c,
                                             float scale, float best) {
     const float e1x = b.x - a.x, e1y = b.y - a.y, e1z = b.z - a.z, e2x = c.x - a.x, e2y = c.y - a.y, e2z = c.z - a.z;
@@ -114,6 +115,7 @@ __device__ __forceinline__ bool ray_tri_may(const float o[3], const float d[3], 
     const float m = 1e-5f * (fabsf(sx) + fabsf(sy) + fabsf(sz) + scale), eu = m * l2, ev = m * l1;
     const float ed = 1e-5f * l1 * l2;
     if (fabsf(det) <= ed) return true;           // the plane nearly along the ray: let FP64 decide
+    if (!(fabsf(det) + fabsf(u) + fabsf(v) + fabsf(t) < INFINITY)) return true;
     if (det < 0.0f) { det = -det; u = -u; v = -v; t = -t; }
     if (u < -eu || v < -ev || u + v > det + ed + eu + ev) return false;
     const float et = m * l1 * l2;
