@@ -3940,7 +3940,7 @@ k_eval(DevScene S, FrameDev F1, const FrameDev *__restrict__ frames, int n_frame
                                                  occ_on ? s_occ_rx + grp * S.n_body * occ_w : nullptr, part,
                                                  NWT, acc, rec, fl, nesc, npath, nrec,
                                                  qm_on ? &s_qmask[warp][0] : nullptr, lanes, &s_pwm[LEGM ? warp : 0][0], &s_cstk[COOP ? warp : 0][0],
-                                                 nullptr, own);
+                                                 nullptr, own && ch0 == 0);     // (listed once: by the first launch of a class)
                 s_fl[warp][lane] = fl;
                 if (own && nesc && ch0 == 0) atomicAdd(esc_counter, (unsigned long long)nesc);
 #pragma unroll 1
