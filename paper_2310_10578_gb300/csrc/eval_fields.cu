@@ -154,7 +154,7 @@ struct Ctx {
     int n_cand;
     const float4 *face_mat;      // face materials, see DevScene (nullptr: all PEC)
     int enc;                     // this launch's creeping rays: extra full turns round the body
-    // occluder masks (FP32 body kernels): occ_w words per body; word w of
+    // occluder masks (body kernels): occ_w words per body; word w of
     // body b's source-side mask has bit j set if body j may block a segment
     // from the source to a point of body b (occ_w = 0: no masks)
     const uint32_t *occ_src;
@@ -841,7 +841,7 @@ __device__ __forceinline__ float seg_d2(float px, float py, float ax, float ay, 
     return hx * hx + hy * hy;
 }
 
-// ---- occluder masks of the planar legs (FP32 fields).  The lanes of a warp
+// ---- occluder masks of the planar legs (both precisions; path lists too).  The lanes of a warp
 // take the same planar candidate for the warp's receivers.  Its legs run
 // between consecutive regions: the source point, the box of the lanes'
 // reflection points on each face, the box of the lanes' receivers.  In
