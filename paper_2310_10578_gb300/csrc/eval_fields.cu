@@ -1759,7 +1759,7 @@ template <typename T>
 __device__ __forceinline__ int cand_wcreep(const Ctx &c, int f, int b, int dir, v3t<T> S, v3t<T> Sw, v3t<T> P,
                                            T band, const Frame<T> &F, Geo<T> &g, const uint32_t *occ_rx) {
     int acc = cand_creep<T, false, false>(c, b, dir, Sw, P, band, F, g);
-    if (acc == D_NO || !F.axis_ok) return acc;       // (no points from an ill-conditioned frame)
+    if (acc == D_NO) return D_NO;
     v3t<T> Qw;
     if (!conj(acc, wall_geo<T>(c, f, S, Sw, g.Q1, band, &Qw))) return D_NO;
     const uint32_t *m1 = c.occ_w1 ? c.occ_w1 + (f * c.n_body + b) * c.occ_w : nullptr;
@@ -3308,7 +3308,9 @@ __device__ __forceinline__ void eval_receiver(const Ctx &c, const FreqC *fqs, in
 #pragma unroll 1
                     for (int dir = 0; dir < 2; ++dir) {
                         Geo<T> g;
-                        int d = cand_wcreep<T>(c, wf, bb, dir, Sx, Sw, P, band, F, g, occ_rx);
+                        // (an ill-conditioned frame has no points: FP64)
+                        int d = F.axis_ok ? cand_wcreep<T>(c, wf, bb, dir, Sx, Sw, P, band, F, g, occ_rx)
+                                          : (F.dec == D_NO ? D_NO : D_UNSURE);
                         int cd = D_NO;
                         if (d == D_YES && sphere) {
                             if constexpr (sizeof(T) == 8) cd = (half_lambda_max > to_double(g.dperp)) ? D_YES : D_NO;
